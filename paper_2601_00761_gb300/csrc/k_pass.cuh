@@ -444,6 +444,20 @@ __device__ __forceinline__ void fwht_pass_body(const PassArgs &a, long long slot
         if constexpr (Cfg::NR <= 1 && PREC == 0) __syncthreads();
     }
 
+    if constexpr (SRC == SRC_BUF && DST == DST_MOMENTS && Cfg::RB == 6) {
+        // 12 warps per SM do not keep enough loads in flight for DRAM: the tile
+        // that a CTA one wave of SMs later reads is brought into L2 (the tiles
+        // of a launch are contiguous and run in order). N = 18, 4096 families,
+        // 2^11-point tiles: 1.49 against 1.79 ps per point; two or more waves
+        // ahead are slower, past twelve slower than none.
+        constexpr long long AHEAD = 152;
+        const long long tiles = a.slot_elems >> Cfg::M, lin = slot * tiles + (long long)tile + AHEAD;
+        if (t == 0 && lin < a.n_fam * tiles)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
+                             reinterpret_cast<const float2 *>(a.src) + ((size_t)lin << Cfg::M)),
+                         "r"((int)sizeof(float2) << Cfg::M) : "memory");
+    }
+
     // ---------------------------------------------------------- prologue
     pass_prologue<Cfg, SRC>(v, a, psi, slot, x, j, half, gbase, t);
 
@@ -543,9 +557,10 @@ __device__ __forceinline__ void fwht_pass_body(const PassArgs &a, long long slot
         const uint32_t zb = (uint32_t)gbase | Cfg::elem(t, 0, 0);
         float2 s2 = make_float2(0.f, 0.f), s4 = s2, s6 = s2, sl = s2, w = s2;
         float qmax = 0.f;
-        const bool wr = a.want_ranges, cand = a.want_cand;
+        constexpr bool RANGES = Cfg::E <= 32;     // 64 points per thread: launched without ranges only
+        const bool wr = RANGES && a.want_ranges, cand = a.want_cand;
         // ranges of 2^ZR_FINE z (written per warp) or tile halves (2^M z)
-        constexpr bool FINE = SRC == SRC_BUF && Cfg::M > ZR_FINE;
+        constexpr bool FINE = RANGES && SRC == SRC_BUF && Cfg::M > ZR_FINE;
         constexpr int RLS = FINE ? ZR_FINE : Cfg::M;
         if (x) {
             const float2 sc = make_float2(2.0f * s, 2.0f * s);
@@ -555,9 +570,9 @@ __device__ __forceinline__ void fwht_pass_body(const PassArgs &a, long long slot
                 // is the pair of weights. Bit k of pm: parity of |x & z0| for
                 // z' = zb | k (z0 then carries the Im part).
                 const uint32_t xd = (uint32_t)((x & ((1ULL << j) - 1ULL)) | ((x >> (j + 1)) << j));
-                const uint32_t pm = walsh_mask5(xd & (Cfg::E - 1)) ^ ((__popc(xd & zb) & 1) ? 0xFFFFFFFFu : 0u);
-                if (cand) moment_sums<Cfg::E, true, true>(v, sc, pm, s2, s4, s6, sl, qmax);
-                else moment_sums<Cfg::E, true, false>(v, sc, pm, s2, s4, s6, sl, qmax);
+                const uint32_t pm = walsh_mask5(xd & (Cfg::E - 1) & 31u) ^ ((__popc(xd & zb) & 1) ? 0xFFFFFFFFu : 0u);
+                if (cand) moment_sums<Cfg::E, RANGES, true>(v, sc, pm, s2, s4, s6, sl, qmax);
+                else moment_sums<Cfg::E, RANGES, false>(v, sc, pm, s2, s4, s6, sl, qmax);
                 w = s2;
             } else {
                 if (cand) moment_sums<Cfg::E, false, true>(v, sc, 0u, s2, s4, s6, sl, qmax);

@@ -103,9 +103,17 @@ cudaError_t launch_f64_single(int M, int src, int dst, const PassArgs &a, cudaSt
 cudaError_t launch_f64_strided(int K, int src, int dst, const PassArgs &a, int tiles, cudaStream_t st);
 cudaError_t launch_f64_row(int M, int src, int dst, const PassArgs &a, int tiles, cudaStream_t st);
 
-// strided tile: 2^K rows x 2^(MS-K) columns; FP32 MS = 13 for every K (64 KB,
-// at least 8 columns = 64 contiguous bytes per row, two CTAs per SM so one
-// CTA's loads overlap the other's butterflies); FP64 MS = 13 (128 KB)
+// FP32 strided tile: 2^K rows x 2^(MS-K) columns. Up to five bits run in one
+// register round without shared memory, and so do six with 64 points per
+// thread; then the smallest tiles (one or two warps, 256-byte rows) overlap
+// best. From seven bits on a tile is exchanged once through shared memory and
+// keeps 16 columns (128-byte rows) as far as 64 KB go. Per packed point,
+// psi-reading pass, against tiles of 2^13 points throughout:
+//   K       4     5     6     7     8     9    10
+//   2^13  1.47  1.50  2.08  2.08  2.10  2.08  2.5 ps
+//   here  1.17  1.19  1.25  1.61  1.82  2.08  2.5 ps
+// (1.18 ps is the DRAM time of the 8 bytes written; with 8 columns, 64-byte
+// rows, K = 7 takes 2.6 ps). FP64 MS = 13 (128 KB).
 constexpr int F32_STRIDED_KMAX = 10, F32_ROW_MMIN = 10, F32_ROW_MMAX = 14, F32_SINGLE_MMAX = 14;
 // register bits of the 13-bit FP32 row pass: 4 (512 threads x 16 points, two
 // CTAs per SM: 32 warps) or 5 (256 x 32)
@@ -122,7 +130,10 @@ constexpr int F32_STRIDED10_RB = SRE_STRIDED10_RB;
 // whether the FP32 row pass of M bits accumulates its z-range weights (the
 // caller zeroes the rows first)
 constexpr bool f32_row_ranges_accumulate(int M) { return ranges_accumulate(1 << (M == 13 ? F32_ROW13_RB : 5)); }
-__host__ __device__ constexpr int f32_strided_ms(int K) { return K + 3 > 13 ? K + 3 : 13; }
+__host__ __device__ constexpr int f32_strided_ms(int K, bool wide = false) {
+    return K <= 5 ? 10 : K == 6 ? 11 : K + (wide ? 5 : 4) < 13 ? K + (wide ? 5 : 4) : 13;
+}
+__host__ __device__ constexpr int f32_strided_rb(int K) { return K == 10 ? F32_STRIDED10_RB : 5; }
 constexpr int F64_STRIDED_M = 13, F64_STRIDED_KMAX = 9, F64_ROW_M = 12, F64_SINGLE_MMAX = 12;
 
 } // namespace sre

@@ -112,9 +112,9 @@ void tune_save_locked() {
     fclose(f);
 }
 
-sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P);
+sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P, bool sweep = false);
 
-sre_status plan_for_tuned(int N, const sre_opts *o, int prec, Plan &P) {
+sre_status plan_for_tuned(int N, const sre_opts *o, int prec, Plan &P, bool sweep = false) {
     sre_opts t;
     sre_default_opts(&t);
     if (o) t = *o;
@@ -127,15 +127,31 @@ sre_status plan_for_tuned(int N, const sre_opts *o, int prec, Plan &P) {
             t.x_batch = g_tune[N].xbatch;
         }
     }
-    return plan_for(N, &t, prec, P);
+    return plan_for(N, &t, prec, P, sweep);
 }
 
-sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P) {
+// Row bits of a sweep that draws no z (exact enumeration, uniform Monte
+// Carlo). The sampled z depend on the order of the transform's stages, so the
+// marginal estimator keeps 13-bit rows; the others take the split with the
+// fewest exchanges through shared memory: rows of ten bits (one warp per tile,
+// one exchange) above a register-only strided pass of up to six, then rows of
+// eleven and twelve (64 points per thread, one exchange). Per packed point,
+// both passes, against the 13-bit rows (one 14-bit tile at N = 15):
+//   N      15    16    17    18    19    20    21    22
+//   13    3.00  3.50  3.44  3.42  4.0   4.01  4.0   4.0  ps
+//   here  2.55  2.57  2.65  2.77  2.8   3.1   3.35  3.6  ps
+// n = 23 needs a third pass below 13 bits.
+int sweep_radix(int n) { return n <= 16 ? 10 : n == 17 ? 11 : n == 23 ? 13 : 12; }
+constexpr int SWEEP_SINGLE_MMAX = 13;
+
+sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P, bool sweep) {
     P = Plan();
     P.N = N;
     P.n = N - 1;
     P.prec = prec;
-    const int single_max = prec == 32 ? F32_SINGLE_MMAX : F64_SINGLE_MMAX;
+    // explicit tilings are taken as they are
+    sweep = sweep && prec == 32 && !(o && (o->radix_log2 > 0 || o->tile_log2 > 0));
+    const int single_max = prec == 32 ? (sweep ? SWEEP_SINGLE_MMAX : F32_SINGLE_MMAX) : F64_SINGLE_MMAX;
     if (P.n <= single_max) {
         P.npass = 1;
         P.M_last = P.n;
@@ -148,13 +164,14 @@ sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P) {
     }
     int nlo, kmax;
     if (prec == 32) {
-        nlo = (o && o->radix_log2 > 0) ? clampi(o->radix_log2, F32_ROW_MMIN, F32_ROW_MMAX) : 13;
+        nlo = (o && o->radix_log2 > 0) ? clampi(o->radix_log2, F32_ROW_MMIN, F32_ROW_MMAX) : sweep ? sweep_radix(P.n) : 13;
         kmax = (o && o->tile_log2 > 0) ? clampi(o->tile_log2, 1, F32_STRIDED_KMAX) : F32_STRIDED_KMAX;
     } else {
         nlo = F64_ROW_M;
         kmax = F64_STRIDED_KMAX;
     }
-    auto ms_of = [&](int K) { return prec == 32 ? f32_strided_ms(K) : F64_STRIDED_M; };
+    // the first pass reads psi (8 bytes << N), which L2 holds up to N = 24
+    auto ms_of = [&](int K, int pass) { return prec == 32 ? f32_strided_ms(K, pass == 0 && N >= 25) : F64_STRIDED_M; };
     // A strided tile is 2^K rows x 2^(ms-K) columns and its columns must fit
     // below the pass's row stride 2^lo: ms - K <= lo. Only the bottom strided
     // pass (lo = nlo) can violate it: K_bottom >= 13 - nlo.
@@ -180,7 +197,7 @@ sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P) {
     int top = P.n;
     for (int i = 0; i < ns; ++i) {
         P.lo[i] = top - P.K[i];
-        P.ms[i] = ms_of(P.K[i]);
+        P.ms[i] = ms_of(P.K[i], i);
         top = P.lo[i];
         if (P.ms[i] - P.K[i] > P.lo[i]) return fail(SRE_EINVAL, "internal plan error (N=%d pass %d)", N, i);
     }
@@ -634,7 +651,7 @@ sre_status nullity_from_count(long long cnt, int N, sre_result *r) {
 sre_status exact_impl(const void *psi, int N, const sre_opts &o, void *ws, size_t ws_bytes, cudaStream_t st,
                       sre_result *out) {
     Plan P, P64;
-    CS(plan_for_tuned(N, &o, 32, P));
+    CS(plan_for_tuned(N, &o, 32, P, true));
     CS(plan_for(N, nullptr, 64, P64));
     Arena dry(nullptr);
     ExactWS w;
@@ -1084,7 +1101,7 @@ sre_status batched_impl(const void *const *psi_ptrs, const int *Ns, int count, c
             b.idx = by[N];
             b.off = off;
             off += (int)b.idx.size();
-            CS(plan_for_tuned(N, &o, 32, b.P));
+            CS(plan_for_tuned(N, &o, 32, b.P, true));
             CS(plan_for(N, nullptr, 64, b.P64));
             b.states_per_chunk = (int)std::max(1LL, BATCH_CHUNK_FAMILIES >> N);
             b.flags = nullptr;
@@ -1540,7 +1557,7 @@ sre_status sre_workspace_bytes(int N, int mode, long long n_x, int z_per_x, cons
     if (mode == -1) {
         if (N < 1 || N > 26) return fail(SRE_EINVAL, "exact: N=%d outside 1..26", N);
         Plan P64;
-        CS(plan_for_tuned(N, &o, 32, P));
+        CS(plan_for_tuned(N, &o, 32, P, true));
         CS(plan_for(N, nullptr, 64, P64));
         Arena A(nullptr);
         ExactWS w;
@@ -1551,7 +1568,7 @@ sre_status sre_workspace_bytes(int N, int mode, long long n_x, int z_per_x, cons
     if (mode != SRE_MC_UNIFORM && mode != SRE_MC_MARGINAL) return fail(SRE_EINVAL, "unknown mode %d", mode);
     if (N < 2 || N > 30) return fail(SRE_EINVAL, "mc: N=%d outside 2..30", N);
     if (n_x < 2 || (mode == SRE_MC_MARGINAL && z_per_x < 1)) return fail(SRE_EINVAL, "n_x >= 2 and z_per_x >= 1 required");
-    CS(plan_for_tuned(N, &o, 32, P));
+    CS(plan_for_tuned(N, &o, 32, P, mode == SRE_MC_UNIFORM));
     Arena A(nullptr);
     McWS w;
     layout_mc(A, P, mode, n_x, z_per_x, w);
@@ -1641,7 +1658,7 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
     CS(check_opts(opts, o));
     cudaStream_t st = (cudaStream_t)stream;
     Plan P;
-    CS(plan_for_tuned(N, &o, 32, P));
+    CS(plan_for_tuned(N, &o, 32, P, mode == SRE_MC_UNIFORM));
     Arena dry(nullptr);
     McWS w;
     layout_mc(dry, P, mode, n_x, z_per_x, w);

@@ -26,12 +26,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-// CTAs per SM targeted by the register allocation of 256-thread tiles of at
-// most 64 KB (a build-time tuning constant).
-#ifndef SRE_MINB_SMALL
-#define SRE_MINB_SMALL 2
-#endif
-
 namespace sre {
 
 template <typename R> struct V2;
@@ -111,10 +105,12 @@ struct TileCfg {
     static constexpr int K = M - LO;
     static constexpr int NR = RB > 0 ? (K + RB - 1) / RB : 0;
     static constexpr int SIZE = 1 << M;
-    // CTAs per SM the register budget is sized for: tiles of at most 64 KB
-    // (FP32 M <= 13) run several per SM so load and compute phases overlap
-    // (256 threads with 32 points each, or 512 threads with 16)
-    static constexpr int MINB = (G == 1 && sizeof(C2) * SIZE <= 65536 && (NT == 256 || NT == 512)) ? SRE_MINB_SMALL : 1;
+    // CTAs per SM the register budget is sized for: FP32 tiles of at most 64 KB
+    // keep 16 warps of 128 registers on an SM (12 warps of 168 when a thread
+    // holds 64 points), in as many CTAs as that makes, so that load, exchange
+    // and butterfly phases of different CTAs overlap
+    static constexpr int REGS = RB >= 6 ? 168 : 128;
+    static constexpr int MINB = (sizeof(C2) == 8 && sizeof(C2) * SIZE * G <= 65536) ? 65536 / (REGS * NT) : 1;
     static_assert(TB >= 0, "tile smaller than a thread's registers");
     static_assert(K >= 0, "bad tile");
 
@@ -162,11 +158,21 @@ struct Rounds {
     __device__ static __forceinline__ void run(C2 (&v)[Cfg::E], C2 *sm, uint32_t t, uint32_t g) {
         C2 *pb = sm + Cfg::phys(Cfg::elem(t, 0, a), g);
         if constexpr (r > 0) {
-            __syncthreads();
+            // a group of at most 32 threads lies in one warp
+            if constexpr (Cfg::T <= 32) __syncwarp();
+            else __syncthreads();
 #pragma unroll
             for (int k = 0; k < Cfg::E; ++k) v[k] = pb[Cfg::pad((uint32_t)k << a)];
         }
-        butterflies<C2, Cfg::E, Cfg::range_lo(i) - a, Cfg::range_hi(i) - a>(v);
+        if constexpr (Cfg::RB == 6 && Cfg::LO > 0) {
+            // six strided bits in one round: the stage order (hence the
+            // rounding) of rounds of five bits, the top bit first
+            static_assert(Cfg::K == 6 && Cfg::NR == 1, "one round of six bits");
+            butterflies<C2, Cfg::E, 5, 6>(v);
+            butterflies<C2, Cfg::E, 0, 5>(v);
+        } else {
+            butterflies<C2, Cfg::E, Cfg::range_lo(i) - a, Cfg::range_hi(i) - a>(v);
+        }
         if constexpr (r < Cfg::NR - 1) {
 #pragma unroll
             for (int k = 0; k < Cfg::E; ++k) pb[Cfg::pad((uint32_t)k << a)] = v[k];
