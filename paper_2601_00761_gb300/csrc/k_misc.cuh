@@ -80,6 +80,13 @@ cudaError_t launch_wait_selftest(const void *src16, int *err, cudaStream_t st);
 cudaError_t launch_zsample(int single, int fine, int M, const PassArgs &a, const DrawInfo *draws, int z_per_x,
                            unsigned long long *zs, float *cz, const unsigned long long *perm, cudaStream_t st);
 
+// The x-marginal into p (d doubles) with work (d doubles) as intermediate, for
+// N >= MARG_NMIN (k_marg.cu); scal holds the norm (launch_norm2).
+constexpr int MARG_ROW_BITS = 11, MARG_STRIDED_MAX = 9;
+constexpr int MARG_NMIN = MARG_ROW_BITS + 2;
+cudaError_t launch_marginal(const float2 *psi, int N, const double *scal, double *p, double *work, int *launches,
+                            cudaStream_t st);
+
 // gates (k_gates.cu)
 struct GateRow { unsigned char op, q0, q1; };
 constexpr unsigned char GATE_OP_U2 = 6;   // general two-qubit gate (matrix table indexed by row)

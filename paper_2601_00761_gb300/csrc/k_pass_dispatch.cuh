@@ -29,12 +29,9 @@ SRE_ALLOW(double, KIND_SINGLE, SRC_PSI_FAMILY, DST_SPECTRUM)
 SRE_ALLOW(double, KIND_SINGLE, SRC_PSI_Q, DST_SQMAP)
 SRE_ALLOW(double, KIND_SINGLE, SRC_BUF, DST_P)
 SRE_ALLOW(double, KIND_STRIDED, SRC_PSI_FAMILY, DST_BUF)
-SRE_ALLOW(double, KIND_STRIDED, SRC_PSI_Q, DST_BUF)
 SRE_ALLOW(double, KIND_STRIDED, SRC_BUF, DST_BUF)
 SRE_ALLOW(double, KIND_ROW, SRC_BUF, DST_NULLCOUNT)
 SRE_ALLOW(double, KIND_ROW, SRC_BUF, DST_SPECTRUM)
-SRE_ALLOW(double, KIND_ROW, SRC_BUF, DST_SQMAP)
-SRE_ALLOW(double, KIND_ROW, SRC_BUF, DST_P)
 #undef SRE_ALLOW
 
 // Tensor-core variants exist for FP32 tiles whose groups are whole warps.

@@ -498,7 +498,6 @@ sre_status run_transform(const Plan &P, PassArgs a, int src0, int dst_last, void
     PassArgs b = a;
     b.lo_g = 0;
     b.src = inter;
-    if (dst_last == DST_SQMAP) b.dst = inter;
     CS(timer_mark(T, P.nstrided, st, true));
     e = P.prec == 32 ? launch_f32_row(P.M_last, SRC_BUF, dst_last, b, (int)P.tiles_last, st)
                      : launch_f64_row(P.M_last, SRC_BUF, dst_last, b, (int)P.tiles_last, st);
@@ -508,8 +507,15 @@ sre_status run_transform(const Plan &P, PassArgs a, int src0, int dst_last, void
     return SRE_OK;
 }
 
-// x-marginal into p (FP64): WHT(|psi|^2) -> square -> WHT -> /d
+// x-marginal into p: WHT(|psi|^2) -> square -> WHT -> /d, in 64-bit integers
+// (k_marg.cu), or in one FP64 tile for the sizes that fit one
 sre_status run_marginal(const void *psi, int N, const double *scal, double *p, double *mwork, cudaStream_t st) {
+    if (N >= MARG_NMIN) {
+        int nl = 0;
+        CK(launch_marginal((const float2 *)psi, N, scal, p, mwork, &nl, st));
+        count_launches(nl);
+        return SRE_OK;
+    }
     Plan P64;
     CS(plan_for(N, nullptr, 64, P64));
     PassArgs a = base_args(P64, psi, scal);
