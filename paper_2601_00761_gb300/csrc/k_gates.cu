@@ -3,8 +3,21 @@
 // preconditioning circuits, T doping and brick-wall circuits of the paper), applied
 // in fused blocks: a run of consecutive gates acting inside a set of at most
 // GATE_BLOCK_Q qubits (always containing qubits 0..4, so every tile is made of
-// 256-byte contiguous runs) is applied to each 2^Q-amplitude tile in shared
-// memory with one global read and one global write of psi per block.
+// 256-byte contiguous runs) is applied to each 2^Q-amplitude tile with one
+// global read and one global write of psi per block.
+//
+// Inside a block the tile passes through the registers in rounds. In a round
+// every thread holds the 32 amplitudes of five local qubits (the round's slots;
+// the others select the thread), and a gate is arithmetic in registers when
+// its qubits are slots; a phase gate runs on any qubit and a CNOT needs only its
+// target among the slots. Between rounds the tile is redistributed through
+// shared memory with one barrier. The host orders a block's gates into rounds
+// (sre_api.cu, run_gate_list). One barrier and one trip through shared memory
+// per gate, as an in-place update of the shared tile takes, bound the kernel
+// before: 1000 random Clifford + T gates at N = 26 took 31 ms in 32 blocks, now
+// 17 ms (2.3 rounds a block; instruction issue bounds it, DRAM would take 5 ms);
+// 552 two-qubit gates at N = 24 10.9 ms in 29 blocks, now 8.9 ms (4.3 rounds a
+// block; 4.0 ms at the full FP32 rate).
 #include "k_misc.cuh"
 
 namespace sre {
@@ -14,11 +27,106 @@ struct GateBlockParams {
     int n_other;                 // qubits outside the block
     unsigned char local[GATE_BLOCK_Q];   // global qubit of local bit i (ascending)
     unsigned char other[32];             // global qubit of tile bit i (ascending)
-    int g0, ng;                  // gate rows [g0, g0 + ng) of the translated list
+    int r0, nr;                  // rounds [r0, r0 + nr)
+    int g0, ng;                  // gate rows of the block
 };
 
-__global__ void __launch_bounds__(256) gate_block_kernel(float2 *psi, const GateRow *gates, const float2 *mats,
-                                                         GateBlockParams p) {
+namespace {
+
+constexpr int GT = 256;                     // threads
+constexpr int GE = 1 << GATE_ROUND_SLOTS;   // amplitudes per thread
+
+// Shared-memory position of local index e: the nibbles above the lowest one
+// are folded into it, so that lanes whose bits fall in different residues
+// mod 4 (the host picks them so) hit different banks. Linear over GF(2).
+__device__ __forceinline__ uint32_t gphys(uint32_t e) { return e ^ ((e >> 4) & 15u) ^ ((e >> 8) & 15u) ^ ((e >> 12) & 15u); }
+
+template <int S>
+__device__ __forceinline__ void gate_h(float2 (&v)[GE]) {
+    const float2 r2 = make_float2(0.70710678118654752440f, 0.70710678118654752440f);
+#pragma unroll
+    for (int k = 0; k < GE; ++k)
+        if (!(k & (1 << S))) {
+            const float2 u = v[k], w = v[k | (1 << S)];
+            v[k] = mul2(r2, add2(u, w));
+            v[k | (1 << S)] = mul2(r2, sub2(u, w));
+        }
+}
+
+// phase on the amplitudes whose index has all bits of MASK
+template <int MASK>
+__device__ __forceinline__ void gate_phase(float2 (&v)[GE], float cr, float ci) {
+#pragma unroll
+    for (int k = 0; k < GE; ++k)
+        if ((k & MASK) == MASK) {
+            const float2 u = v[k];
+            v[k] = make_float2(cr * u.x - ci * u.y, cr * u.y + ci * u.x);
+        }
+}
+
+// e^{i pi ph / 4}
+__device__ __forceinline__ void phase_of(int ph, float &cr, float &ci) {
+    const float r2 = 0.70710678118654752440f;
+    const float a = (ph & 1) ? r2 : (ph & 2) ? 0.f : 1.f;     // |cos|
+    const float b = (ph & 1) ? r2 : (ph & 2) ? 1.f : 0.f;     // |sin|
+    cr = ((ph + 2) & 4) ? -a : a;
+    ci = (ph & 4) ? -b : b;
+}
+
+// exchange of target pairs among the amplitudes whose index has all bits of CM,
+// where the bits of m are set (m is all ones or zero). By exclusive or: as a
+// plain exchange the compiler permutes registers, and where the gates' branches
+// meet it then copies all 64 of them, three times the work of the gate itself.
+template <int CM, int T>
+__device__ __forceinline__ void gate_cx(float2 (&v)[GE], uint32_t m) {
+#pragma unroll
+    for (int k = 0; k < GE; ++k)
+        if ((k & CM) == CM && !(k & (1 << T))) {
+            float2 &a = v[k], &b = v[k | (1 << T)];
+            const uint32_t tx = (__float_as_uint(a.x) ^ __float_as_uint(b.x)) & m;
+            const uint32_t ty = (__float_as_uint(a.y) ^ __float_as_uint(b.y)) & m;
+            a = make_float2(__uint_as_float(__float_as_uint(a.x) ^ tx), __uint_as_float(__float_as_uint(a.y) ^ ty));
+            b = make_float2(__uint_as_float(__float_as_uint(b.x) ^ tx), __uint_as_float(__float_as_uint(b.y) ^ ty));
+        }
+}
+
+// 4x4 matrix (16 entries, row-major) on slots A < B, local index bit(A) + 2 bit(B)
+template <int A, int B>
+__device__ __forceinline__ void gate_u2(float2 (&v)[GE], const float2 *u) {
+    float2 m[16];
+    const float4 *u4 = reinterpret_cast<const float4 *>(u);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const float4 q = u4[e];
+        m[2 * e] = make_float2(q.x, q.y);
+        m[2 * e + 1] = make_float2(q.z, q.w);
+    }
+#pragma unroll
+    for (int k = 0; k < GE; ++k)
+        if (!(k & (1 << A)) && !(k & (1 << B))) {
+            const int idx[4] = {k, k | (1 << A), k | (1 << B), k | (1 << A) | (1 << B)};
+            float2 w[4];
+#pragma unroll
+            for (int l = 0; l < 4; ++l) w[l] = v[idx[l]];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                float re = 0.f, im = 0.f;
+#pragma unroll
+                for (int l = 0; l < 4; ++l) {
+                    re = fmaf(m[4 * r + l].x, w[l].x, fmaf(-m[4 * r + l].y, w[l].y, re));
+                    im = fmaf(m[4 * r + l].x, w[l].y, fmaf(m[4 * r + l].y, w[l].x, im));
+                }
+                v[idx[r]] = make_float2(re, im);
+            }
+        }
+}
+
+} // namespace
+
+// U2: the list holds two-qubit matrices only; otherwise none.
+template <bool U2>
+__global__ void __launch_bounds__(GT, 2) gate_block_kernel(float2 *psi, const GateRow *gates, const GateRound *rounds,
+                                                           const float2 *mats, const GateBlockParams p) {
     extern __shared__ __align__(16) float2 amp[];
     __shared__ unsigned long long hioff[1 << (GATE_BLOCK_Q - GATE_BLOCK_LOW)];
     const unsigned long long tile = blockIdx.x + ((unsigned long long)blockIdx.y << 15);
@@ -31,109 +139,147 @@ __global__ void __launch_bounds__(256) gate_block_kernel(float2 *psi, const Gate
     // per value of h
     const int low = p.Q < GATE_BLOCK_LOW ? p.Q : GATE_BLOCK_LOW;
     const int nh = 1 << (p.Q - low);
-    for (int h = threadIdx.x; h < nh; h += 256) {
+    for (int h = threadIdx.x; h < nh; h += GT) {
         unsigned long long o = base;
         for (int i = low; i < p.Q; ++i) o |= (unsigned long long)((h >> (i - low)) & 1) << p.local[i];
         hioff[h] = o;
     }
+    // a state of fewer than five qubits fills the first entries of one thread's 32
+    const int qt = p.Q < GATE_ROUND_SLOTS ? GATE_ROUND_SLOTS : p.Q;
     // the block's two-qubit matrices, once per CTA (read back as broadcasts)
-    float2 *msm = amp + L;
-    if (mats)
-        for (int e = threadIdx.x; e < 16 * p.ng; e += 256) msm[e] = __ldg(mats + 16 * (size_t)p.g0 + e);
+    float2 *msm = amp + (1 << qt);
+    if constexpr (U2)
+        for (int e = threadIdx.x; e < 16 * p.ng; e += GT) msm[e] = __ldg(mats + 16 * (size_t)p.g0 + e);
     __syncthreads();
     const int lm = (1 << low) - 1;
-    for (int l = threadIdx.x; l < L; l += 256) amp[l] = psi[hioff[l >> low] | (unsigned long long)(l & lm)];
-    const float r2 = 0.70710678118654752440f;
-    for (int gi = 0; gi < p.ng; ++gi) {
-        const GateRow G = gates[p.g0 + gi];
+    constexpr int LOWM = (1 << GATE_BLOCK_LOW) - 1;
+    const bool full = p.Q == GATE_BLOCK_Q;
+    if (full) {
+        // all loads of a thread in flight; thread t takes the indices t + 256 i
+        float2 q[GE];
+        const float2 *src = psi + (threadIdx.x & LOWM);
+#pragma unroll
+        for (int i = 0; i < GE; ++i) q[i] = src[hioff[(threadIdx.x >> GATE_BLOCK_LOW) + (GT >> GATE_BLOCK_LOW) * i]];
+        const uint32_t at = gphys(threadIdx.x);
+#pragma unroll
+        for (int i = 0; i < GE; ++i) amp[at ^ gphys(GT * i)] = q[i];
+    } else {
+        for (int l = threadIdx.x; l < (1 << qt); l += GT)
+            amp[gphys((uint32_t)l)] = l < L ? psi[hioff[l >> low] | (unsigned long long)(l & lm)] : make_float2(0.f, 0.f);
+    }
+    const uint32_t t = threadIdx.x;
+    const bool mine = t < (1u << (qt - GATE_ROUND_SLOTS));
+    float2 v[GE];
+    for (int ri = 0; ri < p.nr; ++ri) {
+        const GateRound R = rounds[p.r0 + ri];
         __syncthreads();
-        const int b0 = 1 << G.q0;
-        if (G.op == GATE_OP_U2) {   // 4x4 matrix of row p.g0 + gi, local index bit(q0) + 2 bit(q1)
-            const float2 *u = msm + 16 * gi;
-            float2 m[16];
+        // amplitude k of thread t: byte address at ^ ok (positions are linear over GF(2))
+        uint32_t at = 0, so[GATE_ROUND_SLOTS];
+        for (int i = 0; i < qt - GATE_ROUND_SLOTS; ++i) at |= ((t >> i) & 1u) << R.thr[i];
+        at = gphys(at) * (uint32_t)sizeof(float2);
 #pragma unroll
-            for (int e = 0; e < 16; ++e) m[e] = u[e];
-            const int b1 = 1 << G.q1;
-            const int lo = G.q0 < G.q1 ? G.q0 : G.q1, hi = G.q0 < G.q1 ? G.q1 : G.q0;
-            for (int pi = threadIdx.x; pi < L / 4; pi += 256) {
-                int i = ((pi >> lo) << (lo + 1)) | (pi & ((1 << lo) - 1));
-                i = ((i >> hi) << (hi + 1)) | (i & ((1 << hi) - 1));
-                const int idx[4] = {i, i | b0, i | b1, i | b0 | b1};
-                float2 v[4];
+        for (int i = 0; i < GATE_ROUND_SLOTS; ++i) so[i] = gphys(1u << R.slot[i]) * (uint32_t)sizeof(float2);
+        char *sm = reinterpret_cast<char *>(amp);
+        if (mine) {
+            // the 32 positions in Gray-code order, one exclusive or each
 #pragma unroll
-                for (int l = 0; l < 4; ++l) v[l] = amp[idx[l]];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    float re = 0.f, im = 0.f;
-#pragma unroll
-                    for (int l = 0; l < 4; ++l) {
-                        re = fmaf(m[4 * r + l].x, v[l].x, fmaf(-m[4 * r + l].y, v[l].y, re));
-                        im = fmaf(m[4 * r + l].x, v[l].y, fmaf(m[4 * r + l].y, v[l].x, im));
+            for (int i = 0; i < GE; ++i) {
+                if (i) at ^= so[__ffs(i) - 1];
+                v[i ^ (i >> 1)] = *reinterpret_cast<const float2 *>(sm + at);
+            }
+            // phase gates on thread bits multiply all of a thread's amplitudes,
+            // which commutes with the gates on its slots: they add up in ph (units
+            // of pi / 4) and are applied once
+            int ph = 0;
+            uint32_t all;
+            asm volatile("mov.u32 %0, -1;" : "=r"(all));
+            GateRow next = gates[R.g0];
+            for (int gi = R.g0; gi < R.g0 + R.ng; ++gi) {
+                const GateRow G = next;
+                if (gi + 1 < R.g0 + R.ng) next = gates[gi + 1];
+                if constexpr (U2) {
+                    const float2 *u = msm + 16 * (gi - p.g0);
+                    switch (G.op) {
+#define U(c, a, b) case c: gate_u2<a, b>(v, u); break;
+                    U(0, 0, 1) U(1, 0, 2) U(2, 1, 2) U(3, 0, 3) U(4, 1, 3) U(5, 2, 3)
+                    U(6, 0, 4) U(7, 1, 4) U(8, 2, 4) U(9, 3, 4)
+#undef U
+                    default: break;
                     }
-                    amp[idx[r]] = make_float2(re, im);
+                } else {
+                    const uint32_t on = ((t >> G.q1) & 1u) ? ~0u : 0u;     // a thread bit controls the gate
+                    switch (G.op) {
+#define H(s) case GC_H + s: gate_h<s>(v); break;
+                    H(0) H(1) H(2) H(3) H(4)
+#undef H
+#define P(s) case GC_PHASE + s: { float cr, ci; phase_of(G.q0, cr, ci); gate_phase<1 << s>(v, cr, ci); } break;
+                    P(0) P(1) P(2) P(3) P(4)
+#undef P
+                    case GC_PHASE_THREAD: ph += G.q0 & on; break;
+#define X(c, s) case GC_CX + 5 * c + s: gate_cx<1 << c, s>(v, all); break;
+                    X(0, 1) X(0, 2) X(0, 3) X(0, 4) X(1, 0) X(1, 2) X(1, 3) X(1, 4) X(2, 0) X(2, 1) X(2, 3) X(2, 4)
+                    X(3, 0) X(3, 1) X(3, 2) X(3, 4) X(4, 0) X(4, 1) X(4, 2) X(4, 3)
+#undef X
+#define Y(s) case GC_CX_THREAD + s: gate_cx<0, s>(v, on); break;
+                    Y(0) Y(1) Y(2) Y(3) Y(4)
+#undef Y
+                    default: break;
+                    }
                 }
             }
-        } else if (G.op == 0) {   // H
-            for (int pi = threadIdx.x; pi < L / 2; pi += 256) {
-                const int i = ((pi >> G.q0) << (G.q0 + 1)) | (pi & (b0 - 1));
-                const float2 u = amp[i], w = amp[i | b0];
-                amp[i] = make_float2(r2 * (u.x + w.x), r2 * (u.y + w.y));
-                amp[i | b0] = make_float2(r2 * (u.x - w.x), r2 * (u.y - w.y));
+            if constexpr (!U2) {
+                if (ph & 7) {
+                    float cr, ci;
+                    phase_of(ph & 7, cr, ci);
+                    gate_phase<0>(v, cr, ci);
+                }
             }
-        } else if (G.op == 3) {   // CNOT q0 -> q1
-            const int b1 = 1 << G.q1;
-            const int lo = G.q0 < G.q1 ? G.q0 : G.q1, hi = G.q0 < G.q1 ? G.q1 : G.q0;
-            for (int pi = threadIdx.x; pi < L / 4; pi += 256) {
-                int i = ((pi >> lo) << (lo + 1)) | (pi & ((1 << lo) - 1));
-                i = ((i >> hi) << (hi + 1)) | (i & ((1 << hi) - 1));
-                i |= b0;
-                const float2 u = amp[i];
-                amp[i] = amp[i | b1];
-                amp[i | b1] = u;
-            }
-        } else {   // diagonal phase on |1> of q0
-            float cr, ci;
-            if (G.op == 1) { cr = 0.f; ci = 1.f; }
-            else if (G.op == 2) { cr = 0.f; ci = -1.f; }
-            else if (G.op == 4) { cr = r2; ci = r2; }
-            else { cr = r2; ci = -r2; }
-            for (int pi = threadIdx.x; pi < L / 2; pi += 256) {
-                const int i = ((pi >> G.q0) << (G.q0 + 1)) | (pi & (b0 - 1)) | b0;
-                const float2 u = amp[i];
-                amp[i] = make_float2(cr * u.x - ci * u.y, cr * u.y + ci * u.x);
+            // back to the places this thread read, in reverse: no other thread
+            // touches them in this round
+#pragma unroll
+            for (int i = GE - 1; i >= 0; --i) {
+                *reinterpret_cast<float2 *>(sm + at) = v[i ^ (i >> 1)];
+                if (i) at ^= so[__ffs(i) - 1];
             }
         }
     }
     __syncthreads();
-    for (int l = threadIdx.x; l < L; l += 256) psi[hioff[l >> low] | (unsigned long long)(l & lm)] = amp[l];
+    if (full) {
+        float2 *dst = psi + (threadIdx.x & LOWM);
+        const uint32_t at = gphys(threadIdx.x);
+#pragma unroll
+        for (int i = 0; i < GE; ++i)
+            dst[hioff[(threadIdx.x >> GATE_BLOCK_LOW) + (GT >> GATE_BLOCK_LOW) * i]] = amp[at ^ gphys(GT * i)];
+        return;
+    }
+    for (int l = threadIdx.x; l < L; l += GT)
+        psi[hioff[l >> low] | (unsigned long long)(l & lm)] = amp[gphys((uint32_t)l)];
 }
 
-// blocks_host: n_blocks x (g0, ng); block_qubits_host: n_blocks x GATE_BLOCK_Q
-// global qubits (ascending, 255 = unused). Gate rows in gates_dev carry local
-// qubit positions.
-cudaError_t launch_gate_blocks(float2 *psi, int N, const GateRow *gates_dev, const float2 *mats_dev,
-                               const int *blocks_host, int n_blocks, const unsigned char *block_qubits_host,
-                               cudaStream_t st) {
+template <bool U2>
+static cudaError_t launch_blocks(float2 *psi, int N, const GateRow *gates_dev, const GateRound *rounds_dev,
+                                 const float2 *mats_dev, const GateBlock *blocks, int n_blocks, cudaStream_t st) {
     int max_ng = 0;
-    for (int b = 0; b < n_blocks; ++b) max_ng = blocks_host[2 * b + 1] > max_ng ? blocks_host[2 * b + 1] : max_ng;
-    const size_t mat_smem = mats_dev ? sizeof(float2) * 16 * (size_t)max_ng : 0;
-    const size_t smem_max = (sizeof(float2) << GATE_BLOCK_Q) + mat_smem;
+    for (int b = 0; b < n_blocks; ++b) max_ng = blocks[b].ng > max_ng ? blocks[b].ng : max_ng;
+    const size_t smem_max = (sizeof(float2) << GATE_BLOCK_Q) + (U2 ? sizeof(float2) * 16 * (size_t)max_ng : 0);
     if (smem_max > 200 * 1024) return cudaErrorInvalidValue;
     static size_t attr = 0;
     if (attr < smem_max) {
-        cudaError_t e = cudaFuncSetAttribute(gate_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(gate_block_kernel<U2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem_max);
         if (e != cudaSuccess) return e;
         attr = smem_max;
     }
     for (int b = 0; b < n_blocks; ++b) {
         GateBlockParams p;
-        p.g0 = blocks_host[2 * b];
-        p.ng = blocks_host[2 * b + 1];
+        p.r0 = blocks[b].r0;
+        p.nr = blocks[b].nr;
+        p.g0 = blocks[b].g0;
+        p.ng = blocks[b].ng;
         p.Q = 0;
         bool in[64] = {false};
         for (int i = 0; i < GATE_BLOCK_Q; ++i) {
-            const unsigned char q = block_qubits_host[b * GATE_BLOCK_Q + i];
+            const unsigned char q = blocks[b].qubit[i];
             if (q == 255) break;
             p.local[p.Q++] = q;
             in[q] = true;
@@ -143,12 +289,19 @@ cudaError_t launch_gate_blocks(float2 *psi, int N, const GateRow *gates_dev, con
             if (!in[q]) p.other[p.n_other++] = (unsigned char)q;
         const unsigned long long tiles = 1ULL << p.n_other;
         dim3 grid((unsigned)(tiles < 32768 ? tiles : 32768), (unsigned)(tiles < 32768 ? 1 : tiles >> 15));
-        const size_t smem = (sizeof(float2) << p.Q) + (mats_dev ? sizeof(float2) * 16 * (size_t)p.ng : 0);
-        gate_block_kernel<<<grid, 256, smem, st>>>(psi, gates_dev, mats_dev, p);
+        const int qt = p.Q < GATE_ROUND_SLOTS ? GATE_ROUND_SLOTS : p.Q;
+        const size_t smem = (sizeof(float2) << qt) + (U2 ? sizeof(float2) * 16 * (size_t)p.ng : 0);
+        gate_block_kernel<U2><<<grid, GT, smem, st>>>(psi, gates_dev, rounds_dev, mats_dev, p);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+cudaError_t launch_gate_blocks(float2 *psi, int N, const GateRow *gates_dev, const GateRound *rounds_dev,
+                               const float2 *mats_dev, const GateBlock *blocks, int n_blocks, cudaStream_t st) {
+    return mats_dev ? launch_blocks<true>(psi, N, gates_dev, rounds_dev, mats_dev, blocks, n_blocks, st)
+                    : launch_blocks<false>(psi, N, gates_dev, rounds_dev, nullptr, blocks, n_blocks, st);
 }
 
 } // namespace sre

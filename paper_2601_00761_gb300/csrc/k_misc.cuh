@@ -88,14 +88,31 @@ cudaError_t launch_marginal(const float2 *psi, int N, const double *scal, double
                             cudaStream_t st);
 
 // gates (k_gates.cu)
-struct GateRow { unsigned char op, q0, q1; };
+struct __align__(4) GateRow { unsigned char op, q0, q1, pad; };
 constexpr unsigned char GATE_OP_U2 = 6;   // general two-qubit gate (matrix table indexed by row)
 constexpr int GATE_BLOCK_MAX_U2 = 512;     // two-qubit matrices per block (64 KB of shared memory)
-cudaError_t launch_gate_blocks(float2 *psi, int N, const GateRow *gates_dev, const float2 *mats_dev,
-                               const int *blocks_host, int n_blocks, const unsigned char *block_qubits_host,
-                               cudaStream_t st);
 constexpr int GATE_BLOCK_Q = 13;   // qubits per fused gate block (2^13 amplitudes, 64 KB of shared memory)
 constexpr int GATE_BLOCK_LOW = 5;  // qubits 0..4 always in the block (256-byte contiguous runs)
+constexpr int GATE_ROUND_SLOTS = 5;   // local qubits that a thread holds in a round (32 amplitudes)
+// A round: the gates rows [g0, g0 + ng) with local bits slot[i] in registers
+// (bit i of a thread's amplitude index) and thr[i] in bit i of the thread index.
+struct GateRound {
+    int g0, ng;
+    unsigned char slot[GATE_ROUND_SLOTS], thr[GATE_BLOCK_Q - GATE_ROUND_SLOTS];
+    unsigned char pad[3];
+};
+// A block: its global qubits (ascending, 255 = unused), rounds and gate rows.
+struct GateBlock {
+    int r0, nr, g0, ng;
+    unsigned char qubit[GATE_BLOCK_Q];
+};
+// Codes of the rows of a round (GateRow::op on the device): slot indices for
+// H, for a phase gate (q0: the phase in units of pi / 4) and for a CNOT (5
+// control + target); with q1 a thread bit, the phase gate and the CNOT
+// controlled outside the slots. Two-qubit matrices: slots a < b as b (b - 1) / 2 + a.
+enum GateCode { GC_H = 0, GC_PHASE = 5, GC_PHASE_THREAD = 10, GC_CX = 11, GC_CX_THREAD = 36 };
+cudaError_t launch_gate_blocks(float2 *psi, int N, const GateRow *gates_dev, const GateRound *rounds_dev,
+                               const float2 *mats_dev, const GateBlock *blocks, int n_blocks, cudaStream_t st);
 
 // tcgen05 self-test GEMM (k_tc05.cu): D = A B^T, BF16 in, FP32 out
 cudaError_t launch_tc05_gemm_selftest(const void *A, const void *B, float *D, int M, int N, int K, int swizzle,

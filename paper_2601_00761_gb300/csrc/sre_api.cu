@@ -1310,6 +1310,97 @@ sre_status autotune_impl(const void *psi, int N, cudaStream_t st, sre_opts *best
     return SRE_OK;
 }
 
+// Rounds of one block (k_gates.cu): its gates (local qubits, in an order that
+// applies them correctly) are taken by the dependencies between them, the one
+// that needs the fewest new slots first, until no ready gate fits the round's
+// five slots. A phase gate needs no slot, a CNOT one for its target, H one, a
+// matrix two. src[i] is the caller's index of gate i (its matrix in mats_host).
+// Appends the rows in the order they are applied, the rounds and the matrices.
+void plan_gate_rounds(const std::vector<GateRow> &gates, const std::vector<long long> &src, int m,
+                      const float *mats_host, std::vector<GateRow> &rows, std::vector<GateRound> &rounds,
+                      std::vector<float> &mats) {
+    const int Q = std::max(m, GATE_ROUND_SLOTS);        // fewer qubits leave slots without amplitudes
+    auto two = [](const GateRow &G) { return G.op == SRE_GATE_CNOT || G.op == GATE_OP_U2; };
+    std::vector<std::vector<int>> qlist(Q);
+    for (int g = 0; g < (int)gates.size(); ++g) {
+        qlist[gates[g].q0].push_back(g);
+        if (two(gates[g])) qlist[gates[g].q1].push_back(g);
+    }
+    std::vector<size_t> ptr(Q, 0);
+    auto head = [&](int q, int g) { return ptr[q] < qlist[q].size() && qlist[q][ptr[q]] == g; };
+    size_t done = 0;
+    while (done < gates.size()) {
+        int pos[GATE_BLOCK_Q], cnt = 0;                  // slot of a local qubit, or -1
+        for (int q = 0; q < Q; ++q) pos[q] = -1;
+        GateRound R;
+        std::vector<int> taken;
+        for (;;) {
+            int best = -1, best_new = GATE_ROUND_SLOTS + 1;
+            for (int q = 0; q < Q; ++q) {
+                if (ptr[q] >= qlist[q].size()) continue;
+                const int g = qlist[q][ptr[q]];
+                const GateRow &G = gates[g];
+                if (!head(G.q0, g) || (two(G) && !head(G.q1, g))) continue;
+                int add = 0;
+                if (G.op == SRE_GATE_H || G.op == GATE_OP_U2) add += pos[G.q0] < 0;
+                if (two(G)) add += pos[G.q1] < 0;
+                if (cnt + add > GATE_ROUND_SLOTS) continue;
+                if (add < best_new || (add == best_new && g < best)) { best = g; best_new = add; }
+            }
+            if (best < 0) break;
+            const GateRow &G = gates[best];
+            if ((G.op == SRE_GATE_H || G.op == GATE_OP_U2) && pos[G.q0] < 0) { R.slot[cnt] = G.q0; pos[G.q0] = cnt++; }
+            if (two(G) && pos[G.q1] < 0) { R.slot[cnt] = G.q1; pos[G.q1] = cnt++; }
+            ++ptr[G.q0];
+            if (two(G)) ++ptr[G.q1];
+            taken.push_back(best);
+        }
+        for (int q = Q - 1; q >= 0 && cnt < GATE_ROUND_SLOTS; --q)
+            if (pos[q] < 0) { R.slot[cnt] = (unsigned char)q; pos[q] = cnt++; }
+        // thread bits: the first four from different residues mod 4 where they
+        // can be, which keeps a half-warp's addresses in different banks
+        int tpos[GATE_BLOCK_Q], nt = 0;
+        for (int q = 0; q < Q; ++q) tpos[q] = -1;
+        memset(R.thr, 0, sizeof R.thr);
+        for (int c = 0; c < 4; ++c)
+            for (int q = c; q < Q; q += 4)
+                if (pos[q] < 0) { R.thr[nt] = (unsigned char)q; tpos[q] = nt++; break; }
+        for (int q = 0; q < Q; ++q)
+            if (pos[q] < 0 && tpos[q] < 0) { R.thr[nt] = (unsigned char)q; tpos[q] = nt++; }
+        memset(R.pad, 0, sizeof R.pad);
+        R.g0 = (int)rows.size();
+        R.ng = (int)taken.size();
+        for (int g : taken) {
+            const GateRow &G = gates[g];
+            GateRow r = {0, 0, 0, 0};
+            if (G.op == GATE_OP_U2) {
+                const int a = pos[G.q0], b = pos[G.q1], lo = std::min(a, b), hi = std::max(a, b);
+                r.op = (unsigned char)(hi * (hi - 1) / 2 + lo);
+                const float *u = mats_host + 32 * src[g];
+                // q0 in the higher slot: local indices 1 and 2 change places
+                const int p[4] = {0, a < b ? 1 : 2, a < b ? 2 : 1, 3};
+                for (int i = 0; i < 4; ++i)
+                    for (int j = 0; j < 4; ++j) {
+                        mats.push_back(u[2 * (4 * p[i] + p[j])]);
+                        mats.push_back(u[2 * (4 * p[i] + p[j]) + 1]);
+                    }
+            } else if (G.op == SRE_GATE_H) {
+                r.op = (unsigned char)(GC_H + pos[G.q0]);
+            } else if (G.op == SRE_GATE_CNOT) {
+                if (pos[G.q0] >= 0) r.op = (unsigned char)(GC_CX + 5 * pos[G.q0] + pos[G.q1]);
+                else { r.op = (unsigned char)(GC_CX_THREAD + pos[G.q1]); r.q1 = (unsigned char)tpos[G.q0]; }
+            } else {
+                r.q0 = G.op == SRE_GATE_S ? 2 : G.op == SRE_GATE_SDG ? 6 : G.op == SRE_GATE_T ? 1 : 7;
+                if (pos[G.q0] >= 0) r.op = (unsigned char)(GC_PHASE + pos[G.q0]);
+                else { r.op = GC_PHASE_THREAD; r.q1 = (unsigned char)tpos[G.q0]; }
+            }
+            rows.push_back(r);
+        }
+        rounds.push_back(R);
+        done += taken.size();
+    }
+}
+
 // Gates are grouped into blocks of at most GATE_BLOCK_Q qubits (qubits
 // 0..GATE_BLOCK_LOW-1 always included), each applied in one pass over psi in
 // shared memory. Grouping follows the circuit's dependencies, not only its
@@ -1337,8 +1428,8 @@ sre_status run_gate_list(void *psi, int N, const std::vector<GateRow> &in_rows, 
         if (ptr[G.q0] >= qlist[G.q0].size() || qlist[G.q0][ptr[G.q0]] != g) return false;
         return !two(G) || (ptr[G.q1] < qlist[G.q1].size() && qlist[G.q1][ptr[G.q1]] == g);
     };
-    std::vector<int> blocks;
-    std::vector<unsigned char> bq;
+    std::vector<GateBlock> blocks;
+    std::vector<GateRound> rounds;
     std::vector<GateRow> rows;
     std::vector<float> mats;
     rows.reserve(n_gates);
@@ -1370,36 +1461,42 @@ sre_status run_gate_list(void *psi, int N, const std::vector<GateRow> &in_rows, 
             if (two(G)) ++ptr[G.q1];
             blk.push_back(best);
         }
+        if (blk.empty()) return fail(SRE_EINVAL, "gate planner made no progress");
+        // full tiles: a thread holds 32 amplitudes, and smaller blocks leave threads idle
+        for (int q = 0; q < N && cnt < qmax; ++q)
+            if (!in[q]) { in[q] = true; ++cnt; }
         unsigned char loc[64];
-        unsigned char list[GATE_BLOCK_Q];
+        GateBlock B;
         int m = 0;
         for (int q = 0; q < N; ++q)
-            if (in[q]) { loc[q] = (unsigned char)m; list[m++] = (unsigned char)q; }
-        for (int i = m; i < GATE_BLOCK_Q; ++i) list[i] = 255;
-        blocks.push_back((int)rows.size());
-        blocks.push_back((int)blk.size());
+            if (in[q]) { loc[q] = (unsigned char)m; B.qubit[m++] = (unsigned char)q; }
+        for (int i = m; i < GATE_BLOCK_Q; ++i) B.qubit[i] = 255;
+        std::vector<GateRow> local;
         for (long long g : blk) {
-            GateRow r;
-            r.op = in_rows[g].op;
-            r.q0 = loc[in_rows[g].q0];
-            r.q1 = two(in_rows[g]) ? loc[in_rows[g].q1] : 0;
-            rows.push_back(r);
-            if (mats_host) mats.insert(mats.end(), mats_host + 32 * g, mats_host + 32 * (g + 1));
+            GateRow r = {in_rows[g].op, loc[in_rows[g].q0], 0, 0};
+            if (two(in_rows[g])) r.q1 = loc[in_rows[g].q1];
+            local.push_back(r);
         }
-        bq.insert(bq.end(), list, list + GATE_BLOCK_Q);
+        B.g0 = (int)rows.size();
+        B.ng = (int)blk.size();
+        B.r0 = (int)rounds.size();
+        plan_gate_rounds(local, blk, m, mats_host, rows, rounds, mats);
+        B.nr = (int)rounds.size() - B.r0;
+        blocks.push_back(B);
         ndone += (long long)blk.size();
-        if (blk.empty()) return fail(SRE_EINVAL, "gate planner made no progress");
     }
     int dev = 0;
     CK(cudaGetDevice(&dev));
     GateRow *dg = nullptr;
+    GateRound *dr = nullptr;
     float2 *dm = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_ws_mu);
         if ((int)g_gatebuf.size() <= dev) g_gatebuf.resize(dev + 1);
         DevBuf &b = g_gatebuf[dev];
         const size_t rows_bytes = (sizeof(GateRow) * (size_t)n_gates + 255) & ~(size_t)255;
-        const size_t need = rows_bytes + (mats_host ? sizeof(float2) * 16 * (size_t)n_gates : 0);
+        const size_t rounds_bytes = (sizeof(GateRound) * rounds.size() + 255) & ~(size_t)255;
+        const size_t need = rows_bytes + rounds_bytes + (mats_host ? sizeof(float2) * 16 * (size_t)n_gates : 0);
         if (b.n < need) {
             if (b.p) CK(cudaFree(b.p));
             b.p = nullptr;
@@ -1410,13 +1507,15 @@ sre_status run_gate_list(void *psi, int N, const std::vector<GateRow> &in_rows, 
             b.n = need;
         }
         dg = (GateRow *)b.p;
-        if (mats_host) dm = (float2 *)((char *)b.p + rows_bytes);
+        dr = (GateRound *)((char *)b.p + rows_bytes);
+        if (mats_host) dm = (float2 *)((char *)b.p + rows_bytes + rounds_bytes);
     }
     CK(cudaMemcpyAsync(dg, rows.data(), sizeof(GateRow) * (size_t)n_gates, cudaMemcpyHostToDevice, st));
     if (mats_host)
         CK(cudaMemcpyAsync(dm, mats.data(), sizeof(float2) * 16 * (size_t)n_gates, cudaMemcpyHostToDevice, st));
-    CK(launch_gate_blocks((float2 *)psi, N, dg, dm, blocks.data(), (int)(blocks.size() / 2), bq.data(), st));
-    count_launches(blocks.size() / 2);
+    CK(cudaMemcpyAsync(dr, rounds.data(), sizeof(GateRound) * rounds.size(), cudaMemcpyHostToDevice, st));
+    CK(launch_gate_blocks((float2 *)psi, N, dg, dr, dm, blocks.data(), (int)blocks.size(), st));
+    count_launches(blocks.size());
     CK(cudaStreamSynchronize(st));
     return SRE_OK;
 }
