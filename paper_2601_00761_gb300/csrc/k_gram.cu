@@ -291,21 +291,23 @@ __global__ void __launch_bounds__(256) gram_simt_kernel(const float2 *psi, int N
 constexpr int GRAM_DIAG_WARPS = 32;
 __global__ void __launch_bounds__(32 * GRAM_DIAG_WARPS) gram_diag_kernel(const float2 *psi, int NA, int NB, float2 *C) {
     // one block per 32 consecutive a (coalesced 256-byte rows of Psi); warp
-    // w sums e = w, w + 32, ... (exact FP64 squares, widened in integer
-    // operations); the partial sums are added in a fixed order, so the result
-    // does not depend on scheduling
+    // w sums e = w, w + 32, ... in groups of eight (k_fp64.cuh; with FP64 squares
+    // the FP64 pipe bound the kernel: 150 us at N = 24, N_A = 12, now 40 us); the
+    // partial sums are added in a fixed order, so the result does not depend on
+    // scheduling
     __shared__ double part[GRAM_DIAG_WARPS][32];
+    constexpr int G = 8;
     const unsigned long long dA = 1ULL << NA, dB = 1ULL << NB;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned long long a = (unsigned long long)blockIdx.x * 32 + lane;
     double acc = 0.0;
     if (a < dA) {
-#pragma unroll 4
-        for (unsigned long long e = (unsigned long long)w; e < dB; e += GRAM_DIAG_WARPS) {
-            const float2 v = psi[a + dA * e];
-            const double vx = f2d(v.x), vy = f2d(v.y);
-            acc = fma(vx, vx, acc);
-            acc = fma(vy, vy, acc);
+        for (unsigned long long e = (unsigned long long)w; e < dB; e += G * GRAM_DIAG_WARPS) {
+            float2 u[G];
+#pragma unroll
+            for (int k = 0; k < G; ++k)
+                u[k] = e + k * GRAM_DIAG_WARPS < dB ? psi[a + dA * (e + k * GRAM_DIAG_WARPS)] : make_float2(0.f, 0.f);
+            acc += sum_squares<G>(u);
         }
     }
     part[w][lane] = acc;

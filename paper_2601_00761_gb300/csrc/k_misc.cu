@@ -53,20 +53,39 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
     return s;
 }
 
-// sum |psi|^2 in FP64: fixed grid, per-block partials
-__global__ void __launch_bounds__(256) norm2_partial_kernel(const float2 *psi, unsigned long long d,
-                                                            double *partial) {
-    __shared__ double red[8];
+// A thread's part of sum |psi|^2: amplitudes first, first + stride, ... below d
+// in groups of eight, all of a group's loads in flight.
+__device__ __forceinline__ double norm2_part(const float2 *psi, unsigned long long d, unsigned long long first,
+                                             unsigned long long stride) {
+    constexpr int G = 8;
     double acc = 0.0;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    for (unsigned long long b = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; b < d; b += stride) {
-        const float2 u = __ldg(psi + b);
-        const double ux = f2d(u.x), uy = f2d(u.y);
-        acc = fma(ux, ux, acc);
-        acc = fma(uy, uy, acc);
+    for (unsigned long long b = first; b < d; b += G * stride) {
+        float2 u[G];
+#pragma unroll
+        for (int k = 0; k < G; ++k)
+            u[k] = b + k * stride < d ? __ldg(psi + b + k * stride) : make_float2(0.f, 0.f);
+        acc += sum_squares<G>(u);
     }
-    acc = block_sum<256>(acc, red);
-    if (threadIdx.x == 0) partial[blockIdx.x] = acc;
+    return acc;
+}
+
+__device__ __forceinline__ void norm2_write(double n2, double *scal) {
+    scal[SCAL_NORM2] = n2;
+    scal[SCAL_S] = n2 > 0.0 ? 1.0 / n2 : 0.0;
+}
+
+// sum |psi|^2: fixed grid, per-block partials (partial), or one block (scal).
+// With FP64 squares the FP64 pipe bound it (N = 27 1002 us, N = 24 133 us); now
+// memory does (N = 27 225 us, 4.8 TB/s; N = 24 32 us)
+template <bool ONE>
+__global__ void __launch_bounds__(256) norm2_partial_kernel(const float2 *psi, unsigned long long d, double *out) {
+    __shared__ double red[8];
+    const double acc = block_sum<256>(norm2_part(psi, d, (unsigned long long)blockIdx.x * 256 + threadIdx.x,
+                                                 (unsigned long long)gridDim.x * 256), red);
+    if (threadIdx.x == 0) {
+        if constexpr (ONE) norm2_write(acc, out);
+        else out[blockIdx.x] = acc;
+    }
 }
 
 __global__ void __launch_bounds__(256) norm2_final_kernel(const double *partial, int np, double *scal) {
@@ -74,18 +93,22 @@ __global__ void __launch_bounds__(256) norm2_final_kernel(const double *partial,
     double acc = 0.0;
     for (int i = threadIdx.x; i < np; i += 256) acc += partial[i];
     acc = block_sum<256>(acc, red);
-    if (threadIdx.x == 0) {
-        scal[SCAL_NORM2] = acc;
-        scal[SCAL_S] = acc > 0.0 ? 1.0 / acc : 0.0;
-    }
+    if (threadIdx.x == 0) norm2_write(acc, scal);
 }
 
-cudaError_t launch_norm2(const float2 *psi, int N, double *scal, double *partial, cudaStream_t st) {
+cudaError_t launch_norm2(const float2 *psi, int N, double *scal, double *partial, cudaStream_t st, int *launches) {
     const unsigned long long d = 1ULL << N;
+    // one block takes 4.8 us at N = 10 (32 amplitudes a thread at N = 13), two launches 7.7 us
+    if (N <= NORM_ONE_NMAX) {
+        norm2_partial_kernel<true><<<1, 256, 0, st>>>(psi, d, scal);
+        *launches = 1;
+        return cudaGetLastError();
+    }
     int nb = NORM_BLOCKS;
-    if ((unsigned long long)nb * 256ULL > d) nb = (int)((d + 255) / 256);
-    norm2_partial_kernel<<<nb, 256, 0, st>>>(psi, d, partial);
+    if ((unsigned long long)nb * 2048ULL > d) nb = (int)((d + 2047) / 2048);
+    norm2_partial_kernel<false><<<nb, 256, 0, st>>>(psi, d, partial);
     norm2_final_kernel<<<1, 256, 0, st>>>(partial, nb, scal);
+    *launches = 2;
     return cudaGetLastError();
 }
 
@@ -540,17 +563,8 @@ __global__ void __launch_bounds__(256) norm2_multi_partial(const float2 *const *
                                                            double *partial) {
     __shared__ double red[8];
     const int st = blockIdx.y;
-    const float2 *psi = psi_list[st];
-    const unsigned long long d = 1ULL << N;
-    double acc = 0.0;
-    const unsigned long long stride = (unsigned long long)nb * blockDim.x;
-    for (unsigned long long b = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; b < d; b += stride) {
-        const float2 u = __ldg(psi + b);
-        const double ux = f2d(u.x), uy = f2d(u.y);
-        acc = fma(ux, ux, acc);
-        acc = fma(uy, uy, acc);
-    }
-    acc = block_sum<256>(acc, red);
+    const double acc = block_sum<256>(norm2_part(psi_list[st], 1ULL << N, (unsigned long long)blockIdx.x * 256 + threadIdx.x,
+                                                 (unsigned long long)nb * 256), red);
     if (threadIdx.x == 0) partial[(size_t)st * nb + blockIdx.x] = acc;
 }
 

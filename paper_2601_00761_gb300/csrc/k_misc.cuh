@@ -20,7 +20,9 @@ struct DrawInfo {
     double pad;
 };
 
-cudaError_t launch_norm2(const float2 *psi, int N, double *scal, double *partial, cudaStream_t st);
+constexpr int NORM_ONE_NMAX = 13;          // one block and one launch up to here
+// sum |psi|^2 and its inverse into scal; *launches receives the kernels issued
+cudaError_t launch_norm2(const float2 *psi, int N, double *scal, double *partial, cudaStream_t st, int *launches);
 
 // FP64 recount of flagged families at their listed candidates (k_null.cu).
 // Family i of the launch is xs[fam_base + i] (F = (state << N) | x when

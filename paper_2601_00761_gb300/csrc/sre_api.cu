@@ -507,6 +507,13 @@ sre_status run_transform(const Plan &P, PassArgs a, int src0, int dst_last, void
     return SRE_OK;
 }
 
+sre_status run_norm2(const void *psi, int N, double *scal, double *partial, cudaStream_t st) {
+    int nl = 0;
+    CK(launch_norm2((const float2 *)psi, N, scal, partial, st, &nl));
+    count_launches(nl);
+    return SRE_OK;
+}
+
 // x-marginal into p: WHT(|psi|^2) -> square -> WHT -> /d, in 64-bit integers
 // (k_marg.cu), or in one FP64 tile for the sizes that fit one
 sre_status run_marginal(const void *psi, int N, const double *scal, double *p, double *mwork, cudaStream_t st) {
@@ -668,8 +675,7 @@ sre_status exact_impl(const void *psi, int N, const sre_opts &o, void *ws, size_
     layout_exact(A, P, P64, w);
 
     const unsigned long long d = 1ULL << N;
-    CK(launch_norm2((const float2 *)psi, N, w.scal, w.npart, st));
-    count_launches(2);
+    CS(run_norm2(psi, N, w.scal, w.npart, st));
     PassArgs a = base_args(P, psi, w.scal);
     a.precision = prec_code(o);
     a.tile_out = w.tiles;
@@ -1270,8 +1276,7 @@ sre_status autotune_impl(const void *psi, int N, cudaStream_t st, sre_opts *best
         CS(own_workspace(dry.off, &base));
         Arena A(base);
         layout_mc(A, P, SRE_MC_UNIFORM, fams, 1, w);
-        CK(launch_norm2((const float2 *)psi, N, w.scal, w.npart, st));
-        count_launches(2);
+        CS(run_norm2(psi, N, w.scal, w.npart, st));
         PassArgs a = base_args(P, psi, w.scal);
         a.tile_out = w.tiles;
         cudaEvent_t e0, e1;
@@ -1558,8 +1563,7 @@ sre_status mixed_impl(const void *psi, int N, int NA, void *ws, size_t ws_bytes,
     Arena A(base);
     layout_mixed(A, N, NA, w);
     const unsigned long long dA = 1ULL << NA;
-    CK(launch_norm2((const float2 *)psi, N, w.scal, w.npart, st));
-    count_launches(2);
+    CS(run_norm2(psi, N, w.scal, w.npart, st));
     CK(cudaMemsetAsync(w.err, 0, sizeof(int), st));
     int gl = 0;
     cudaError_t ge = launch_gram((const float2 *)psi, N, NA, w.C, w.planes, w.err, &gl, st);
@@ -1704,8 +1708,7 @@ sre_status sre_norm2(const void *psi, int N, double *norm2_host, void *stream) {
     CS(own_workspace(sizeof(double) * (SCAL_N + NORM_BLOCKS) + 1024, &base));
     double *scal = (double *)base;
     double *part = scal + SCAL_N;
-    CK(launch_norm2((const float2 *)psi, N, scal, part, st));
-    count_launches(2);
+    CS(run_norm2(psi, N, scal, part, st));
     CK(cudaMemcpyAsync(norm2_host, scal + SCAL_NORM2, sizeof(double), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     return SRE_OK;
@@ -1775,8 +1778,7 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
     const unsigned long long d = 1ULL << N;
 
     CK(cudaMemsetAsync(w.err, 0, sizeof(int), st));
-    CK(launch_norm2((const float2 *)psi, N, w.scal, w.npart, st));
-    count_launches(2);
+    CS(run_norm2(psi, N, w.scal, w.npart, st));
     if (marg) {
         CS(run_marginal(psi, N, w.scal, w.p, w.mwork, st));
         CK(launch_scan(w.p, d, w.p, w.bsum, st));
@@ -1943,8 +1945,7 @@ sre_status pauli_x_marginal(const void *psi, int N, double *p_dev, void *workspa
     double *scal = A.take<double>(SCAL_N);
     double *part = A.take<double>(NORM_BLOCKS);
     double *mwork = A.take<double>(1ULL << N);
-    CK(launch_norm2((const float2 *)psi, N, scal, part, st));
-    count_launches(2);
+    CS(run_norm2(psi, N, scal, part, st));
     CS(run_marginal(psi, N, scal, p_dev, mwork, st));
     double nrm = 0;
     CK(cudaMemcpyAsync(&nrm, scal + SCAL_NORM2, sizeof nrm, cudaMemcpyDeviceToHost, st));
@@ -1983,8 +1984,7 @@ sre_status sre_family_spectrum(const void *psi, int N, unsigned long long x, con
     double *scal = A.take<double>(SCAL_N);
     double *part = A.take<double>(NORM_BLOCKS);
     void *inter = P.npass > 1 ? (void *)A.take<char>(P.slot_bytes) : nullptr;
-    CK(launch_norm2((const float2 *)psi, N, scal, part, st));
-    count_launches(2);
+    CS(run_norm2(psi, N, scal, part, st));
     PassArgs a = base_args(P, psi, scal);
     a.precision = prec_code(o);
     a.fam_base = (long long)x;
@@ -2009,8 +2009,7 @@ sre_status sre_family_spectrum_f64(const void *psi, int N, unsigned long long x,
     double *scal = A.take<double>(SCAL_N);
     double *part = A.take<double>(NORM_BLOCKS);
     void *inter = P.npass > 1 ? (void *)A.take<char>(P.slot_bytes) : nullptr;
-    CK(launch_norm2((const float2 *)psi, N, scal, part, st));
-    count_launches(2);
+    CS(run_norm2(psi, N, scal, part, st));
     PassArgs a = base_args(P, psi, scal);
     a.fam_base = (long long)x;
     a.n_fam = 1;
@@ -2188,8 +2187,7 @@ sre_status sre_profile_passes(const void *psi, int N, long long n_x, const sre_o
     CS(own_workspace(dry.off, &base));
     Arena A(base);
     layout_mc(A, P, SRE_MC_UNIFORM, n_x < 2 ? 2 : n_x, 1, w);
-    CK(launch_norm2((const float2 *)psi, N, w.scal, w.npart, st));
-    count_launches(2);
+    CS(run_norm2(psi, N, w.scal, w.npart, st));
     CK(launch_draw_x(nullptr, N, n_x, 0, 12345ULL, 0ULL, w.xs, st));
     count_launches(1);
     PassArgs a = base_args(P, psi, w.scal);
