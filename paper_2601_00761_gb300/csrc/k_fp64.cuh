@@ -70,4 +70,29 @@ struct NeuSum {
     __device__ __forceinline__ double value() const { return s + c; }
 };
 
+// Sums over a warp of V values per lane (V a power of two up to 32) by recursive
+// halving: each step hands half of the values to the partner lane, so the warp
+// issues V - 1 + (5 - log2 V) additions instead of 5 V. Returns the total of
+// value id (set per lane; lanes that share an id hold the same total).
+template <int V>
+__device__ __forceinline__ double warp_sums(double (&v)[V], int &id) {
+    static_assert(V >= 1 && V <= 32 && (V & (V - 1)) == 0, "a power of two");
+    const int lane = threadIdx.x & 31;
+    id = 0;
+    int o = 16;
+#pragma unroll
+    for (int w = V / 2; w >= 1; w /= 2) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+            const double send = up ? v[i] : v[i + w], keep = up ? v[i + w] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        id |= up ? w : 0;
+        o >>= 1;
+    }
+    for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
+}
+
 }  // namespace sre

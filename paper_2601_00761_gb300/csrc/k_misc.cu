@@ -78,10 +78,12 @@ __device__ __forceinline__ void norm2_write(double n2, double *scal) {
 // With FP64 squares the FP64 pipe bound it (N = 27 1002 us, N = 24 133 us); now
 // memory does (N = 27 225 us, 4.8 TB/s; N = 24 32 us)
 template <bool ONE>
-__global__ void __launch_bounds__(256) norm2_partial_kernel(const float2 *psi, unsigned long long d, double *out) {
+__global__ void __launch_bounds__(256) norm2_partial_kernel(const float2 *psi, unsigned long long d, double *out,
+                                                            unsigned long long *zero) {
     __shared__ double red[8];
     const double acc = block_sum<256>(norm2_part(psi, d, (unsigned long long)blockIdx.x * 256 + threadIdx.x,
                                                  (unsigned long long)gridDim.x * 256), red);
+    if (zero && blockIdx.x == 0 && threadIdx.x < 2) zero[threadIdx.x] = 0ULL;
     if (threadIdx.x == 0) {
         if constexpr (ONE) norm2_write(acc, out);
         else out[blockIdx.x] = acc;
@@ -96,17 +98,18 @@ __global__ void __launch_bounds__(256) norm2_final_kernel(const double *partial,
     if (threadIdx.x == 0) norm2_write(acc, scal);
 }
 
-cudaError_t launch_norm2(const float2 *psi, int N, double *scal, double *partial, cudaStream_t st, int *launches) {
+cudaError_t launch_norm2(const float2 *psi, int N, double *scal, double *partial, cudaStream_t st, int *launches,
+                         unsigned long long *zero) {
     const unsigned long long d = 1ULL << N;
     // one block takes 4.8 us at N = 10 (32 amplitudes a thread at N = 13), two launches 7.7 us
     if (N <= NORM_ONE_NMAX) {
-        norm2_partial_kernel<true><<<1, 256, 0, st>>>(psi, d, scal);
+        norm2_partial_kernel<true><<<1, 256, 0, st>>>(psi, d, scal, zero);
         *launches = 1;
         return cudaGetLastError();
     }
     int nb = NORM_BLOCKS;
     if ((unsigned long long)nb * 2048ULL > d) nb = (int)((d + 2047) / 2048);
-    norm2_partial_kernel<false><<<nb, 256, 0, st>>>(psi, d, partial);
+    norm2_partial_kernel<false><<<nb, 256, 0, st>>>(psi, d, partial, zero);
     norm2_final_kernel<<<1, 256, 0, st>>>(partial, nb, scal);
     *launches = 2;
     return cudaGetLastError();
@@ -162,56 +165,84 @@ cudaError_t launch_fam_reduce(const TilePartial *tp, long long n_fam, int tiles,
     return cudaGetLastError();
 }
 
-// totals over families (exact sweep): per-block partials over contiguous
-// chunks (fixed order), then one block; also the list of candidate families
-// (order irrelevant: the FP64 counts are integers).
-__global__ void __launch_bounds__(256) exact_partial_kernel(const FamMoments *fm, long long n_fam, double *partial,
-                                                            unsigned long long *flag_list,
-                                                            unsigned long long *n_flag) {
-    __shared__ double red[8];
-    const long long per = (n_fam + gridDim.x - 1) / gridDim.x;
-    const long long lo = (long long)blockIdx.x * per, hi = lo + per < n_fam ? lo + per : n_fam;
+// Totals over the families of each of a run of states: blocks (x) over
+// contiguous chunks of a state's families (y), partial sums in the order of the
+// families, and the state's last block to finish adds the partials in block
+// order, so nothing depends on scheduling. The candidate families go to flags
+// (their order is irrelevant: the FP64 counts are integers). FP64 issue bounds
+// it; with 1024 blocks whatever the size and one warp-wide sum per value the two
+// kernels before took 27 + 20 us for the 1024 families of N = 10 and 38 + 20 us
+// for N = 18, one block per state of a batch 175 us: now 11, 15 (N = 16) and 32 us.
+__global__ void __launch_bounds__(256) totals_kernel(const TotalsArgs a) {
+    __shared__ double red[8][8];
+    __shared__ bool last;
+    const int st = a.s0 + blockIdx.y, nb = gridDim.x;
+    const FamMoments *fm = a.fm + ((((long long)st) << a.N) - a.fm_first);
+    const long long n = 1LL << a.N, per = (n + nb - 1) / nb;
+    const long long lo = (long long)blockIdx.x * per, hi = lo + per < n ? lo + per : n;
     NeuSum s0, s1, s2, s3, sq;
-    double c = 0;
     for (long long f = lo + threadIdx.x; f < hi; f += 256) {
-        const FamMoments &m = fm[f];
-        s0.add(m.m[0]); s1.add(m.m[1]); s2.add(m.m[2]); s3.add(m.m[3]); c += (double)m.cand;
+        const FamMoments m = fm[f];
+        s0.add(m.m[0]); s1.add(m.m[1]); s2.add(m.m[2]); s3.add(m.m[3]);
         if (f > 0) sq.add(m.m[1] * m.m[1]);
-        if (m.cand && flag_list) {
-            unsigned long long pos = atomicAdd(n_flag, 1ULL);
-            flag_list[pos] = (unsigned long long)f;
+        if (m.cand && a.flags) a.flags[atomicAdd(a.n_flag, 1ULL)] = ((unsigned long long)st << a.N) | (unsigned long long)f;
+    }
+    // value v of the block in thread v of warp 0
+    auto block_totals = [&](double (&v)[8]) -> double {
+        int id;
+        const double t = warp_sums<8>(v, id);
+        __syncthreads();
+        if ((threadIdx.x & 3) == 0) red[threadIdx.x >> 5][id] = t;
+        __syncthreads();
+        double r = 0.0;
+        if (threadIdx.x < 32) {
+            const int w = threadIdx.x >> 3, i = threadIdx.x & 7;
+            r = red[2 * w][i] + red[2 * w + 1][i];
+            r += __shfl_xor_sync(0xffffffffu, r, 8);
+            r += __shfl_xor_sync(0xffffffffu, r, 16);
+        }
+        return r;
+    };
+    double v[8] = {s0.value(), s1.value(), s2.value(), s3.value(), sq.value(), 0.0, 0.0, 0.0};
+    const double t = block_totals(v);
+    double *part = a.partial + 5 * ((size_t)blockIdx.y * nb);
+    if (nb > 1) {
+        if (threadIdx.x < 5) {
+            part[5 * (size_t)blockIdx.x + threadIdx.x] = t;
+            __threadfence();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            last = atomicAdd(a.done + blockIdx.y, 1u) == (unsigned)nb - 1;
+        }
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        NeuSum q[5];
+        for (int i = threadIdx.x; i < nb; i += 256)
+#pragma unroll
+            for (int k = 0; k < 5; ++k) q[k].add(__ldcg(part + 5 * (size_t)i + k));
+#pragma unroll
+        for (int k = 0; k < 5; ++k) v[k] = q[k].value();
+        v[5] = v[6] = v[7] = 0.0;
+        const double u = block_totals(v);
+        if (threadIdx.x < 5) a.out[TOT_N * (size_t)st + (threadIdx.x < 4 ? threadIdx.x : 5)] = u;
+    } else if (threadIdx.x < 5) {
+        a.out[TOT_N * (size_t)st + (threadIdx.x < 4 ? threadIdx.x : 5)] = t;
+    }
+    if (threadIdx.x == 0) {
+        a.out[TOT_N * (size_t)st + 6] = fm[0].m[1];
+        if (a.norm2) {
+            // every block of the launch's only state has flagged its families
+            a.out[TOT_N] = *a.norm2;
+            a.out[TOT_N + 1] = a.n_flag ? (double)*reinterpret_cast<volatile unsigned long long *>(a.n_flag) : 0.0;
         }
     }
-    double a0 = s0.value(), a1 = s1.value(), a2 = s2.value(), a3 = s3.value(), q = sq.value();
-    a0 = block_sum<256>(a0, red);
-    a1 = block_sum<256>(a1, red);
-    a2 = block_sum<256>(a2, red);
-    a3 = block_sum<256>(a3, red);
-    c = block_sum<256>(c, red);
-    q = block_sum<256>(q, red);
-    if (threadIdx.x == 0) {
-        double *o = partial + 6 * blockIdx.x;
-        o[0] = a0; o[1] = a1; o[2] = a2; o[3] = a3; o[4] = c; o[5] = q;
-    }
 }
 
-__global__ void __launch_bounds__(256) exact_final_kernel(const double *partial, int n_part, const FamMoments *fm0,
-                                                          double *out) {
-    __shared__ double red[8];
-    for (int a = 0; a < 6; ++a) {
-        NeuSum ns;
-        for (int i = threadIdx.x; i < n_part; i += 256) ns.add(partial[6 * i + a]);
-        const double s = block_sum<256>(ns.value(), red);
-        if (threadIdx.x == 0) out[a] = s;
-    }
-    if (threadIdx.x == 0) out[6] = fm0[0].m[1];
-}
-
-cudaError_t launch_exact_totals(const FamMoments *fm, long long n_fam, double *partial, int n_part,
-                                double *out, unsigned long long *flag_list, unsigned long long *n_flag,
-                                cudaStream_t st) {
-    exact_partial_kernel<<<n_part, 256, 0, st>>>(fm, n_fam, partial, flag_list, n_flag);
-    exact_final_kernel<<<1, 256, 0, st>>>(partial, n_part, fm, out);
+cudaError_t launch_totals(const TotalsArgs &a, int ns, cudaStream_t st) {
+    totals_kernel<<<dim3((unsigned)totals_blocks(a.N, ns), (unsigned)ns), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -584,47 +615,6 @@ cudaError_t launch_norm2_multi(const float2 *const *psi_list, int n_states, int 
                                double *norm2, double *s, cudaStream_t st) {
     norm2_multi_partial<<<dim3(nb, n_states), 256, 0, st>>>(psi_list, N, nb, partial);
     norm2_multi_final<<<n_states, 256, 0, st>>>(partial, nb, norm2, s);
-    return cudaGetLastError();
-}
-
-// per-state totals of the family sums of states [s0, s0 + ns): one block per
-// state over its 2^N consecutive families (fixed order); candidate families
-// appended to flags as F = (state << N) | x.
-__global__ void __launch_bounds__(256) state_totals_kernel(const FamMoments *fm, long long fm_first_family, int N,
-                                                           int s0, double *totals, unsigned long long *flags,
-                                                           unsigned long long *n_flag) {
-    __shared__ double red[8];
-    const int st = s0 + blockIdx.x;
-    const long long nf = 1LL << N;
-    const long long f0 = ((long long)st << N) - fm_first_family;
-    NeuSum n0, n1, n2, n3, nq;
-    double c = 0;
-    for (long long f = threadIdx.x; f < nf; f += 256) {
-        const FamMoments &m = fm[f0 + f];
-        n0.add(m.m[0]); n1.add(m.m[1]); n2.add(m.m[2]); n3.add(m.m[3]); c += (double)m.cand;
-        if (f > 0) nq.add(m.m[1] * m.m[1]);
-        if (m.cand) {
-            const unsigned long long pos = atomicAdd(n_flag, 1ULL);
-            flags[pos] = ((unsigned long long)st << N) | (unsigned long long)f;
-        }
-    }
-    double a0 = n0.value(), a1 = n1.value(), a2 = n2.value(), a3 = n3.value(), q = nq.value();
-    a0 = block_sum<256>(a0, red);
-    a1 = block_sum<256>(a1, red);
-    a2 = block_sum<256>(a2, red);
-    a3 = block_sum<256>(a3, red);
-    c = block_sum<256>(c, red);
-    q = block_sum<256>(q, red);
-    if (threadIdx.x == 0) {
-        double *o = totals + TOT_N * (size_t)st;
-        o[0] = a0; o[1] = a1; o[2] = a2; o[3] = a3; o[4] = c; o[5] = q; o[6] = fm[f0].m[1];
-    }
-}
-
-cudaError_t launch_state_totals(const FamMoments *fm, long long fm_first_family, int N, int s0, int ns,
-                                double *totals, unsigned long long *flags, unsigned long long *n_flag,
-                                cudaStream_t st) {
-    state_totals_kernel<<<ns, 256, 0, st>>>(fm, fm_first_family, N, s0, totals, flags, n_flag);
     return cudaGetLastError();
 }
 

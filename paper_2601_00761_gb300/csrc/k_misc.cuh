@@ -21,8 +21,32 @@ struct DrawInfo {
 };
 
 constexpr int NORM_ONE_NMAX = 13;          // one block and one launch up to here
-// sum |psi|^2 and its inverse into scal; *launches receives the kernels issued
-cudaError_t launch_norm2(const float2 *psi, int N, double *scal, double *partial, cudaStream_t st, int *launches);
+// sum |psi|^2 and its inverse into scal; *launches receives the kernels issued;
+// zero (or NULL): two words that the launch clears
+cudaError_t launch_norm2(const float2 *psi, int N, double *scal, double *partial, cudaStream_t st, int *launches,
+                         unsigned long long *zero = nullptr);
+
+// Totals of the family sums of states s0 .. s0 + ns - 1 (N qubits each; family
+// f of state st at fm[(st << N) + f - fm_first]) into out[TOT_N st ..] (slot 4
+// is unused). flags / n_flag (or NULL): list and count of the candidate
+// families. partial: 5 totals_blocks(N, ns) doubles a state; done: a zeroed
+// counter a state. norm2 (one state only, or NULL): the norm, which then goes to
+// out[TOT_N] with the number of flagged families in out[TOT_N + 1].
+constexpr int TOTALS_BLOCKS = 304;
+inline int totals_blocks(int N, int ns) {
+    const long long want = (1LL << N) / 256, most = ns > 0 ? (TOTALS_BLOCKS + ns - 1) / ns : 1;
+    return (int)(want < 1 ? 1 : want < most ? want : most);
+}
+struct TotalsArgs {
+    const FamMoments *fm;
+    long long fm_first;
+    int N, s0;
+    double *out, *partial;
+    unsigned *done;
+    unsigned long long *flags, *n_flag;
+    const double *norm2;
+};
+cudaError_t launch_totals(const TotalsArgs &a, int ns, cudaStream_t st);
 
 // FP64 recount of flagged families at their listed candidates (k_null.cu).
 // Family i of the launch is xs[fam_base + i] (F = (state << N) | x when
@@ -44,6 +68,7 @@ struct NullDirectArgs {
     int cand_max, kdirect;
     double eps;
     unsigned long long *counts, *ovf, *ovf_n;
+    unsigned long long *total;        // sum of the counts of every launch (zeroed before the first), or NULL
 };
 cudaError_t launch_null_direct(const NullDirectArgs &a, long long n_fam, cudaStream_t st);
 // per-family sums of a launch's tile partials into fm[fm_base + slot], or,
@@ -51,9 +76,6 @@ cudaError_t launch_null_direct(const NullDirectArgs &a, long long n_fam, cudaStr
 cudaError_t launch_fam_reduce(const TilePartial *tp, long long n_fam, int tiles, const unsigned long long *xs,
                               long long fam_base, int N, int M_last, int RL, FamMoments *fm, long long fm_base,
                               float *W, long long nr, cudaStream_t st, const unsigned long long *perm = nullptr);
-cudaError_t launch_exact_totals(const FamMoments *fm, long long n_fam, double *partial, int n_part,
-                                double *out, unsigned long long *flag_list, unsigned long long *n_flag,
-                                cudaStream_t st);
 cudaError_t launch_sum_u64(const unsigned long long *v, long long n, unsigned long long *out, cudaStream_t st);
 cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, double *bsum, cudaStream_t st);
 cudaError_t launch_draw_x(const double *cdf, int N, long long n_x, int mode, unsigned long long seed,
@@ -65,9 +87,6 @@ cudaError_t launch_mc_stats(const FamMoments *fm, const float *cz, long long n_x
                             double *y, double *out, cudaStream_t st);
 cudaError_t launch_norm2_multi(const float2 *const *psi_list, int n_states, int N, double *partial, int nb,
                                double *norm2, double *s, cudaStream_t st);
-cudaError_t launch_state_totals(const FamMoments *fm, long long fm_first_family, int N, int s0, int ns,
-                                double *totals, unsigned long long *flags, unsigned long long *n_flag,
-                                cudaStream_t st);
 cudaError_t launch_count_scatter(const unsigned long long *flags, const unsigned long long *counts, long long n,
                                  int N, unsigned long long *state_count, cudaStream_t st);
 cudaError_t launch_philox_test(const unsigned long long *ctr_key, unsigned long long *out, int n, cudaStream_t st);

@@ -22,6 +22,8 @@
 //    operations per point.
 // Points of a coset that were not listed lie below the threshold and count
 // nothing, so every route counts exactly the FP64 decisions.
+#include <cooperative_groups.h>
+
 #include "k_misc.cuh"
 #include "k_fp64.cuh"
 
@@ -32,6 +34,7 @@ namespace {
 constexpr int ND_THREADS = 256;
 constexpr int ND_GROUP = 8;      // z' summed per sweep over g (direct route)
 constexpr int NB_CHUNK = 16;     // bins accumulated per sweep over g (coset route)
+constexpr int ND_CLUSTER = 8, ND_CLUSTER_FAMS = 38;   // 152 SMs / 8 = 19 clusters, two rounds
 constexpr int NB_MAXBITS = 6;    // span dimension up to which the coset route is taken
 
 // v with its sign bit flipped when sgn = 1u << 31
@@ -58,11 +61,11 @@ __device__ __forceinline__ void hval(const float2 *psi, uint32_t x, int j, uint3
 
 // direct route: H at G listed z' per sweep over all g
 template <int G>
-__device__ __forceinline__ void direct_sums(const float2 *psi, uint32_t x, int j, uint32_t half,
-                                            const uint32_t (&zl)[ND_GROUP], double (&ar)[ND_GROUP],
-                                            double (&ai)[ND_GROUP]) {
+__device__ __forceinline__ void direct_sums(const float2 *psi, uint32_t x, int j, uint32_t half, uint32_t first,
+                                            uint32_t stride, const uint32_t (&zl)[ND_GROUP], double (&ar)[NB_CHUNK],
+                                            double (&ai)[NB_CHUNK]) {
 #pragma unroll 2
-    for (uint32_t g = threadIdx.x; g < half; g += ND_THREADS) {
+    for (uint32_t g = first; g < half; g += stride) {
         double hr, hi;
         hval(psi, x, j, half, g, hr, hi);
 #pragma unroll
@@ -84,7 +87,8 @@ __device__ __forceinline__ void direct_sums(const float2 *psi, uint32_t x, int j
 template <int MB>
 __device__ __forceinline__ void coset_sums(const float2 *psi, uint32_t x, int j, uint32_t half, uint32_t z0,
                                            const uint32_t *vb, const uint32_t *piv, int m, uint32_t offq,
-                                           double (&ar)[NB_CHUNK], double (&ai)[NB_CHUNK]) {
+                                           uint32_t first, uint32_t stride, double (&ar)[NB_CHUNK],
+                                           double (&ai)[NB_CHUNK]) {
     constexpr int NBIN = 1 << MB;
     uint32_t offl[NBIN];
 #pragma unroll
@@ -96,7 +100,7 @@ __device__ __forceinline__ void coset_sums(const float2 *psi, uint32_t x, int j,
         offl[b] = o;
     }
     const uint32_t nr = half >> m;
-    for (uint32_t r = threadIdx.x; r < nr; r += ND_THREADS) {
+    for (uint32_t r = first; r < nr; r += stride) {
         uint32_t gr = r, C = 0;
         for (int i = 0; i < m; ++i) gr = (uint32_t)insert0(gr, (int)piv[i]);
         for (int i = 0; i < m; ++i) C |= (uint32_t)(__popc(gr & vb[i]) & 1) << piv[i];
@@ -113,35 +117,41 @@ __device__ __forceinline__ void coset_sums(const float2 *psi, uint32_t x, int j,
     }
 }
 
-// fixed-order block sums of the first n (<= NB_CHUNK) pairs (ar, ai): warp
-// butterflies, then the warps in order; the sums land in out_r/out_i[0..n)
-template <int NV>
-__device__ __forceinline__ void block_sums(double (&ar)[NV], double (&ai)[NV], int n, double (*red)[2 * NB_CHUNK],
-                                           double *out_r, double *out_i) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// fixed-order block sums of the first NB pairs (ar, ai): recursive halving in
+// the warps (k_fp64.cuh), then the warps in order, and with a cluster of CL CTAs
+// the CTAs in order; the sums land in out_r/out_i[0..NB) of the cluster's first
+// CTA. With a warp butterfly per value these sums took 10 us of FP64 issue for a
+// family with one candidate.
+template <int NB, int CL>
+__device__ __forceinline__ void block_sums(double (&ar)[NB_CHUNK], double (&ai)[NB_CHUNK], double (*red)[2 * NB_CHUNK],
+                                           double *cta, double *out_r, double *out_i) {
+    double v[2 * NB];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ar[i] += __shfl_xor_sync(0xffffffffu, ar[i], o);
-            ai[i] += __shfl_xor_sync(0xffffffffu, ai[i], o);
-        }
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            red[warp][i] = ar[i];
-            red[warp][NB_CHUNK + i] = ai[i];
-        }
-    }
+    for (int i = 0; i < NB; ++i) { v[i] = ar[i]; v[NB + i] = ai[i]; }
+    int id;
+    const double w = warp_sums<2 * NB>(v, id);
+    red[threadIdx.x >> 5][id] = w;                      // lanes that share an id hold the same value
     __syncthreads();
     const int t = threadIdx.x;
-    if (t < 2 * n) {
-        const int i = t < n ? t : t - n, col = t < n ? i : NB_CHUNK + i;
-        double v = 0.0;
-        for (int w = 0; w < ND_THREADS / 32; ++w) v += red[w][col];
-        if (t < n) out_r[i] = v;
-        else out_i[i] = v;
+    double s = 0.0;
+    if (t < 2 * NB) {
+#pragma unroll
+        for (int i = 0; i < ND_THREADS / 32; ++i) s += red[i][t];
+    }
+    if constexpr (CL > 1) {
+        namespace cg = cooperative_groups;
+        auto cl = cg::this_cluster();
+        if (t < 2 * NB) cta[t] = s;
+        cl.sync();
+        if (cl.block_rank() == 0 && t < 2 * NB) {
+            s = 0.0;
+            for (int r = 0; r < CL; ++r) s += *cl.map_shared_rank(cta + t, r);
+        }
+        cl.sync();                                       // cta is reused
+    }
+    if (t < 2 * NB) {
+        if (t < NB) out_r[t] = s;
+        else out_i[t - NB] = s;
     }
     __syncthreads();
 }
@@ -156,17 +166,22 @@ __device__ __forceinline__ int count_pair(double hr, double hi, bool xnz, double
 
 enum { NR_COSET = 0, NR_DIRECT = 1, NR_OVERFLOW = 2 };
 
+// CL: CTAs of a cluster that share a family
+template <int CL>
 __global__ void __launch_bounds__(ND_THREADS) null_direct_kernel(const NullDirectArgs a) {
     __shared__ uint32_t zs[NULL_CAND_MAX];
     __shared__ uint32_t vb[NB_MAXBITS], piv[NB_MAXBITS];
     __shared__ int s_mode, s_m;
     __shared__ double red[ND_THREADS / 32][2 * NB_CHUNK];
     __shared__ double bin_r[1 << NB_MAXBITS], bin_i[1 << NB_MAXBITS];
-    const long long slot = blockIdx.x;
+    __shared__ double cta[2 * NB_CHUNK];
+    const long long slot = blockIdx.x / CL;
+    const uint32_t rank = blockIdx.x % CL, first = rank * ND_THREADS + threadIdx.x, stride = CL * ND_THREADS;
+    const bool lead = rank == 0;                      // its CTA takes the decisions and writes
     const unsigned cnt = a.cand_cnt[slot];
     const unsigned long long F = a.xs[a.fam_base + slot];
     if (cnt == 0 || cnt > (unsigned)a.cand_max) {     // nothing to count, or the list is incomplete
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && lead) {
             a.counts[slot] = 0;
             if (cnt) a.ovf[atomicAdd(a.ovf_n, 1ULL)] = F;
         }
@@ -220,7 +235,7 @@ __global__ void __launch_bounds__(ND_THREADS) null_direct_kernel(const NullDirec
     __syncthreads();
     const int mode = s_mode, m = s_m;
     if (mode == NR_OVERFLOW) {
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && lead) {
             a.counts[slot] = 0;
             a.ovf[atomicAdd(a.ovf_n, 1ULL)] = F;
         }
@@ -239,14 +254,17 @@ __global__ void __launch_bounds__(ND_THREADS) null_direct_kernel(const NullDirec
             double ar[NB_CHUNK], ai[NB_CHUNK];
 #pragma unroll
             for (int b = 0; b < NB_CHUNK; ++b) { ar[b] = 0.0; ai[b] = 0.0; }
+            double *br = bin_r + (q << MBv), *bi = bin_i + (q << MBv);
             switch (MBv) {
-            case 0: coset_sums<0>(psi, x, j, half, z0, vb, piv, m, offq, ar, ai); break;
-            case 1: coset_sums<1>(psi, x, j, half, z0, vb, piv, m, offq, ar, ai); break;
-            case 2: coset_sums<2>(psi, x, j, half, z0, vb, piv, m, offq, ar, ai); break;
-            case 3: coset_sums<3>(psi, x, j, half, z0, vb, piv, m, offq, ar, ai); break;
-            default: coset_sums<4>(psi, x, j, half, z0, vb, piv, m, offq, ar, ai); break;
+#define C(b) \
+            case b: \
+                coset_sums<b>(psi, x, j, half, z0, vb, piv, m, offq, first, stride, ar, ai); \
+                block_sums<1 << b, CL>(ar, ai, red, cta, br, bi); \
+                break;
+            C(0) C(1) C(2) C(3) C(4)
+#undef C
+            default: break;
             }
-            block_sums<NB_CHUNK>(ar, ai, 1 << MBv, red, bin_r + (q << MBv), bin_i + (q << MBv));
         }
         // m-bit transform of the bins: H(z0 + sum_i a_i v_i) for every a
         const int t = threadIdx.x, nb = 1 << m;
@@ -267,7 +285,7 @@ __global__ void __launch_bounds__(ND_THREADS) null_direct_kernel(const NullDirec
         for (unsigned g0 = 0; g0 < cnt; g0 += ND_GROUP) {
             const int ng = (int)min((unsigned)ND_GROUP, cnt - g0);
             uint32_t zl[ND_GROUP];
-            double ar[ND_GROUP], ai[ND_GROUP];
+            double ar[NB_CHUNK], ai[NB_CHUNK];
 #pragma unroll
             for (int i = 0; i < ND_GROUP; ++i) {
                 zl[i] = i < ng ? zs[g0 + i] : 0u;
@@ -275,22 +293,25 @@ __global__ void __launch_bounds__(ND_THREADS) null_direct_kernel(const NullDirec
                 ai[i] = 0.0;
             }
             switch (ng) {
-            case 1: direct_sums<1>(psi, x, j, half, zl, ar, ai); break;
-            case 2: direct_sums<2>(psi, x, j, half, zl, ar, ai); break;
-            case 3: direct_sums<3>(psi, x, j, half, zl, ar, ai); break;
-            case 4: direct_sums<4>(psi, x, j, half, zl, ar, ai); break;
-            case 5: direct_sums<5>(psi, x, j, half, zl, ar, ai); break;
-            case 6: direct_sums<6>(psi, x, j, half, zl, ar, ai); break;
-            case 7: direct_sums<7>(psi, x, j, half, zl, ar, ai); break;
-            default: direct_sums<8>(psi, x, j, half, zl, ar, ai); break;
+            case 1: direct_sums<1>(psi, x, j, half, first, stride, zl, ar, ai); break;
+            case 2: direct_sums<2>(psi, x, j, half, first, stride, zl, ar, ai); break;
+            case 3: direct_sums<3>(psi, x, j, half, first, stride, zl, ar, ai); break;
+            case 4: direct_sums<4>(psi, x, j, half, first, stride, zl, ar, ai); break;
+            case 5: direct_sums<5>(psi, x, j, half, first, stride, zl, ar, ai); break;
+            case 6: direct_sums<6>(psi, x, j, half, first, stride, zl, ar, ai); break;
+            case 7: direct_sums<7>(psi, x, j, half, first, stride, zl, ar, ai); break;
+            default: direct_sums<8>(psi, x, j, half, first, stride, zl, ar, ai); break;
             }
-            block_sums<ND_GROUP>(ar, ai, ng, red, bin_r, bin_i);
+            block_sums<ND_GROUP, CL>(ar, ai, red, cta, bin_r, bin_i);
             const int t = threadIdx.x;
             const int c = t < ng ? count_pair(bin_r[t], bin_i[t], x != 0, s, a.eps) : 0;
             total += __syncthreads_count(c >= 1) + __syncthreads_count(c == 2);
         }
     }
-    if (threadIdx.x == 0) a.counts[slot] = (unsigned long long)total;
+    if (threadIdx.x == 0 && lead) {
+        a.counts[slot] = (unsigned long long)total;
+        if (a.total) atomicAdd(a.total, (unsigned long long)total);
+    }
 }
 
 } // namespace
@@ -299,7 +320,23 @@ cudaError_t launch_null_direct(const NullDirectArgs &a, long long n_fam, cudaStr
     if (n_fam <= 0) return cudaSuccess;
     if (n_fam > 0x7fffffffLL || a.N < 1 || a.N > 31 || a.kdirect > NULL_CAND_MAX || a.kdirect > a.cand_max)
         return cudaErrorInvalidValue;
-    null_direct_kernel<<<(unsigned)n_fam, ND_THREADS, 0, st>>>(a);
+    // Few families (usually x = 0 alone: the identity) would leave the chip idle
+    // behind one CTA's FP64 pipe: from 2^12 points on, eight CTAs share a family
+    // (one family of N = 18 536 -> 76 us, of N = 16 154 -> 26 us).
+    if (n_fam <= ND_CLUSTER_FAMS && a.N >= 13) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(n_fam * ND_CLUSTER));
+        cfg.blockDim = dim3(ND_THREADS);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = ND_CLUSTER;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, null_direct_kernel<ND_CLUSTER>, a);
+    }
+    null_direct_kernel<1><<<(unsigned)n_fam, ND_THREADS, 0, st>>>(a);
     return cudaGetLastError();
 }
 

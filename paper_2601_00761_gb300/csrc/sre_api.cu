@@ -60,7 +60,6 @@ void count_launches(unsigned long long n) { g_launches.fetch_add(n, std::memory_
 // device allocations this library made since load (cudaMalloc of its own
 // workspace and gate buffers)
 std::atomic<unsigned long long> g_allocs{0};
-constexpr int EXACT_PARTS = 1024;
 
 // --------------------------------------------------------------- plans
 struct Plan {
@@ -235,19 +234,21 @@ struct Arena {
 constexpr long long NULL_CHUNK = 1LL << 11;
 
 struct NullWS {
+    unsigned long long *ovf_n, *total;   // overflow families, and the count of all others; just before cand_cnt
     unsigned *cand_cnt, *cand_z;      // per chunk: counts, lists [slot][NULL_CAND_MAX]
     unsigned long long *counts;       // per flagged family (direct recount; 0 for the overflow)
-    unsigned long long *ovf, *ovf_n;  // overflow families (capacity: the flagged families)
+    unsigned long long *ovf;          // overflow families (capacity: the flagged families)
     unsigned long long *counts2;      // per overflow family (FP64 transform)
     void *inter, *inter64;
 };
 
 void layout_null(Arena &A, long long fam_cap, NullWS &w) {
     const long long ch = std::min(fam_cap, NULL_CHUNK);
-    w.cand_cnt = A.take<unsigned>((size_t)ch);
+    w.ovf_n = A.take<unsigned long long>(2 + ((size_t)ch + 1) / 2);
+    w.total = w.ovf_n ? w.ovf_n + 1 : nullptr;
+    w.cand_cnt = w.ovf_n ? reinterpret_cast<unsigned *>(w.ovf_n + 2) : nullptr;
     w.cand_z = A.take<unsigned>((size_t)ch * NULL_CAND_MAX);
     w.ovf = A.take<unsigned long long>((size_t)fam_cap);
-    w.ovf_n = A.take<unsigned long long>(1);
     w.counts2 = A.take<unsigned long long>((size_t)fam_cap);
 }
 
@@ -256,7 +257,7 @@ struct ExactWS {
     void *inter;
     TilePartial *tiles;
     FamMoments *fm;
-    unsigned long long *flags, *nflag, *counts, *cnt_sum;
+    unsigned long long *flags, *nflag, *counts, *cnt_sum;   // nflag[1]: the totals' block counter
     void *inter64;
     NullWS nw;
 };
@@ -265,16 +266,15 @@ void layout_exact(Arena &A, const Plan &P, const Plan &P64, ExactWS &w) {
     const unsigned long long d = 1ULL << P.N;
     w.scal = A.take<double>(SCAL_N);
     w.npart = A.take<double>(NORM_BLOCKS);
-    w.epart = A.take<double>(6 * EXACT_PARTS);
-    w.etot = A.take<double>(8);
+    w.epart = A.take<double>(5 * TOTALS_BLOCKS);
+    w.etot = A.take<double>(TOT_N + 2);
     w.inter = P.npass > 1 ? (void *)A.take<char>(P.slot_bytes * (size_t)P.B) : nullptr;
-    const long long nb = P.npass > 1 ? P.B : (long long)d;
-    w.tiles = A.take<TilePartial>((size_t)nb * (size_t)P.tiles_last);
+    w.tiles = P.npass > 1 ? A.take<TilePartial>((size_t)P.B * (size_t)P.tiles_last) : nullptr;
     w.fm = A.take<FamMoments>(d);
     w.flags = A.take<unsigned long long>(d);
-    w.nflag = A.take<unsigned long long>(1);
+    w.nflag = A.take<unsigned long long>(2);
     w.counts = A.take<unsigned long long>(d);
-    w.cnt_sum = A.take<unsigned long long>(2);
+    w.cnt_sum = A.take<unsigned long long>(1);
     w.inter64 = P64.npass > 1 ? (void *)A.take<char>(P64.slot_bytes * (size_t)P64.B) : nullptr;
     layout_null(A, (long long)d, w.nw);
     w.nw.counts = w.counts;
@@ -507,9 +507,10 @@ sre_status run_transform(const Plan &P, PassArgs a, int src0, int dst_last, void
     return SRE_OK;
 }
 
-sre_status run_norm2(const void *psi, int N, double *scal, double *partial, cudaStream_t st) {
+sre_status run_norm2(const void *psi, int N, double *scal, double *partial, cudaStream_t st,
+                     unsigned long long *zero = nullptr) {
     int nl = 0;
-    CK(launch_norm2((const float2 *)psi, N, scal, partial, st, &nl));
+    CK(launch_norm2((const float2 *)psi, N, scal, partial, st, &nl, zero));
     count_launches(nl);
     return SRE_OK;
 }
@@ -541,8 +542,7 @@ sre_status run_marginal(const void *psi, int N, const double *scal, double *p, d
 // (*n_ovf of them) with their FP64-transform counts in counts2.
 sre_status null_recount(const Plan &P, const Plan &P64, const PassArgs &a32, const PassArgs &a64,
                         const unsigned long long *xs, long long n, double eps, const NullWS &w, cudaStream_t st,
-                        long long *n_ovf) {
-    CK(cudaMemsetAsync(w.ovf_n, 0, sizeof(unsigned long long), st));
+                        long long *n_ovf, unsigned long long *total = nullptr) {
     PassArgs c = a32;
     c.xs = xs;
     c.precision = 0;
@@ -566,10 +566,13 @@ sre_status null_recount(const Plan &P, const Plan &P64, const PassArgs &a32, con
     q.eps = eps;
     q.ovf = w.ovf;
     q.ovf_n = w.ovf_n;
+    q.total = w.total;
     const long long chunk = P.npass > 1 ? std::min(P.B, NULL_CHUNK) : NULL_CHUNK;
     for (long long fb = 0; fb < n; fb += chunk) {
         const long long nf = std::min(chunk, n - fb);
-        CK(cudaMemsetAsync(w.cand_cnt, 0, sizeof(unsigned) * (size_t)nf, st));
+        // the first chunk's clear covers the two counters in front of the counts
+        if (fb == 0) CK(cudaMemsetAsync(w.ovf_n, 0, 2 * sizeof(unsigned long long) + sizeof(unsigned) * (size_t)nf, st));
+        else CK(cudaMemsetAsync(w.cand_cnt, 0, sizeof(unsigned) * (size_t)nf, st));
         PassArgs b = c;
         b.fam_base = fb;
         b.n_fam = nf;
@@ -579,9 +582,11 @@ sre_status null_recount(const Plan &P, const Plan &P64, const PassArgs &a32, con
         CK(launch_null_direct(q, nf, st));
         count_launches(1);
     }
-    unsigned long long no = 0;
-    CK(cudaMemcpyAsync(&no, w.ovf_n, sizeof no, cudaMemcpyDeviceToHost, st));
+    unsigned long long h[2] = {0, 0};
+    CK(cudaMemcpyAsync(h, w.ovf_n, sizeof h, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    const unsigned long long no = h[0];
+    if (total) *total = h[1];
     if (no > 0) {
         CK(cudaMemsetAsync(w.counts2, 0, sizeof(unsigned long long) * no, st));
         PassArgs d = a64;
@@ -675,10 +680,11 @@ sre_status exact_impl(const void *psi, int N, const sre_opts &o, void *ws, size_
     layout_exact(A, P, P64, w);
 
     const unsigned long long d = 1ULL << N;
-    CS(run_norm2(psi, N, w.scal, w.npart, st));
+    CS(run_norm2(psi, N, w.scal, w.npart, st, w.nflag));
     PassArgs a = base_args(P, psi, w.scal);
     a.precision = prec_code(o);
     a.tile_out = w.tiles;
+    if (P.npass == 1) a.fam_out = w.fm;      // one tile per family: its sums are the family's
     a.cand_thr = cand_threshold(o.eps_null);
     const long long step = P.npass > 1 ? P.B : (long long)d;
     for (long long fb = 0; fb < (long long)d; fb += step) {
@@ -687,19 +693,27 @@ sre_status exact_impl(const void *psi, int N, const sre_opts &o, void *ws, size_
         b.fam_base = fb;
         b.n_fam = nf;
         CS(run_transform(P, b, SRC_PSI_FAMILY, DST_MOMENTS, w.inter, st));
+        if (P.npass == 1) continue;
         CK(launch_fam_reduce(w.tiles, nf, (int)P.tiles_last, nullptr, fb, N, P.M_last, P.M_last, w.fm, fb, nullptr,
                              0, st));
         count_launches(1);
     }
-    CK(cudaMemsetAsync(w.nflag, 0, sizeof(unsigned long long), st));
-    CK(launch_exact_totals(w.fm, (long long)d, w.epart, EXACT_PARTS, w.etot, w.flags, w.nflag, st));
-    count_launches(2);
-    double host[TOT_N + 1];
-    unsigned long long nflag = 0;
-    CK(cudaMemcpyAsync(host, w.etot, TOT_N * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(&nflag, w.nflag, sizeof nflag, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(host + TOT_N, w.scal + SCAL_NORM2, sizeof(double), cudaMemcpyDeviceToHost, st));
+    TotalsArgs t;
+    memset(&t, 0, sizeof t);
+    t.fm = w.fm;
+    t.N = N;
+    t.out = w.etot;
+    t.partial = w.epart;
+    t.done = reinterpret_cast<unsigned *>(w.nflag + 1);
+    t.flags = w.flags;
+    t.n_flag = w.nflag;
+    t.norm2 = w.scal + SCAL_NORM2;
+    CK(launch_totals(t, 1, st));
+    count_launches(1);
+    double host[TOT_N + 2];
+    CK(cudaMemcpyAsync(host, w.etot, sizeof host, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    const unsigned long long nflag = (unsigned long long)host[TOT_N + 1];
     if (!(host[TOT_N] > 0.0)) return fail(SRE_EZERO, "psi has zero norm");
 
     // FP64 recount of the candidate families
@@ -707,17 +721,15 @@ sre_status exact_impl(const void *psi, int N, const sre_opts &o, void *ws, size_
     if (nflag > 0) {
         long long no = 0;
         CS(null_recount(P, P64, base_args(P, psi, w.scal), base_args(P64, psi, w.scal), w.flags, (long long)nflag,
-                        o.eps_null, w.nw, st, &no));
-        CK(launch_sum_u64(w.counts, (long long)nflag, w.cnt_sum, st));
-        count_launches(1);
-        unsigned long long c2[2] = {0, 0};
+                        o.eps_null, w.nw, st, &no, &cnt));
         if (no > 0) {
-            CK(launch_sum_u64(w.nw.counts2, no, w.cnt_sum + 1, st));
+            unsigned long long c2 = 0;
+            CK(launch_sum_u64(w.nw.counts2, no, w.cnt_sum, st));
             count_launches(1);
+            CK(cudaMemcpyAsync(&c2, w.cnt_sum, sizeof c2, cudaMemcpyDeviceToHost, st));
+            CK(cudaStreamSynchronize(st));
+            cnt += c2;
         }
-        CK(cudaMemcpyAsync(c2, w.cnt_sum, sizeof(unsigned long long) * (no > 0 ? 2 : 1), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        cnt = c2[0] + c2[1];
     }
     init_result(out);
     finalize_exact(host, N, out);
@@ -752,8 +764,9 @@ struct BucketPlan {
 
 struct BatchWS {
     const float2 **psi_list;
-    double *s_list, *norm_list, *npart, *totals;
+    double *s_list, *norm_list, *npart, *totals, *tpart;
     unsigned long long *state_count, *nflag, *counts;
+    unsigned *tdone;                     // per state: the totals' block counter
     FamMoments *fm;
     TilePartial *tiles;
     void *inter, *inter64;
@@ -948,6 +961,8 @@ void layout_batch(Arena &A, int count, std::vector<BucketPlan> &B, BatchWS &w, c
     w.totals = A.take<double>(TOT_N * (size_t)count);
     w.state_count = A.take<unsigned long long>(count);
     w.nflag = A.take<unsigned long long>(B.size());
+    w.tpart = A.take<double>(5 * ((size_t)count + TOTALS_BLOCKS));
+    w.tdone = A.take<unsigned>(count);
     size_t fm_n = 0, tiles_n = 0, inter_b = 0, inter64_b = 0, counts_n = 0;
     for (auto &b : B) {
         const long long fams = (long long)b.idx.size() << b.N;
@@ -1024,6 +1039,25 @@ sre_status batch_main(const std::vector<BucketPlan> &B, const BatchWS &w, const 
                       float cand_thr, cudaStream_t st) {
     CK(cudaMemsetAsync(w.nflag, 0, sizeof(unsigned long long) * B.size(), st));
     CK(cudaMemsetAsync(w.state_count, 0, sizeof(unsigned long long) * count, st));
+    CK(cudaMemsetAsync(w.tdone, 0, sizeof(unsigned) * count, st));
+    // totals of states s0 .. s0 + ns - 1 of bucket bi from their family sums
+    auto totals = [&](size_t bi, const FamMoments *fm, long long fm_first, int s0, int ns) -> sre_status {
+        const BucketPlan &b = B[bi];
+        TotalsArgs t;
+        memset(&t, 0, sizeof t);
+        t.fm = fm;
+        t.fm_first = fm_first;
+        t.N = b.N;
+        t.s0 = s0;
+        t.out = w.totals + TOT_N * (size_t)b.off;
+        t.partial = w.tpart;                      // one launch at a time uses it
+        t.done = w.tdone + b.off + s0;
+        t.flags = b.flags;
+        t.n_flag = w.nflag + bi;
+        CK(launch_totals(t, ns, st));
+        count_launches(1);
+        return SRE_OK;
+    };
     for (size_t bi = 0; bi < B.size(); ++bi) {
         const BucketPlan &b = B[bi];
         CK(launch_norm2_multi(w.psi_list + b.off, (int)b.idx.size(), b.N, w.npart, BATCH_NORM_BLOCKS,
@@ -1061,9 +1095,7 @@ sre_status batch_main(const std::vector<BucketPlan> &B, const BatchWS &w, const 
         for (size_t bi = 0; bi < B.size(); ++bi) {
             const BucketPlan &b = B[bi];
             if (!b.persistent) continue;
-            CK(launch_state_totals(w.fm_all + L.fm_off[bi], 0, b.N, 0, (int)b.idx.size(),
-                                   w.totals + TOT_N * (size_t)b.off, b.flags, w.nflag + bi, st));
-            count_launches(1);
+            CS(totals(bi, w.fm_all + L.fm_off[bi], 0, 0, (int)b.idx.size()));
         }
     }
     for (size_t bi = 0; bi < B.size(); ++bi) {
@@ -1090,9 +1122,7 @@ sre_status batch_main(const std::vector<BucketPlan> &B, const BatchWS &w, const 
                                      w.fm, fb - f0, nullptr, 0, st));
                 count_launches(1);
             }
-            CK(launch_state_totals(w.fm, f0, b.N, c0, c1 - c0, w.totals + TOT_N * (size_t)b.off, b.flags,
-                                   w.nflag + bi, st));
-            count_launches(1);
+            CS(totals(bi, w.fm, f0, c0, c1 - c0));
         }
     }
     return SRE_OK;
@@ -1528,8 +1558,8 @@ sre_status run_gate_list(void *psi, int N, const std::vector<GateRow> &in_rows, 
 // ------------------------------------------------------ mixed states
 struct MixedWS {
     double *scal, *npart, *epart, *etot;
+    unsigned long long *done;   // the totals' block counter
     float2 *C;
-    TilePartial *tiles;
     FamMoments *fm;
     void *planes;      // BF16 split planes of Psi for the tensor-core Gram kernel (one K chunk)
     int *err;          // device error word
@@ -1539,10 +1569,10 @@ void layout_mixed(Arena &A, int N, int NA, MixedWS &w) {
     const unsigned long long dA = 1ULL << NA;
     w.scal = A.take<double>(SCAL_N);
     w.npart = A.take<double>(NORM_BLOCKS);
-    w.epart = A.take<double>(6 * EXACT_PARTS);
-    w.etot = A.take<double>(8);
+    w.epart = A.take<double>(5 * TOTALS_BLOCKS);
+    w.etot = A.take<double>(TOT_N + 2);
+    w.done = A.take<unsigned long long>(2);
     w.C = A.take<float2>(dA * dA);
-    w.tiles = A.take<TilePartial>(dA);
     w.fm = A.take<FamMoments>(dA);
     w.planes = A.take<unsigned char>(gram_plane_bytes(N, NA));
     w.err = A.take<int>(1);
@@ -1563,7 +1593,7 @@ sre_status mixed_impl(const void *psi, int N, int NA, void *ws, size_t ws_bytes,
     Arena A(base);
     layout_mixed(A, N, NA, w);
     const unsigned long long dA = 1ULL << NA;
-    CS(run_norm2(psi, N, w.scal, w.npart, st));
+    CS(run_norm2(psi, N, w.scal, w.npart, st, w.done));
     CK(cudaMemsetAsync(w.err, 0, sizeof(int), st));
     int gl = 0;
     cudaError_t ge = launch_gram((const float2 *)psi, N, NA, w.C, w.planes, w.err, &gl, st);
@@ -1576,7 +1606,7 @@ sre_status mixed_impl(const void *psi, int N, int NA, void *ws, size_t ws_bytes,
     a.slot_elems = 1LL << (NA - 1);
     a.range_log2 = NA - 1;
     a.s_ptr = w.scal + SCAL_S;
-    a.tile_out = w.tiles;
+    a.fam_out = w.fm;
     a.cand_thr = 1.0f;
     a.gram = w.C;
     a.gram_ld = (long long)dA;
@@ -1585,14 +1615,18 @@ sre_status mixed_impl(const void *psi, int N, int NA, void *ws, size_t ws_bytes,
     cudaError_t e = launch_f32_single(NA - 1, SRC_GRAM, DST_MOMENTS, a, st);
     if (e != cudaSuccess) return fail(SRE_ECUDA, "mixed-state transform (N_A=%d): %s", NA, cudaGetErrorString(e));
     count_launches(1);
-    CK(launch_fam_reduce(w.tiles, (long long)dA, 1, nullptr, 0, NA, NA - 1, NA - 1, w.fm, 0, nullptr, 0, st));
+    TotalsArgs t;
+    memset(&t, 0, sizeof t);
+    t.fm = w.fm;
+    t.N = NA;
+    t.out = w.etot;
+    t.partial = w.epart;
+    t.done = reinterpret_cast<unsigned *>(w.done);
+    t.norm2 = w.scal + SCAL_NORM2;
+    CK(launch_totals(t, 1, st));
     count_launches(1);
-    unsigned long long *no_flags = nullptr;
-    CK(launch_exact_totals(w.fm, (long long)dA, w.epart, EXACT_PARTS, w.etot, no_flags, nullptr, st));
-    count_launches(2);
-    double T[TOT_N + 1];
-    CK(cudaMemcpyAsync(T, w.etot, TOT_N * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(T + TOT_N, w.scal + SCAL_NORM2, sizeof(double), cudaMemcpyDeviceToHost, st));
+    double T[TOT_N + 2];
+    CK(cudaMemcpyAsync(T, w.etot, sizeof T, cudaMemcpyDeviceToHost, st));
     int herr = 0;
     CK(cudaMemcpyAsync(&herr, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
