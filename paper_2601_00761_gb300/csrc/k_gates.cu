@@ -16,14 +16,14 @@
 // per gate, as an in-place update of the shared tile takes, bound the kernel
 // before: 1000 random Clifford + T gates at N = 26 took 31 ms in 32 blocks, now
 // 17 ms (2.3 rounds a block; instruction issue bounds it, DRAM would take 5 ms);
-// 552 two-qubit gates at N = 24 10.9 ms in 29 blocks, now 8.9 ms (4.3 rounds a
+// 552 two-qubit gates at N = 24 10.9 ms in 29 blocks, now 8.2 ms (4.3 rounds a
 // block; 4.0 ms at the full FP32 rate).
 #include "k_misc.cuh"
 
 namespace sre {
 
 struct GateBlockParams {
-    int Q;                       // qubits in the block
+    int Q;                       // qubits in the block (GATE_BLOCK_Q in the rounds kernel)
     int n_other;                 // qubits outside the block
     unsigned char local[GATE_BLOCK_Q];   // global qubit of local bit i (ascending)
     unsigned char other[32];             // global qubit of tile bit i (ascending)
@@ -133,28 +133,24 @@ __global__ void __launch_bounds__(GT, 2) gate_block_kernel(float2 *psi, const Ga
     if (tile >= (1ULL << p.n_other)) return;   // uniform over the CTA
     unsigned long long base = 0;
     for (int i = 0; i < p.n_other; ++i) base |= ((tile >> i) & 1ULL) << p.other[i];
-    const int L = 1 << p.Q;
     // local bits 0..LOW-1 are global bits 0..LOW-1 (contiguous runs); the
     // global offset of the remaining local bits h = l >> LOW, one table entry
     // per value of h
-    const int low = p.Q < GATE_BLOCK_LOW ? p.Q : GATE_BLOCK_LOW;
-    const int nh = 1 << (p.Q - low);
-    for (int h = threadIdx.x; h < nh; h += GT) {
+    static_assert(GT == 1 << (GATE_BLOCK_Q - GATE_BLOCK_LOW), "one entry per thread");
+    {
         unsigned long long o = base;
-        for (int i = low; i < p.Q; ++i) o |= (unsigned long long)((h >> (i - low)) & 1) << p.local[i];
-        hioff[h] = o;
+#pragma unroll
+        for (int i = GATE_BLOCK_LOW; i < GATE_BLOCK_Q; ++i)
+            o |= (unsigned long long)((threadIdx.x >> (i - GATE_BLOCK_LOW)) & 1) << p.local[i];
+        hioff[threadIdx.x] = o;
     }
-    // a state of fewer than five qubits fills the first entries of one thread's 32
-    const int qt = p.Q < GATE_ROUND_SLOTS ? GATE_ROUND_SLOTS : p.Q;
     // the block's two-qubit matrices, once per CTA (read back as broadcasts)
-    float2 *msm = amp + (1 << qt);
+    float2 *msm = amp + (1 << GATE_BLOCK_Q);
     if constexpr (U2)
         for (int e = threadIdx.x; e < 16 * p.ng; e += GT) msm[e] = __ldg(mats + 16 * (size_t)p.g0 + e);
     __syncthreads();
-    const int lm = (1 << low) - 1;
     constexpr int LOWM = (1 << GATE_BLOCK_LOW) - 1;
-    const bool full = p.Q == GATE_BLOCK_Q;
-    if (full) {
+    {
         // all loads of a thread in flight; thread t takes the indices t + 256 i
         float2 q[GE];
         const float2 *src = psi + (threadIdx.x & LOWM);
@@ -163,24 +159,22 @@ __global__ void __launch_bounds__(GT, 2) gate_block_kernel(float2 *psi, const Ga
         const uint32_t at = gphys(threadIdx.x);
 #pragma unroll
         for (int i = 0; i < GE; ++i) amp[at ^ gphys(GT * i)] = q[i];
-    } else {
-        for (int l = threadIdx.x; l < (1 << qt); l += GT)
-            amp[gphys((uint32_t)l)] = l < L ? psi[hioff[l >> low] | (unsigned long long)(l & lm)] : make_float2(0.f, 0.f);
     }
     const uint32_t t = threadIdx.x;
-    const bool mine = t < (1u << (qt - GATE_ROUND_SLOTS));
+    static_assert(GT == 1 << (GATE_BLOCK_Q - GATE_ROUND_SLOTS), "a thread per coset of the slots");
     float2 v[GE];
     for (int ri = 0; ri < p.nr; ++ri) {
         const GateRound R = rounds[p.r0 + ri];
         __syncthreads();
         // amplitude k of thread t: byte address at ^ ok (positions are linear over GF(2))
         uint32_t at = 0, so[GATE_ROUND_SLOTS];
-        for (int i = 0; i < qt - GATE_ROUND_SLOTS; ++i) at |= ((t >> i) & 1u) << R.thr[i];
+#pragma unroll
+        for (int i = 0; i < GATE_BLOCK_Q - GATE_ROUND_SLOTS; ++i) at |= ((t >> i) & 1u) << R.thr[i];
         at = gphys(at) * (uint32_t)sizeof(float2);
 #pragma unroll
         for (int i = 0; i < GATE_ROUND_SLOTS; ++i) so[i] = gphys(1u << R.slot[i]) * (uint32_t)sizeof(float2);
         char *sm = reinterpret_cast<char *>(amp);
-        if (mine) {
+        {
             // the 32 positions in Gray-code order, one exclusive or each
 #pragma unroll
             for (int i = 0; i < GE; ++i) {
@@ -244,31 +238,120 @@ __global__ void __launch_bounds__(GT, 2) gate_block_kernel(float2 *psi, const Ga
         }
     }
     __syncthreads();
-    if (full) {
-        float2 *dst = psi + (threadIdx.x & LOWM);
-        const uint32_t at = gphys(threadIdx.x);
+    float2 *dst = psi + (threadIdx.x & LOWM);
+    const uint32_t at = gphys(threadIdx.x);
 #pragma unroll
-        for (int i = 0; i < GE; ++i)
-            dst[hioff[(threadIdx.x >> GATE_BLOCK_LOW) + (GT >> GATE_BLOCK_LOW) * i]] = amp[at ^ gphys(GT * i)];
-        return;
-    }
-    for (int l = threadIdx.x; l < L; l += GT)
-        psi[hioff[l >> low] | (unsigned long long)(l & lm)] = amp[gphys((uint32_t)l)];
+    for (int i = 0; i < GE; ++i)
+        dst[hioff[(threadIdx.x >> GATE_BLOCK_LOW) + (GT >> GATE_BLOCK_LOW) * i]] = amp[at ^ gphys(GT * i)];
 }
 
-template <bool U2>
-static cudaError_t launch_blocks(float2 *psi, int N, const GateRow *gates_dev, const GateRound *rounds_dev,
-                                 const float2 *mats_dev, const GateBlock *blocks, int n_blocks, cudaStream_t st) {
+// One barrier per gate, every thread on the pairs of each gate in the shared
+// tile (gates_in_place says for which lists). Rows: opcodes and local qubits.
+__global__ void __launch_bounds__(GT) gate_inplace_kernel(float2 *psi, const GateRow *gates, const float2 *mats,
+                                                          const GateBlockParams p) {
+    extern __shared__ __align__(16) float2 amp[];
+    __shared__ unsigned long long hioff[1 << (GATE_BLOCK_Q - GATE_BLOCK_LOW)];
+    // rows and matrices come through shared memory, GS gates at a time
+    constexpr int GS = 64;
+    __shared__ GateRow srow[GS];
+    __shared__ __align__(16) float2 smat[16 * GS];
+    const unsigned long long tile = blockIdx.x + ((unsigned long long)blockIdx.y << 15);
+    if (tile >= (1ULL << p.n_other)) return;   // uniform over the CTA
+    unsigned long long base = 0;
+    for (int i = 0; i < p.n_other; ++i) base |= ((tile >> i) & 1ULL) << p.other[i];
+    const int L = 1 << p.Q;
+    const int low = p.Q < GATE_BLOCK_LOW ? p.Q : GATE_BLOCK_LOW, lm = (1 << low) - 1;
+    for (int h = threadIdx.x; h < 1 << (p.Q - low); h += GT) {
+        unsigned long long o = base;
+        for (int i = low; i < p.Q; ++i) o |= (unsigned long long)((h >> (i - low)) & 1) << p.local[i];
+        hioff[h] = o;
+    }
+    __syncthreads();
+    for (int l = threadIdx.x; l < L; l += GT) amp[l] = psi[hioff[l >> low] | (unsigned long long)(l & lm)];
+    const float r2 = 0.70710678118654752440f;
+    for (int gi = 0; gi < p.ng; ++gi) {
+        const int ci = gi & (GS - 1);
+        if (ci == 0) {
+            const int nc = p.ng - gi < GS ? p.ng - gi : GS;
+            __syncthreads();
+            for (int e = threadIdx.x; e < nc; e += GT) srow[e] = gates[p.g0 + gi + e];
+            if (mats)
+                for (int e = threadIdx.x; e < 16 * nc; e += GT) smat[e] = __ldg(mats + 16 * (size_t)(p.g0 + gi) + e);
+        }
+        __syncthreads();
+        const GateRow G = srow[ci];
+        const int b0 = 1 << G.q0;
+        if (G.op == GATE_OP_U2) {   // 4x4 matrix, local index bit(q0) + 2 bit(q1)
+            float2 m[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) m[e] = smat[16 * ci + e];
+            const int b1 = 1 << G.q1;
+            const int lo = G.q0 < G.q1 ? G.q0 : G.q1, hi = G.q0 < G.q1 ? G.q1 : G.q0;
+            for (int pi = threadIdx.x; pi < L / 4; pi += GT) {
+                int i = ((pi >> lo) << (lo + 1)) | (pi & ((1 << lo) - 1));
+                i = ((i >> hi) << (hi + 1)) | (i & ((1 << hi) - 1));
+                const int idx[4] = {i, i | b0, i | b1, i | b0 | b1};
+                float2 v[4];
+#pragma unroll
+                for (int l = 0; l < 4; ++l) v[l] = amp[idx[l]];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    float re = 0.f, im = 0.f;
+#pragma unroll
+                    for (int l = 0; l < 4; ++l) {
+                        re = fmaf(m[4 * r + l].x, v[l].x, fmaf(-m[4 * r + l].y, v[l].y, re));
+                        im = fmaf(m[4 * r + l].x, v[l].y, fmaf(m[4 * r + l].y, v[l].x, im));
+                    }
+                    amp[idx[r]] = make_float2(re, im);
+                }
+            }
+        } else if (G.op == 0) {   // H
+            for (int pi = threadIdx.x; pi < L / 2; pi += GT) {
+                const int i = ((pi >> G.q0) << (G.q0 + 1)) | (pi & (b0 - 1));
+                const float2 u = amp[i], w = amp[i | b0];
+                amp[i] = make_float2(r2 * (u.x + w.x), r2 * (u.y + w.y));
+                amp[i | b0] = make_float2(r2 * (u.x - w.x), r2 * (u.y - w.y));
+            }
+        } else if (G.op == 3) {   // CNOT q0 -> q1
+            const int b1 = 1 << G.q1;
+            const int lo = G.q0 < G.q1 ? G.q0 : G.q1, hi = G.q0 < G.q1 ? G.q1 : G.q0;
+            for (int pi = threadIdx.x; pi < L / 4; pi += GT) {
+                int i = ((pi >> lo) << (lo + 1)) | (pi & ((1 << lo) - 1));
+                i = ((i >> hi) << (hi + 1)) | (i & ((1 << hi) - 1));
+                i |= b0;
+                const float2 u = amp[i];
+                amp[i] = amp[i | b1];
+                amp[i | b1] = u;
+            }
+        } else {   // diagonal phase on |1> of q0
+            float cr, ci;
+            phase_of(G.op == 1 ? 2 : G.op == 2 ? 6 : G.op == 4 ? 1 : 7, cr, ci);
+            for (int pi = threadIdx.x; pi < L / 2; pi += GT) {
+                const int i = ((pi >> G.q0) << (G.q0 + 1)) | (pi & (b0 - 1)) | b0;
+                const float2 u = amp[i];
+                amp[i] = make_float2(cr * u.x - ci * u.y, cr * u.y + ci * u.x);
+            }
+        }
+    }
+    __syncthreads();
+    for (int l = threadIdx.x; l < L; l += GT) psi[hioff[l >> low] | (unsigned long long)(l & lm)] = amp[l];
+}
+
+cudaError_t launch_gate_blocks(float2 *psi, int N, const GateRow *gates_dev, const GateRound *rounds_dev,
+                               const float2 *mats_dev, const GateBlock *blocks, int n_blocks, cudaStream_t st) {
     int max_ng = 0;
     for (int b = 0; b < n_blocks; ++b) max_ng = blocks[b].ng > max_ng ? blocks[b].ng : max_ng;
-    const size_t smem_max = (sizeof(float2) << GATE_BLOCK_Q) + (U2 ? sizeof(float2) * 16 * (size_t)max_ng : 0);
+    const size_t tile_max = sizeof(float2) << (N < GATE_BLOCK_Q ? N : GATE_BLOCK_Q);
+    const size_t smem_max = rounds_dev && mats_dev ? tile_max + sizeof(float2) * 16 * (size_t)max_ng : tile_max;
     if (smem_max > 200 * 1024) return cudaErrorInvalidValue;
-    static size_t attr = 0;
-    if (attr < smem_max) {
-        cudaError_t e = cudaFuncSetAttribute(gate_block_kernel<U2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem_max);
+    static size_t attr[3] = {0, 0, 0};
+    const int which = !rounds_dev ? 0 : mats_dev ? 1 : 2;
+    if (attr[which] < smem_max) {
+        const void *k = which == 0 ? (const void *)gate_inplace_kernel
+                      : which == 1 ? (const void *)gate_block_kernel<true> : (const void *)gate_block_kernel<false>;
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
         if (e != cudaSuccess) return e;
-        attr = smem_max;
+        attr[which] = smem_max;
     }
     for (int b = 0; b < n_blocks; ++b) {
         GateBlockParams p;
@@ -288,20 +371,15 @@ static cudaError_t launch_blocks(float2 *psi, int N, const GateRow *gates_dev, c
         for (int q = 0; q < N; ++q)
             if (!in[q]) p.other[p.n_other++] = (unsigned char)q;
         const unsigned long long tiles = 1ULL << p.n_other;
-        dim3 grid((unsigned)(tiles < 32768 ? tiles : 32768), (unsigned)(tiles < 32768 ? 1 : tiles >> 15));
-        const int qt = p.Q < GATE_ROUND_SLOTS ? GATE_ROUND_SLOTS : p.Q;
-        const size_t smem = (sizeof(float2) << qt) + (U2 ? sizeof(float2) * 16 * (size_t)p.ng : 0);
-        gate_block_kernel<U2><<<grid, GT, smem, st>>>(psi, gates_dev, rounds_dev, mats_dev, p);
+        const dim3 grid((unsigned)(tiles < 32768 ? tiles : 32768), (unsigned)(tiles < 32768 ? 1 : tiles >> 15));
+        const size_t tile_bytes = sizeof(float2) << p.Q, mat_bytes = sizeof(float2) * 16 * (size_t)p.ng;
+        if (!rounds_dev) gate_inplace_kernel<<<grid, GT, tile_bytes, st>>>(psi, gates_dev, mats_dev, p);
+        else if (mats_dev) gate_block_kernel<true><<<grid, GT, tile_bytes + mat_bytes, st>>>(psi, gates_dev, rounds_dev, mats_dev, p);
+        else gate_block_kernel<false><<<grid, GT, tile_bytes, st>>>(psi, gates_dev, rounds_dev, nullptr, p);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
-}
-
-cudaError_t launch_gate_blocks(float2 *psi, int N, const GateRow *gates_dev, const GateRound *rounds_dev,
-                               const float2 *mats_dev, const GateBlock *blocks, int n_blocks, cudaStream_t st) {
-    return mats_dev ? launch_blocks<true>(psi, N, gates_dev, rounds_dev, mats_dev, blocks, n_blocks, st)
-                    : launch_blocks<false>(psi, N, gates_dev, rounds_dev, nullptr, blocks, n_blocks, st);
 }
 
 } // namespace sre

@@ -132,6 +132,18 @@ struct GateBlock {
 // control + target); with q1 a thread bit, the phase gate and the CNOT
 // controlled outside the slots. Two-qubit matrices: slots a < b as b (b - 1) / 2 + a.
 enum GateCode { GC_H = 0, GC_PHASE = 5, GC_PHASE_THREAD = 10, GC_CX = 11, GC_CX_THREAD = 36 };
+// Whether a list runs gate by gate in shared memory instead of in register
+// rounds. A state of fewer than 13 qubits would leave most threads of a round
+// idle (32 amplitudes each): a call with 400 random gates at N = 8 takes 109 us in
+// place and 178 in rounds, 24 brick-wall layers at N = 12 174 and 188 us. And a
+// short list of matrices on a few tiles pays for fetching the rounds' unrolled
+// code more than for its barriers: 4 layers (26 to 34 gates) take 72 and 81 us at
+// N = 14, 91 and 100 us at N = 18, but 122 and 103 us at N = 20 (128 tiles); N = 13
+// 88 and 75 us; 2 N layers 362 and 310 us at N = 14.
+inline bool gates_in_place(int N, long long n_gates, bool mats) {
+    return N < GATE_BLOCK_Q || (mats && n_gates <= 40 && N > GATE_BLOCK_Q && N <= 18);
+}
+// A gate list in its blocks; rounds_dev NULL: in place (rows with opcodes and local qubits).
 cudaError_t launch_gate_blocks(float2 *psi, int N, const GateRow *gates_dev, const GateRound *rounds_dev,
                                const float2 *mats_dev, const GateBlock *blocks, int n_blocks, cudaStream_t st);
 

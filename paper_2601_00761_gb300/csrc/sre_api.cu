@@ -1351,10 +1351,9 @@ sre_status autotune_impl(const void *psi, int N, cudaStream_t st, sre_opts *best
 // five slots. A phase gate needs no slot, a CNOT one for its target, H one, a
 // matrix two. src[i] is the caller's index of gate i (its matrix in mats_host).
 // Appends the rows in the order they are applied, the rounds and the matrices.
-void plan_gate_rounds(const std::vector<GateRow> &gates, const std::vector<long long> &src, int m,
-                      const float *mats_host, std::vector<GateRow> &rows, std::vector<GateRound> &rounds,
-                      std::vector<float> &mats) {
-    const int Q = std::max(m, GATE_ROUND_SLOTS);        // fewer qubits leave slots without amplitudes
+void plan_gate_rounds(const std::vector<GateRow> &gates, const std::vector<long long> &src, const float *mats_host,
+                      std::vector<GateRow> &rows, std::vector<GateRound> &rounds, std::vector<float> &mats) {
+    constexpr int Q = GATE_BLOCK_Q;
     auto two = [](const GateRow &G) { return G.op == SRE_GATE_CNOT || G.op == GATE_OP_U2; };
     std::vector<std::vector<int>> qlist(Q);
     for (int g = 0; g < (int)gates.size(); ++g) {
@@ -1449,8 +1448,7 @@ sre_status run_gate_list(void *psi, int N, const std::vector<GateRow> &in_rows, 
                          cudaStream_t st) {
     const long long n_gates = (long long)in_rows.size();
     if (n_gates == 0) return SRE_OK;
-    const int low = N < GATE_BLOCK_LOW ? N : GATE_BLOCK_LOW;
-    const int qmax = N < GATE_BLOCK_Q ? N : GATE_BLOCK_Q;
+    const int low = std::min(N, GATE_BLOCK_LOW), qmax = std::min(N, GATE_BLOCK_Q);
     auto two = [](const GateRow &G) { return G.op == SRE_GATE_CNOT || G.op == GATE_OP_U2; };
     std::vector<std::vector<long long>> qlist(N);
     for (long long g = 0; g < n_gates; ++g) {
@@ -1470,6 +1468,17 @@ sre_status run_gate_list(void *psi, int N, const std::vector<GateRow> &in_rows, 
     rows.reserve(n_gates);
     if (mats_host) mats.reserve(32 * (size_t)n_gates);
     long long ndone = 0;
+    const bool in_place = gates_in_place(N, n_gates, mats_host != nullptr);
+    if (N <= GATE_BLOCK_Q && in_place) {      // one tile holds the state: the list as it is
+        GateBlock B;
+        for (int i = 0; i < GATE_BLOCK_Q; ++i) B.qubit[i] = i < N ? (unsigned char)i : 255;
+        B.r0 = B.nr = B.g0 = 0;
+        B.ng = (int)n_gates;
+        blocks.push_back(B);
+        rows = in_rows;
+        if (mats_host) mats.assign(mats_host, mats_host + 32 * (size_t)n_gates);
+        ndone = n_gates;
+    }
     while (ndone < n_gates) {
         bool in[64] = {false};
         int cnt = 0;
@@ -1497,8 +1506,7 @@ sre_status run_gate_list(void *psi, int N, const std::vector<GateRow> &in_rows, 
             blk.push_back(best);
         }
         if (blk.empty()) return fail(SRE_EINVAL, "gate planner made no progress");
-        // full tiles: a thread holds 32 amplitudes, and smaller blocks leave threads idle
-        for (int q = 0; q < N && cnt < qmax; ++q)
+        for (int q = 0; q < N && cnt < qmax && !in_place; ++q)       // the rounds' tiles are full
             if (!in[q]) { in[q] = true; ++cnt; }
         unsigned char loc[64];
         GateBlock B;
@@ -1515,41 +1523,47 @@ sre_status run_gate_list(void *psi, int N, const std::vector<GateRow> &in_rows, 
         B.g0 = (int)rows.size();
         B.ng = (int)blk.size();
         B.r0 = (int)rounds.size();
-        plan_gate_rounds(local, blk, m, mats_host, rows, rounds, mats);
+        if (in_place) {
+            rows.insert(rows.end(), local.begin(), local.end());
+            if (mats_host)
+                for (long long g : blk) mats.insert(mats.end(), mats_host + 32 * g, mats_host + 32 * (g + 1));
+        } else {
+            plan_gate_rounds(local, blk, mats_host, rows, rounds, mats);
+        }
         B.nr = (int)rounds.size() - B.r0;
         blocks.push_back(B);
         ndone += (long long)blk.size();
     }
     int dev = 0;
     CK(cudaGetDevice(&dev));
-    GateRow *dg = nullptr;
-    GateRound *dr = nullptr;
-    float2 *dm = nullptr;
+    // one buffer, one upload: rows, rounds, matrices
+    const size_t rows_bytes = (sizeof(GateRow) * rows.size() + 255) & ~(size_t)255;
+    const size_t rounds_bytes = (sizeof(GateRound) * rounds.size() + 255) & ~(size_t)255;
+    std::vector<unsigned char> up(rows_bytes + rounds_bytes + sizeof(float) * mats.size());
+    memcpy(up.data(), rows.data(), sizeof(GateRow) * rows.size());
+    if (!rounds.empty()) memcpy(up.data() + rows_bytes, rounds.data(), sizeof(GateRound) * rounds.size());
+    if (!mats.empty()) memcpy(up.data() + rows_bytes + rounds_bytes, mats.data(), sizeof(float) * mats.size());
+    char *dev_buf = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_ws_mu);
         if ((int)g_gatebuf.size() <= dev) g_gatebuf.resize(dev + 1);
         DevBuf &b = g_gatebuf[dev];
-        const size_t rows_bytes = (sizeof(GateRow) * (size_t)n_gates + 255) & ~(size_t)255;
-        const size_t rounds_bytes = (sizeof(GateRound) * rounds.size() + 255) & ~(size_t)255;
-        const size_t need = rows_bytes + rounds_bytes + (mats_host ? sizeof(float2) * 16 * (size_t)n_gates : 0);
-        if (b.n < need) {
+        if (b.n < up.size()) {
             if (b.p) CK(cudaFree(b.p));
             b.p = nullptr;
             b.n = 0;
-            cudaError_t e = cudaMalloc(&b.p, need);
+            cudaError_t e = cudaMalloc(&b.p, up.size());
             g_allocs.fetch_add(1, std::memory_order_relaxed);
             if (e != cudaSuccess) return fail(SRE_ENOMEM, "gate buffer: %s", cudaGetErrorString(e));
-            b.n = need;
+            b.n = up.size();
         }
-        dg = (GateRow *)b.p;
-        dr = (GateRound *)((char *)b.p + rows_bytes);
-        if (mats_host) dm = (float2 *)((char *)b.p + rows_bytes + rounds_bytes);
+        dev_buf = (char *)b.p;
     }
-    CK(cudaMemcpyAsync(dg, rows.data(), sizeof(GateRow) * (size_t)n_gates, cudaMemcpyHostToDevice, st));
-    if (mats_host)
-        CK(cudaMemcpyAsync(dm, mats.data(), sizeof(float2) * 16 * (size_t)n_gates, cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(dr, rounds.data(), sizeof(GateRound) * rounds.size(), cudaMemcpyHostToDevice, st));
-    CK(launch_gate_blocks((float2 *)psi, N, dg, dr, dm, blocks.data(), (int)blocks.size(), st));
+    CK(cudaMemcpyAsync(dev_buf, up.data(), up.size(), cudaMemcpyHostToDevice, st));
+    const GateRow *dg = (const GateRow *)dev_buf;
+    const float2 *dm = mats_host ? (const float2 *)(dev_buf + rows_bytes + rounds_bytes) : nullptr;
+    CK(launch_gate_blocks((float2 *)psi, N, dg, in_place ? nullptr : (const GateRound *)(dev_buf + rows_bytes), dm,
+                          blocks.data(), (int)blocks.size(), st));
     count_launches(blocks.size());
     CK(cudaStreamSynchronize(st));
     return SRE_OK;
