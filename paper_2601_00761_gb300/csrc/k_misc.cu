@@ -157,11 +157,51 @@ __global__ void __launch_bounds__(256) fam_reduce_kernel(const TilePartial *tp, 
     }
 }
 
+// The same sums in the same order for families of many tiles, a warp for each of
+// the four values: the chain of a lane's FP64 additions bounds it (2^16 tiles: 2048
+// additions). One warp per family for all values takes 20 us for 128 families of
+// 2^10 tiles (N = 24) and 920 us for 8 of 2^16 (N = 30); this 7 and 240 us.
+__global__ void __launch_bounds__(32) fam_reduce_value_kernel(const TilePartial *tp, int tiles, long long fam_base,
+                                                              FamMoments *fm, long long fm_base,
+                                                              const unsigned long long *perm) {
+    const long long f = blockIdx.y;
+    const int k = blockIdx.x, lane = threadIdx.x;
+    const TilePartial *row = tp + (size_t)f * (size_t)tiles;
+    double v = 0.0;
+    unsigned c = 0;
+    for (int t0 = 0; t0 < tiles; t0 += 8 * 32) {       // tiles is a power of two, at least 256
+        double q[8];
+        unsigned b[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const TilePartial &p = row[t0 + 32 * i + lane];
+            q[i] = p.m[k];
+            b[i] = k == 0 ? p.cand : 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            v += q[i];
+            c |= b[i];
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    c = __reduce_or_sync(0xffffffffu, c);
+    if (lane == 0) {
+        FamMoments &o = fm[perm ? (long long)perm[fam_base + f] : fm_base + f];
+        o.m[k] = v;
+        if (k == 0) o.cand = (unsigned long long)c;
+    }
+}
+
 cudaError_t launch_fam_reduce(const TilePartial *tp, long long n_fam, int tiles, const unsigned long long *xs,
                               long long fam_base, int N, int M_last, int RL, FamMoments *fm, long long fm_base,
                               float *W, long long nr, cudaStream_t st, const unsigned long long *perm) {
-    fam_reduce_kernel<<<(unsigned)((n_fam + 7) / 8), 256, 0, st>>>(tp, n_fam, tiles, xs, fam_base, N, M_last, RL,
-                                                                  fm, fm_base, W, nr, perm);
+    if (!W && tiles >= 256 && n_fam <= 65535)
+        fam_reduce_value_kernel<<<dim3(4, (unsigned)n_fam), 32, 0, st>>>(tp, tiles, fam_base, fm, fm_base, perm);
+    else
+        fam_reduce_kernel<<<(unsigned)((n_fam + 7) / 8), 256, 0, st>>>(tp, n_fam, tiles, xs, fam_base, N, M_last, RL,
+                                                                      fm, fm_base, W, nr, perm);
     return cudaGetLastError();
 }
 
@@ -265,47 +305,65 @@ cudaError_t launch_sum_u64(const unsigned long long *v, long long n, unsigned lo
 }
 
 // ------------------------------------------------------------- CDF scan
-// Inclusive FP64 scan in natural index order, fixed association (chunks of
-// SCAN_CHUNK elements; 256 threads x 16 consecutive elements per chunk).
+// FP64 sums of p over chunks of SCAN_CHUNK elements, in a fixed association.
 __global__ void __launch_bounds__(256) scan_chunk_sums(const double *p, unsigned long long n, double *bsum) {
     __shared__ double red[8];
-    const unsigned long long base = (unsigned long long)blockIdx.x * SCAN_CHUNK + threadIdx.x * 16ULL;
+    const unsigned long long base = (unsigned long long)blockIdx.x * SCAN_CHUNK + threadIdx.x;
     double a = 0.0;
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-        if (base + i < n) a += p[base + i];
-    // fixed-order block total: per-thread partials summed in thread order
-    __shared__ double part[256];
-    part[threadIdx.x] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int t = 0; t < 256; ++t) s += part[t];
-        bsum[blockIdx.x] = s;
-    }
-    (void)red;
+        if (base + 256 * i < n) a += p[base + 256 * i];
+    a = block_sum<256>(a, red);
+    if (threadIdx.x == 0) bsum[blockIdx.x] = a;
 }
 
-__global__ void __launch_bounds__(256) scan_block_offsets(double *bsum, long long nb) {
-    // exclusive prefix of bsum, in place, sequential over fixed segments
-    __shared__ double seg[257];
-    const long long per = (nb + 255) / 256;
-    const long long lo = threadIdx.x * per, hi = lo + per < nb ? lo + per : nb;
-    double s = 0.0;
-    for (long long i = lo; i < hi; ++i) s += bsum[i];
-    seg[threadIdx.x + 1] = s;
+// Exclusive prefix of bsum in place within tiles of SCAN_TILE chunks, and the
+// total: of the only tile in bsum[nb], else of each in tot.
+constexpr long long SCAN_TILE = 8192;
+__global__ void __launch_bounds__(1024) scan_tile_offsets(double *bsum, long long nb, double *tot) {
+    __shared__ double wsum[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long i0 = (long long)blockIdx.x * SCAN_TILE + 8LL * threadIdx.x;
+    double v[8], a = 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        v[k] = i0 + k < nb ? bsum[i0 + k] : 0.0;
+        a += v[k];
+    }
+    double s = a;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += u;
+    }
+    if (lane == 31) wsum[warp] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        seg[0] = 0.0;
-        for (int t = 1; t <= 256; ++t) seg[t] += seg[t - 1];
+    if (warp == 0) {
+        double w = wsum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double u = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += u;
+        }
+        wsum[lane] = w;
     }
     __syncthreads();
-    double run = seg[threadIdx.x];
-    for (long long i = lo; i < hi; ++i) {
-        const double v = bsum[i];
-        bsum[i] = run;
-        run += v;
-    }
+    double run = (warp ? wsum[warp - 1] : 0.0) + (s - a);
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (i0 + k < nb) {
+            bsum[i0 + k] = run;
+            run += v[k];
+        }
+    if (threadIdx.x == 0) (gridDim.x == 1 ? bsum[nb] : tot[blockIdx.x]) = wsum[31];
+}
+// several tiles: add the totals of the tiles before each (at most 32: N = 30)
+__global__ void __launch_bounds__(1024) scan_tile_add(double *bsum, long long nb, const double *tot) {
+    double before = 0.0;
+    for (unsigned g = 0; g < blockIdx.x; ++g) before += tot[g];
+    const long long i0 = (long long)blockIdx.x * SCAN_TILE;
+    for (long long i = i0 + threadIdx.x; i < i0 + SCAN_TILE && i < nb; i += 1024) bsum[i] += before;
+    if (threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) bsum[nb] = before + tot[blockIdx.x];
 }
 
 __global__ void __launch_bounds__(256) scan_chunk_apply(const double *p, unsigned long long n, const double *boff,
@@ -334,11 +392,16 @@ __global__ void __launch_bounds__(256) scan_chunk_apply(const double *p, unsigne
     }
 }
 
-cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, double *bsum, cudaStream_t st) {
-    const long long nb = (long long)((n + SCAN_CHUNK - 1) / SCAN_CHUNK);
+// chunk sums and their prefix; with cdf, the whole inclusive CDF as well
+cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, double *bsum, int *launches,
+                        cudaStream_t st) {
+    const long long nb = (long long)((n + SCAN_CHUNK - 1) / SCAN_CHUNK), tiles = (nb + SCAN_TILE - 1) / SCAN_TILE;
+    double *tot = bsum + nb + 1;
     scan_chunk_sums<<<(unsigned)nb, 256, 0, st>>>(p, n, bsum);
-    scan_block_offsets<<<1, 256, 0, st>>>(bsum, nb);
-    scan_chunk_apply<<<(unsigned)nb, 256, 0, st>>>(p, n, bsum, cdf);
+    scan_tile_offsets<<<(unsigned)tiles, 1024, 0, st>>>(bsum, nb, tot);
+    if (tiles > 1) scan_tile_add<<<(unsigned)tiles, 1024, 0, st>>>(bsum, nb, tot);
+    if (cdf) scan_chunk_apply<<<(unsigned)nb, 256, 0, st>>>(p, n, bsum, cdf);
+    *launches = 2 + (tiles > 1 ? 1 : 0) + (cdf ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -378,6 +441,72 @@ __global__ void draw_x_kernel(const double *cdf, int N, long long n_x, int mode,
     xs[i] = x;
 }
 
+// x draws straight from p and the prefix of its chunk sums, without the CDF: a
+// block per draw finds the chunk by bisection and sums that chunk alone. Family 0
+// is x = 0; the others x ~ p(x | x != 0).
+__global__ void __launch_bounds__(128) draw_x_chunk_kernel(const double *p, const double *boff, int N, long long nb,
+                                                           unsigned long long seed, unsigned long long ctr0,
+                                                           unsigned long long *xs) {
+    __shared__ double wsum[4];
+    __shared__ unsigned first;
+    const long long i = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (i == 0) {
+        if (threadIdx.x == 0) xs[0] = 0ULL;
+        return;
+    }
+    const double c0 = p[0], total = boff[nb];
+    const double t = c0 + mc_uniform(seed, ctr0, (unsigned long long)i, 0ULL) * (total - c0);
+    long long lo = 0, hi = nb - 1;                 // smallest chunk whose end lies above t, else the last
+    while (lo < hi) {
+        const long long mid = (lo + hi) >> 1;
+        if (boff[mid + 1] > t) hi = mid; else lo = mid + 1;
+    }
+    constexpr int PER = (int)SCAN_CHUNK / 128;
+    const unsigned long long base = (unsigned long long)lo * SCAN_CHUNK;
+    const double *q = p + base + (unsigned long long)threadIdx.x * PER;
+    double v[PER], a = 0.0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        v[k] = q[k];
+        a += v[k];
+    }
+    double s = a;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += u;
+    }
+    if (lane == 31) wsum[warp] = s;
+    if (threadIdx.x == 0) first = (unsigned)SCAN_CHUNK;
+    __syncthreads();
+    double run = boff[lo];
+    for (int w = 0; w < warp; ++w) run += wsum[w];
+    run += s - a;
+    unsigned pick = (unsigned)SCAN_CHUNK;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        run += v[k];
+        if (run > t && pick == (unsigned)SCAN_CHUNK) pick = threadIdx.x * PER + k;
+    }
+    if (pick < (unsigned)SCAN_CHUNK) atomicMin(&first, pick);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long x = base + (first < (unsigned)SCAN_CHUNK ? first : (unsigned)SCAN_CHUNK - 1);
+        // rounding left the chunk's end at or below t: its last x of positive p
+        if (first == (unsigned)SCAN_CHUNK)
+            while (x > base && !(p[x] > 0.0)) --x;
+        xs[i] = x ? x : 1ULL;
+    }
+}
+
+cudaError_t launch_draw_x_chunks(const double *p, const double *boff, int N, long long n_x, unsigned long long seed,
+                                 unsigned long long ctr0, unsigned long long *xs, cudaStream_t st) {
+    const long long nb = (long long)((1ULL << N) / SCAN_CHUNK);
+    draw_x_chunk_kernel<<<(unsigned)n_x, 128, 0, st>>>(p, boff, N, nb, seed, ctr0, xs);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_draw_x(const double *cdf, int N, long long n_x, int mode, unsigned long long seed,
                           unsigned long long ctr0, unsigned long long *xs, cudaStream_t st) {
     draw_x_kernel<<<(unsigned)((n_x + 255) / 256), 256, 0, st>>>(cdf, N, n_x, mode, seed, ctr0, xs);
@@ -401,8 +530,6 @@ cudaError_t launch_draw_x(const double *cdf, int N, long long n_x, int mode, uns
 // power of two) are first staged in shared memory by coalesced loads, with
 // one padding word per chunk so the chunk-wise reads are free of bank
 // conflicts.
-constexpr long long ZSEL_STAGE_MAX = 16384;
-template <bool STAGED>
 __global__ void __launch_bounds__(256) zrange_select_kernel(const float *Wf, long long nr, long long n_fam,
                                                             long long fam_base, int z_per_x, unsigned long long seed,
                                                             unsigned long long ctr0, DrawInfo *draws,
@@ -416,15 +543,10 @@ __global__ void __launch_bounds__(256) zrange_select_kernel(const float *Wf, lon
     const unsigned long long fam = perm ? perm[fam_base + f] : (unsigned long long)(fam_base + f);
     const long long per = (nr + 255) / 256;
     const float *wrow = Wf + (size_t)f * nr;
-    const int lp = STAGED ? 31 - __clz((int)per) : 0;
-    if constexpr (STAGED) {
-        for (uint32_t i = threadIdx.x; i < (uint32_t)nr; i += 256) swf[i + (i >> lp)] = wrow[i];
-        __syncthreads();
-    }
-    auto wf = [&](long long i) -> double {
-        if constexpr (STAGED) return (double)swf[(uint32_t)i + ((uint32_t)i >> lp)];
-        else return (double)wrow[i];
-    };
+    const int lp = 31 - __clz((int)per);
+    for (uint32_t i = threadIdx.x; i < (uint32_t)nr; i += 256) swf[i + (i >> lp)] = wrow[i];
+    __syncthreads();
+    auto wf = [&](long long i) -> double { return (double)swf[(uint32_t)i + ((uint32_t)i >> lp)]; };
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long lo = tid * per, hi = lo + per < nr ? lo + per : nr;
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
@@ -505,24 +627,151 @@ __global__ void __launch_bounds__(256) zrange_select_kernel(const float *Wf, lon
     }
 }
 
+// The same selection for rows of more than ZSEL_STAGE_MAX ranges, in two launches
+// that add in the same order: a thread of zrange_select_kernel walked its chunk
+// (4096 ranges at N = 30) through uncached loads, 1.33 ms for 8 families; these
+// take 0.12 + 0.27 ms (chains of dependent FP64 additions).
+// zchunk_sums_kernel: lane (chunk, chain q) adds the ranges 4 i + q of the chunk.
+__global__ void __launch_bounds__(32) zchunk_sums_kernel(const float *Wf, long long nr, double *sums) {
+    const long long per = nr / 256;
+    const int lane = threadIdx.x, q = lane & 3;
+    const long long chunk = 8LL * blockIdx.x + (lane >> 2);
+    const float *w = Wf + (size_t)blockIdx.y * nr + chunk * per + q;
+    double a = 0.0;
+    for (long long i = 0; i < per; i += 64) {          // per is a power of two, at least 128
+        float v[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = w[i + 4 * k];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) a += f2d(v[k]);
+    }
+    // (a0 + a1) + (a2 + a3)
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    a += __shfl_xor_sync(0xffffffffu, a, 2);
+    if (q == 0) sums[256 * (size_t)blockIdx.y + chunk] = a;
+}
+// A block per family and ZSEL_DRAWS draws, a warp per draw: the chunk's ranges
+// arrive 32 at a time and are added one after another.
+constexpr int ZSEL_DRAWS = 4;
+__global__ void __launch_bounds__(32 * ZSEL_DRAWS) zrange_draw_kernel(const float *Wf, long long nr, const double *sums,
+                                                                      long long fam_base, int z_per_x,
+                                                                      unsigned long long seed, unsigned long long ctr0,
+                                                                      DrawInfo *draws, const unsigned long long *perm) {
+    __shared__ double seg[257];
+    const long long f = blockIdx.y;
+    const unsigned long long fam = perm ? perm[fam_base + f] : (unsigned long long)(fam_base + f);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float *wrow = Wf + (size_t)f * nr;
+    const long long per = nr / 256;
+    if (warp == 0) {
+        // the scan of zrange_select_kernel: warps of 32 chunks, then their sums
+        double wv[8], ws = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            double v = sums[256 * (size_t)f + 32 * w + lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const double u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += u;
+            }
+            wv[w] = v;
+            const double last = __shfl_sync(0xffffffffu, v, 31);
+            if (lane == w) ws = last;
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            const double u = __shfl_up_sync(0xffffffffu, ws, o);
+            if (lane >= o) ws += u;
+        }
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const double before = __shfl_sync(0xffffffffu, ws, w > 0 ? w - 1 : 0);
+            seg[1 + 32 * w + lane] = wv[w] + (w > 0 ? before : 0.0);
+        }
+        if (lane == 0) seg[0] = 0.0;
+    }
+    __syncthreads();
+    const int k = blockIdx.x * ZSEL_DRAWS + warp;
+    if (k >= z_per_x) return;
+    const double total = seg[256];
+    const double t = mc_uniform(seed, ctr0, fam, 1ULL + (unsigned long long)k) * total;
+    long long r = -1;
+    double clo = 0.0, chi = 0.0;
+    // walk one chunk from its start; the first range whose end lies above tt,
+    // else (or for tt = infinity) the last one of positive weight
+    auto walk = [&](int chunk, double tt) {
+        const long long c0 = (long long)chunk * per;
+        double run = seg[chunk];
+        float next = wrow[c0 + lane];
+        for (long long b = 0; b < per; b += 32) {
+            const double w = f2d(next);
+            if (b + 32 < per) next = wrow[c0 + b + 32 + lane];
+            // every lane adds all 32 in turn; lane i keeps the sums around its range
+            double before = 0.0, after = 0.0;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const double nrun = run + __shfl_sync(0xffffffffu, w, i);
+                before = i == lane ? run : before;
+                after = i == lane ? nrun : after;
+                run = nrun;
+            }
+            const unsigned hits = __ballot_sync(0xffffffffu, after > tt);
+            const unsigned pos = __ballot_sync(0xffffffffu, w > 0.0);
+            // a hit ends the walk; otherwise remember the last range of positive weight
+            const int pick = hits ? __ffs(hits) - 1 : 31 - __clz(pos);
+            if (pick >= 0) {
+                r = c0 + b + pick;
+                clo = __shfl_sync(0xffffffffu, before, pick);
+                chi = __shfl_sync(0xffffffffu, after, pick);
+            }
+            if (hits) break;
+        }
+    };
+    if (total > t) {
+        int a = 0, b = 255;                            // smallest a with S_{a+1} > t
+        while (a < b) {
+            const int mid = (a + b) >> 1;
+            if (seg[mid + 1] > t) b = mid; else a = mid + 1;
+        }
+        walk(a, t);
+    }
+    if (r < 0)
+        for (int c = 255; c >= 0 && r < 0; --c)
+            if (seg[c + 1] > seg[c]) walk(c, __longlong_as_double(0x7ff0000000000000LL));
+    if (r < 0) { r = 0; clo = 0.0; chi = (double)wrow[0]; }
+    if (lane == 0) {
+        DrawInfo di;
+        di.range = (unsigned long long)r;
+        di.t = t - clo;
+        di.wr = chi - clo;
+        di.pad = 0.0;
+        draws[(size_t)fam * z_per_x + k] = di;
+    }
+}
+
 cudaError_t launch_zrange_select(const float *Wf, long long nr, long long n_fam, long long fam_base, int z_per_x,
                                  unsigned long long seed, unsigned long long ctr0, DrawInfo *draws,
-                                 const unsigned long long *perm, cudaStream_t st) {
-    if (nr <= ZSEL_STAGE_MAX && (nr & (nr - 1)) == 0) {
+                                 const unsigned long long *perm, double *sums, int *launches, cudaStream_t st) {
+    if (nr & (nr - 1)) return cudaErrorInvalidValue;         // 2^(N - RL)
+    if (nr <= ZSEL_STAGE_MAX) {
         const size_t smem = sizeof(float) * (size_t)(nr + 256 + 1);
         static bool attr = false;
         if (!attr) {
-            cudaError_t e = cudaFuncSetAttribute(zrange_select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaError_t e = cudaFuncSetAttribute(zrange_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)(sizeof(float) * (ZSEL_STAGE_MAX + 257)));
             if (e != cudaSuccess) return e;
             attr = true;
         }
-        zrange_select_kernel<true><<<(unsigned)n_fam, 256, smem, st>>>(Wf, nr, n_fam, fam_base, z_per_x, seed, ctr0,
-                                                                       draws, perm);
-    } else {
-        zrange_select_kernel<false><<<(unsigned)n_fam, 256, 0, st>>>(Wf, nr, n_fam, fam_base, z_per_x, seed, ctr0,
-                                                                     draws, perm);
+        zrange_select_kernel<<<(unsigned)n_fam, 256, smem, st>>>(Wf, nr, n_fam, fam_base, z_per_x, seed, ctr0, draws,
+                                                                 perm);
+        *launches = 1;
+        return cudaGetLastError();
     }
+    // at most 128 families a launch here (N >= 25)
+    zchunk_sums_kernel<<<dim3(32, (unsigned)n_fam), 32, 0, st>>>(Wf, nr, sums);
+    zrange_draw_kernel<<<dim3((unsigned)((z_per_x + ZSEL_DRAWS - 1) / ZSEL_DRAWS), (unsigned)n_fam), 32 * ZSEL_DRAWS, 0, st>>>(
+        Wf, nr, sums, fam_base, z_per_x, seed, ctr0, draws, perm);
+    *launches = 2;
     return cudaGetLastError();
 }
 
@@ -531,60 +780,74 @@ cudaError_t launch_zrange_select(const float *Wf, long long nr, long long n_fam,
 // y[i][3..5] = the family's exact conditional means (-sum c^2 log2 c^2,
 // sum c^4, sum c^6) / sum c^2 (marginal mode; family 0, the x = 0 stratum,
 // takes the exact means in both slots), or, uniform mode, the SM Sec. I
-// family values h_x, m_{2;x}, m_{3;x} in y[i][0..2].
-__global__ void mc_family_stats_kernel(const FamMoments *fm, const float *cz, long long n_x, int z_per_x, int N,
-                                       int mode, double *y) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// family values h_x, m_{2;x}, m_{3;x} in y[i][0..2]. A warp per family, lanes over
+// its draws (a thread per family
+// left most SMs idle: N = 24, 4096 families of 256 draws 240 us, now 52 us)
+__global__ void __launch_bounds__(256) mc_family_stats_kernel(const FamMoments *fm, const float *cz, long long n_x,
+                                                              int z_per_x, int N, int mode, double *y) {
+    const int lane = threadIdx.x & 31;
+    const long long i = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (i >= n_x) return;
     const double d = ldexp(1.0, N);
-    const FamMoments &m = fm[i];
+    const FamMoments m = fm[i];
     double *o = y + 6 * i;
     if (mode == 0) {
-        o[0] = N * (m.m[0] / d) - m.m[3] / d;
-        o[1] = m.m[1] / (d * d);
-        o[2] = m.m[2] / (d * d * d);
-        o[3] = o[4] = o[5] = 0.0;
-    } else {
-        double a0 = 0, a1 = 0, a2 = 0;
-        for (int k = 0; k < z_per_x; ++k) {
+        if (lane == 0) {
+            o[0] = N * (m.m[0] / d) - m.m[3] / d;
+            o[1] = m.m[1] / (d * d);
+            o[2] = m.m[2] / (d * d * d);
+            o[3] = o[4] = o[5] = 0.0;
+        }
+        return;
+    }
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    if (i > 0)
+        for (int k = lane; k < z_per_x; k += 32) {
             const double c = (double)cz[(size_t)i * z_per_x + k];
             const double c2 = c * c;
-            a0 += -log2(c2);
-            a1 += c2;
-            a2 += c2 * c2;
+            a[0] += -log2(c2);
+            a[1] += c2;
+            a[2] += c2 * c2;
         }
-        o[3] = -m.m[3] / m.m[0]; o[4] = m.m[1] / m.m[0]; o[5] = m.m[2] / m.m[0];
-        if (i == 0) { o[0] = o[3]; o[1] = o[4]; o[2] = o[5]; }
-        else { o[0] = a0 / z_per_x; o[1] = a1 / z_per_x; o[2] = a2 / z_per_x; }
+    int id;
+    const double t = warp_sums<4>(a, id);                // value v in lanes 8 v .. 8 v + 7
+    if ((lane & 7) == 0 && id < 3) {
+        const double exact = (id == 0 ? -m.m[3] : id == 1 ? m.m[1] : m.m[2]) / m.m[0];
+        o[3 + id] = exact;
+        o[id] = i == 0 ? exact : t / z_per_x;
     }
 }
 
 // out[0..5] = sum_{i >= first} y[i][a], out[6..11] = sum y^2, out[12..17] = y[0][a],
-// out[18] = sum over families of sum c^2 / (d p(x)) estimate (marginal) -- fixed order.
+// out[18] = sum over families of sum c^2 / (d p(x)) estimate (marginal) -- fixed
+// order, one block per value (one block for all: 165 us for 5001 families).
 __global__ void __launch_bounds__(256) mc_totals_kernel(const double *y, long long n_x, int first,
                                                         const FamMoments *fm, double *out) {
     __shared__ double red[8];
-    for (int a = 0; a < 6; ++a) {
-        NeuSum ns, nq;
+    const int a = blockIdx.x;
+    NeuSum ns, nq;
+    if (a < 6) {
         for (long long i = first + threadIdx.x; i < n_x; i += 256) {
             const double v = y[6 * i + a];
             ns.add(v);
             nq.add(v * v);
         }
-        const double s = block_sum<256>(ns.value(), red);
-        const double q = block_sum<256>(nq.value(), red);
-        if (threadIdx.x == 0) { out[a] = s; out[6 + a] = q; out[12 + a] = y[a]; }
+    } else {
+        for (long long i = threadIdx.x; i < n_x; i += 256) ns.add(fm[i].m[0]);
     }
-    NeuSum np_;
-    for (long long i = threadIdx.x; i < n_x; i += 256) np_.add(fm[i].m[0]);
-    const double p = block_sum<256>(np_.value(), red);
-    if (threadIdx.x == 0) out[18] = p;
+    const double s = block_sum<256>(ns.value(), red);
+    if (a == 6) {
+        if (threadIdx.x == 0) out[18] = s;
+        return;
+    }
+    const double q = block_sum<256>(nq.value(), red);
+    if (threadIdx.x == 0) { out[a] = s; out[6 + a] = q; out[12 + a] = y[a]; }
 }
 
 cudaError_t launch_mc_stats(const FamMoments *fm, const float *cz, long long n_x, int z_per_x, int N, int mode,
                             double *y, double *out, cudaStream_t st) {
-    mc_family_stats_kernel<<<(unsigned)((n_x + 127) / 128), 128, 0, st>>>(fm, cz, n_x, z_per_x, N, mode, y);
-    mc_totals_kernel<<<1, 256, 0, st>>>(y, n_x, 1, fm, out);
+    mc_family_stats_kernel<<<(unsigned)((n_x + 7) / 8), 256, 0, st>>>(fm, cz, n_x, z_per_x, N, mode, y);
+    mc_totals_kernel<<<7, 256, 0, st>>>(y, n_x, 1, fm, out);
     return cudaGetLastError();
 }
 

@@ -77,12 +77,21 @@ cudaError_t launch_fam_reduce(const TilePartial *tp, long long n_fam, int tiles,
                               long long fam_base, int N, int M_last, int RL, FamMoments *fm, long long fm_base,
                               float *W, long long nr, cudaStream_t st, const unsigned long long *perm = nullptr);
 cudaError_t launch_sum_u64(const unsigned long long *v, long long n, unsigned long long *out, cudaStream_t st);
-cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, double *bsum, cudaStream_t st);
+// bsum: n / SCAN_CHUNK + SCAN_EXTRA doubles, the exclusive prefix of p's chunk
+// sums and the total; cdf (or NULL): the inclusive CDF of p (may be p itself)
+constexpr long long SCAN_EXTRA = 40;
+cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, double *bsum, int *launches,
+                        cudaStream_t st);
 cudaError_t launch_draw_x(const double *cdf, int N, long long n_x, int mode, unsigned long long seed,
                           unsigned long long ctr0, unsigned long long *xs, cudaStream_t st);
+// marginal draws from p and the prefix of its chunk sums (N >= 12)
+cudaError_t launch_draw_x_chunks(const double *p, const double *boff, int N, long long n_x, unsigned long long seed,
+                                 unsigned long long ctr0, unsigned long long *xs, cudaStream_t st);
+constexpr long long ZSEL_STAGE_MAX = 16384;   // ranges of a row that is staged in shared memory
+// sums: 256 doubles per family of a launch (rows of more ranges than that)
 cudaError_t launch_zrange_select(const float *Wf, long long nr, long long n_fam, long long fam_base, int z_per_x,
                                  unsigned long long seed, unsigned long long ctr0, DrawInfo *draws,
-                                 const unsigned long long *perm, cudaStream_t st);
+                                 const unsigned long long *perm, double *sums, int *launches, cudaStream_t st);
 cudaError_t launch_mc_stats(const FamMoments *fm, const float *cz, long long n_x, int z_per_x, int N, int mode,
                             double *y, double *out, cudaStream_t st);
 cudaError_t launch_norm2_multi(const float2 *const *psi_list, int n_states, int N, double *partial, int nb,

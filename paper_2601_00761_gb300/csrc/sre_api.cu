@@ -294,6 +294,7 @@ struct McWS {
     DrawInfo *draws;
     unsigned long long *zs;
     float *cz;
+    double *zsum;    // chunk sums of the range rows (rows of more than ZSEL_STAGE_MAX ranges)
     double *y, *out;
     int *err;        // device error word (SRE_ERR_* bits)
 };
@@ -305,7 +306,7 @@ void layout_mc(Arena &A, const Plan &P, int mode, long long n_x, int zpx, McWS &
     w.npart = A.take<double>(NORM_BLOCKS);
     w.p = marg ? A.take<double>(d) : nullptr;
     w.mwork = marg ? A.take<double>(d) : nullptr;
-    w.bsum = marg ? A.take<double>(d / SCAN_CHUNK + 1) : nullptr;
+    w.bsum = marg ? A.take<double>(d / SCAN_CHUNK + SCAN_EXTRA) : nullptr;
     w.xs = A.take<unsigned long long>(n_x);
     w.xs_ord = P.npass > 1 ? A.take<unsigned long long>(n_x) : nullptr;
     w.perm = P.npass > 1 ? A.take<unsigned long long>(n_x) : nullptr;
@@ -319,6 +320,7 @@ void layout_mc(Arena &A, const Plan &P, int mode, long long n_x, int zpx, McWS &
     w.draws = marg ? A.take<DrawInfo>(nd) : nullptr;
     w.zs = marg ? A.take<unsigned long long>(nd) : nullptr;
     w.cz = A.take<float>(nd);
+    w.zsum = marg && nr > ZSEL_STAGE_MAX ? A.take<double>(256 * (size_t)B) : nullptr;
     w.y = A.take<double>(6 * (size_t)n_x);
     w.out = A.take<double>(24);
     w.err = A.take<int>(1);
@@ -1829,10 +1831,17 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
     CS(run_norm2(psi, N, w.scal, w.npart, st));
     if (marg) {
         CS(run_marginal(psi, N, w.scal, w.p, w.mwork, st));
-        CK(launch_scan(w.p, d, w.p, w.bsum, st));
-        count_launches(3);
+        // a draw through the chunk sums reads one chunk (20 ns of the chip), the
+        // whole CDF costs 10 ps per x: few draws on a large state skip the CDF
+        const bool chunks = (unsigned long long)n_x <= d / 2048;
+        int nl = 0;
+        CK(launch_scan(w.p, d, chunks ? nullptr : w.p, w.bsum, &nl, st));
+        count_launches(nl);
+        if (chunks) CK(launch_draw_x_chunks(w.p, w.bsum, N, n_x, seed, counter0, w.xs, st));
+        else CK(launch_draw_x(w.p, N, n_x, 1, seed, counter0, w.xs, st));
+    } else {
+        CK(launch_draw_x(nullptr, N, n_x, 0, seed, counter0, w.xs, st));
     }
-    CK(launch_draw_x(w.p, N, n_x, marg ? 1 : 0, seed, counter0, w.xs, st));
     count_launches(1);
     // Multi-pass plans process the families in an order that lets the
     // families of one launch share psi in L2: by the top bit j of x (the same
@@ -1897,8 +1906,9 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
                              (marg && !fine) ? w.Wf : nullptr, nr, st, perm));
         count_launches(1);
         if (marg) {
-            CK(launch_zrange_select(w.Wf, nr, nf, fb, z_per_x, seed, counter0, w.draws, perm, st));
-            count_launches(1);
+            int nl = 0;
+            CK(launch_zrange_select(w.Wf, nr, nf, fb, z_per_x, seed, counter0, w.draws, perm, w.zsum, &nl, st));
+            count_launches(nl);
             PassArgs c = b;
             c.src = w.inter;
             c.lo_g = 0;
@@ -1914,7 +1924,7 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
     int herr = 0;
     CK(cudaMemcpyAsync(&herr, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
     h[21] = 0.0;
-    if (marg) CK(cudaMemcpyAsync(h + 21, w.p, sizeof(double), cudaMemcpyDeviceToHost, st));   // p(0) = CDF(0)
+    if (marg) CK(cudaMemcpyAsync(h + 21, w.p, sizeof(double), cudaMemcpyDeviceToHost, st));   // p(0)
     if (xs_dev) CK(cudaMemcpyAsync(xs_dev, w.xs, n_x * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
     if (marg && zs_dev)
         CK(cudaMemcpyAsync(zs_dev, w.zs, (size_t)n_x * z_per_x * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st));
