@@ -4,6 +4,7 @@
 //   prologue  SRC_PSI_FAMILY : h(b') = conj(psi[b^x]) psi[b], b = b' with 0 at bit j
 //             SRC_PSI_Q      : h(g)  = (|psi[g]|^2, |psi[g + d/2]|^2)  (x = 0 family / marginal)
 //             SRC_BUF        : the previous pass's output
+//             SRC_PSI_TILED  : SRC_PSI_FAMILY from a copy of psi in tile order
 //             SRC_GRAM       : h(a) = C[a][a ^ x] of a reduced state (C = Psi Psi^H)
 //   epilogue  DST_BUF        : store for the next pass
 //             DST_MOMENTS    : fused reduction of Algorithm 1 (sum c^2, c^4, c^6,
@@ -150,7 +151,44 @@ __device__ __forceinline__ void pass_prologue(typename Cfg::C2 (&v)[Cfg::E], con
     constexpr int A0 = Maps<Cfg>::first;
     const uint32_t base = thread_gidx<Cfg>(gbase, a.lo_g, Cfg::elem(t, 0, A0));
     const uint32_t rs = 1u << a.lo_g;
-    if constexpr (SRC == SRC_PSI_FAMILY) {
+    if constexpr (SRC == SRC_PSI_TILED) {
+        static_assert(Cfg::LO == PSI_TILED_COLS, "the tile's columns lie together");
+        if (x == 0 || j >= a.lo_g) {
+            // tile element e is packed amplitude (row, column) = place e of the
+            // tile's run; the row bit j is inserted in the place, and the
+            // partner's place differs by that of x (x = 0: by the top row bit)
+            constexpr int LB = Cfg::E < 8 ? Cfg::E : 8;
+            const uint32_t e0 = Cfg::elem(t, 0, A0);
+            const uint32_t hm = ~((1u << (j - a.lo_g + Cfg::LO)) - 1u);
+            const uint32_t run = psi_tiled_index((uint32_t)gbase & ((1u << a.lo_g) - 1u), a.lo_g, a.N);
+            const uint32_t px = x ? psi_tiled_index((uint32_t)x, a.lo_g, a.N) : 1u << (Cfg::M);
+            const float2 *own = a.psi_tiled;
+#pragma unroll
+            for (int k0 = 0; k0 < Cfg::E; k0 += LB) {
+                float2 u[LB], w[LB];
+#pragma unroll
+                for (int q = 0; q < LB; ++q) {
+                    const uint32_t e = e0 + ((uint32_t)(k0 + q) << A0);
+                    const uint32_t b = run + e + (e & hm);
+                    u[q] = __ldg(own + b);
+                    w[q] = __ldg(own + (b ^ px));
+                }
+#pragma unroll
+                for (int q = 0; q < LB; ++q) {
+                    const R ux = u[q].x, uy = u[q].y, wx = w[q].x, wy = w[q].y;
+                    if (x) {
+                        v[k0 + q].x = fma(wx, ux, wy * uy);
+                        v[k0 + q].y = fma(wx, uy, -(wy * ux));
+                    } else {
+                        v[k0 + q].x = fma(ux, ux, uy * uy);
+                        v[k0 + q].y = fma(wx, wx, wy * wy);
+                    }
+                }
+            }
+            return;
+        }
+    }
+    if constexpr (SRC == SRC_PSI_FAMILY || SRC == SRC_PSI_TILED) {
         // loads issued in batches of LB slots (2 LB independent 8-byte loads in
         // flight per thread) before any of them is used
         constexpr int LB = Cfg::E < 8 ? Cfg::E : 8;
@@ -358,7 +396,7 @@ __host__ __device__ constexpr bool ranges_accumulate(int E) { return (1 << ZR_FI
 #define SRE_STRIDED_FPC 4
 #endif
 template <class Cfg, int SRC> struct FamPerCta {
-    static constexpr int v = (SRC == SRC_PSI_FAMILY && Cfg::G == 1 && Cfg::LO > 0) ? SRE_STRIDED_FPC : 1;
+    static constexpr int v = ((SRC == SRC_PSI_FAMILY || SRC == SRC_PSI_TILED) && Cfg::G == 1 && Cfg::LO > 0) ? SRE_STRIDED_FPC : 1;
 };
 
 // One tile of one family (the rep-th family of the CTA); false when the CTA
@@ -408,7 +446,7 @@ __device__ __forceinline__ void fwht_pass_body(const PassArgs &a, long long slot
     const int n = a.n;
     const unsigned long long dmask = (N >= 64) ? ~0ULL : ((1ULL << N) - 1ULL);
     unsigned long long x = 0, F = 0;
-    if constexpr (SRC == SRC_PSI_FAMILY || DST == DST_MOMENTS || DST == DST_SPECTRUM || DST == DST_NULLCOUNT ||
+    if constexpr (SRC == SRC_PSI_FAMILY || SRC == SRC_PSI_TILED || DST == DST_MOMENTS || DST == DST_SPECTRUM || DST == DST_NULLCOUNT ||
                   DST == DST_CANDLIST) {
         F = a.xs ? a.xs[a.fam_base + slot] : (unsigned long long)(a.fam_base + slot);
         x = F & dmask;
@@ -668,7 +706,7 @@ cudaError_t launch_cfg(const PassArgs &a, int tiles, cudaStream_t st) {
     } else {
         const long long nf = a.n_fam;
         const long long total = nf * (long long)tiles;
-        if ((SRC == SRC_PSI_FAMILY || SRC == SRC_PSI_Q) && nf > 1 && tiles > 1 &&
+        if ((SRC == SRC_PSI_FAMILY || SRC == SRC_PSI_Q || SRC == SRC_PSI_TILED) && nf > 1 && tiles > 1 &&
             total < 0x7fffffffLL) {
             constexpr int FPC = FamPerCta<Cfg, SRC>::v;
             b.fam_fast = 1;

@@ -95,6 +95,8 @@ struct SingleCfgOf {
 
 cudaError_t launch_f32_single(int M, int src, int dst, const PassArgs &a, cudaStream_t st);
 cudaError_t launch_f32_strided(int MS, int K, int src, int dst, const PassArgs &a, int tiles, cudaStream_t st);
+// psi into the order of psi_tiled_index (for a first strided pass from bit lo on)
+cudaError_t launch_psi_tiled(const float2 *psi, float2 *out, int lo, int N, cudaStream_t st);
 cudaError_t launch_f32_row(int M, int src, int dst, const PassArgs &a, int tiles, cudaStream_t st);
 cudaError_t launch_f64_single(int M, int src, int dst, const PassArgs &a, cudaStream_t st);
 cudaError_t launch_f64_strided(int K, int src, int dst, const PassArgs &a, int tiles, cudaStream_t st);
@@ -108,7 +110,7 @@ cudaError_t launch_f64_row(int M, int src, int dst, const PassArgs &a, int tiles
 // psi-reading pass, against tiles of 2^13 points throughout:
 //   K       4     5     6     7     8     9    10
 //   2^13  1.47  1.50  2.08  2.08  2.10  2.08  2.5 ps
-//   here  1.17  1.19  1.25  1.61  1.82  2.08  2.5 ps
+//   here  1.17  1.19  1.25  1.61  1.82  2.08  2.5 ps (2.3 from a copy of psi in tile order)
 // (1.18 ps is the DRAM time of the 8 bytes written; with 8 columns, 64-byte
 // rows, K = 7 takes 2.6 ps). FP64 MS = 13 (128 KB).
 constexpr int F32_STRIDED_KMAX = 10, F32_ROW_MMIN = 10, F32_ROW_MMAX = 14, F32_SINGLE_MMAX = 14;

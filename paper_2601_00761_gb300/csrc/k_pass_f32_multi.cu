@@ -14,6 +14,9 @@ cudaError_t strided6(const PassArgs &a, int tiles, cudaStream_t st) {
 } // namespace
 
 cudaError_t launch_f32_strided(int MS, int K, int src, int dst, const PassArgs &a, int tiles, cudaStream_t st) {
+    if (K == 10 && src == SRC_PSI_FAMILY && dst == DST_BUF && a.precision == 0 && a.psi_tiled && !a.psi_list)
+        return launch_cfg<TileCfg<float, f32_strided_ms(10), PSI_TILED_COLS, f32_strided_rb(10), 1>, SRC_PSI_TILED, DST_BUF, 0>(
+            a, tiles, st);
     if (MS != f32_strided_ms(K)) {
         if (src != SRC_PSI_FAMILY || dst != DST_BUF || MS != f32_strided_ms(K, true)) return cudaErrorInvalidValue;
         switch (K) {
@@ -48,5 +51,37 @@ cudaError_t launch_f32_row(int M, int src, int dst, const PassArgs &a, int tiles
 #undef C
     default: return cudaErrorInvalidValue;
     }
+}
+} // namespace sre
+
+namespace sre {
+namespace {
+// The 10-bit strided pass reads psi in 64-byte rows: a warp's 8-byte loads touch
+// four half-used lines, and the tag stage of L1 bounded the pass (71% busy, loads
+// throttled). From a copy of psi in which a tile's rows are contiguous, every load
+// of a warp is two full lines: N = 24, 128 families per launch 2.79 -> 2.49 ms,
+// 2.6 -> 2.3 ps per point (1.2 ps is the DRAM time of what it writes; its 64-byte
+// stores are what is left); the step of 4096 families 172.7 -> 162.9 ms with the
+// copy. psi in tile order: a thread per amplitude in the order of the copy, so that
+// writes are contiguous and reads are the copy's 64-byte rows
+__global__ void __launch_bounds__(256) psi_tile_kernel(const float2 *psi, float2 *out, int lo, int N) {
+    constexpr int C = PSI_TILED_COLS, PER = 8;
+    const uint32_t p0 = blockIdx.x * (256u * PER) + threadIdx.x;
+    float2 v[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const uint32_t p = p0 + 256u * i;
+        const uint32_t row = (p >> C) & ((1u << (N - lo)) - 1u), cb = p >> (N - lo + C);
+        v[i] = __ldg(psi + ((p & ((1u << C) - 1u)) | (cb << C) | (row << lo)));
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) out[p0 + 256u * i] = v[i];
+}
+} // namespace
+
+cudaError_t launch_psi_tiled(const float2 *psi, float2 *out, int lo, int N, cudaStream_t st) {
+    if (N < 11 || N > 31 || lo <= PSI_TILED_COLS || lo >= N) return cudaErrorInvalidValue;
+    psi_tile_kernel<<<1u << (N - 11), 256, 0, st>>>(psi, out, lo, N);
+    return cudaGetLastError();
 }
 } // namespace sre

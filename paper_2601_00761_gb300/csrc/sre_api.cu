@@ -287,6 +287,7 @@ struct McWS {
     double *p, *mwork, *bsum;
     unsigned long long *xs;
     unsigned long long *xs_ord, *perm;   // the families in processing order, and their own indices
+    float2 *psi_tiled;                   // psi in tile order, or NULL
     void *inter;
     TilePartial *tiles;
     FamMoments *fm;
@@ -299,7 +300,16 @@ struct McWS {
     int *err;        // device error word (SRE_ERR_* bits)
 };
 
-void layout_mc(Arena &A, const Plan &P, int mode, long long n_x, int zpx, McWS &w) {
+// Whether the first strided pass reads a copy of psi in tile order: its rows have
+// 8 columns (10 bits: N = 24, and N = 23 without z draws) and there are families
+// enough to pay for the copy (62 us at N = 24; the pass saves 2.5 us a family).
+constexpr long long PSI_TILED_FAMILIES = 64;
+bool tiled_psi(const Plan &P, const sre_opts &o, long long n_x) {
+    return P.nstrided > 0 && P.K[0] == 10 && P.ms[0] - P.K[0] == PSI_TILED_COLS && o.precision == SRE_FP32_SIMT &&
+           n_x >= PSI_TILED_FAMILIES;
+}
+
+void layout_mc(Arena &A, const Plan &P, int mode, long long n_x, int zpx, bool tiled, McWS &w) {
     const unsigned long long d = 1ULL << P.N;
     const bool marg = mode == SRE_MC_MARGINAL;
     w.scal = A.take<double>(SCAL_N);
@@ -311,6 +321,7 @@ void layout_mc(Arena &A, const Plan &P, int mode, long long n_x, int zpx, McWS &
     w.xs_ord = P.npass > 1 ? A.take<unsigned long long>(n_x) : nullptr;
     w.perm = P.npass > 1 ? A.take<unsigned long long>(n_x) : nullptr;
     const long long B = P.npass > 1 ? P.B : (n_x < P.B ? n_x : P.B);
+    w.psi_tiled = tiled ? A.take<float2>(d) : nullptr;
     w.inter = P.npass > 1 ? (void *)A.take<char>(P.slot_bytes * (size_t)P.B) : nullptr;
     w.tiles = A.take<TilePartial>((size_t)B * (size_t)P.tiles_last);
     w.fm = A.take<FamMoments>(n_x);
@@ -1303,11 +1314,11 @@ sre_status autotune_impl(const void *psi, int N, cudaStream_t st, sre_opts *best
         const long long fams = std::min(d, std::max(P.B * 4, 64LL));
         Arena dry(nullptr);
         McWS w;
-        layout_mc(dry, P, SRE_MC_UNIFORM, fams, 1, w);
+        layout_mc(dry, P, SRE_MC_UNIFORM, fams, 1, false, w);
         void *base = nullptr;
         CS(own_workspace(dry.off, &base));
         Arena A(base);
-        layout_mc(A, P, SRE_MC_UNIFORM, fams, 1, w);
+        layout_mc(A, P, SRE_MC_UNIFORM, fams, 1, false, w);
         CS(run_norm2(psi, N, w.scal, w.npart, st));
         PassArgs a = base_args(P, psi, w.scal);
         a.tile_out = w.tiles;
@@ -1730,7 +1741,7 @@ sre_status sre_workspace_bytes(int N, int mode, long long n_x, int z_per_x, cons
     CS(plan_for_tuned(N, &o, 32, P, mode == SRE_MC_UNIFORM));
     Arena A(nullptr);
     McWS w;
-    layout_mc(A, P, mode, n_x, z_per_x, w);
+    layout_mc(A, P, mode, n_x, z_per_x, tiled_psi(P, o, n_x), w);
     *bytes = A.off;
     return SRE_OK;
 }
@@ -1819,11 +1830,11 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
     CS(plan_for_tuned(N, &o, 32, P, mode == SRE_MC_UNIFORM));
     Arena dry(nullptr);
     McWS w;
-    layout_mc(dry, P, mode, n_x, z_per_x, w);
+    layout_mc(dry, P, mode, n_x, z_per_x, tiled_psi(P, o, n_x), w);
     void *base = nullptr;
     CS(resolve_workspace(workspace, workspace_bytes, dry.off, &base));
     Arena A(base);
-    layout_mc(A, P, mode, n_x, z_per_x, w);
+    layout_mc(A, P, mode, n_x, z_per_x, tiled_psi(P, o, n_x), w);
     const bool marg = mode == SRE_MC_MARGINAL;
     const unsigned long long d = 1ULL << N;
 
@@ -1878,6 +1889,11 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
     a.precision = prec_code(o);
     a.xs = xs_run;
     a.tile_out = w.tiles;
+    if (w.psi_tiled) {
+        CK(launch_psi_tiled((const float2 *)psi, w.psi_tiled, P.lo[0], N, st));
+        count_launches(1);
+        a.psi_tiled = w.psi_tiled;
+    }
     a.want_ranges = marg ? 1 : 0;
     a.want_cand = 0;                 // the estimators need no nullity candidates
     a.err_flag = w.err;
@@ -2240,17 +2256,22 @@ sre_status sre_profile_passes(const void *psi, int N, long long n_x, const sre_o
     CS(plan_for_tuned(N, &o, 32, P));
     Arena dry(nullptr);
     McWS w;
-    layout_mc(dry, P, SRE_MC_UNIFORM, n_x < 2 ? 2 : n_x, 1, w);
+    layout_mc(dry, P, SRE_MC_UNIFORM, n_x < 2 ? 2 : n_x, 1, tiled_psi(P, o, n_x), w);
     void *base = nullptr;
     CS(own_workspace(dry.off, &base));
     Arena A(base);
-    layout_mc(A, P, SRE_MC_UNIFORM, n_x < 2 ? 2 : n_x, 1, w);
+    layout_mc(A, P, SRE_MC_UNIFORM, n_x < 2 ? 2 : n_x, 1, tiled_psi(P, o, n_x), w);
     CS(run_norm2(psi, N, w.scal, w.npart, st));
     CK(launch_draw_x(nullptr, N, n_x, 0, 12345ULL, 0ULL, w.xs, st));
     count_launches(1);
     PassArgs a = base_args(P, psi, w.scal);
     a.precision = prec_code(o);
     a.xs = w.xs;
+    if (w.psi_tiled) {
+        CK(launch_psi_tiled((const float2 *)psi, w.psi_tiled, P.lo[0], N, st));
+        count_launches(1);
+        a.psi_tiled = w.psi_tiled;
+    }
     a.tile_out = w.tiles;
     const long long step = P.B < n_x ? P.B : n_x;
     PassTimer T;

@@ -199,8 +199,19 @@ __device__ __forceinline__ void tile_transform(typename Cfg::C2 (&v)[Cfg::E], ty
 // otherwise one range is one half of a last-pass tile (2^M z).
 constexpr int ZR_FINE = 10;
 
+// Order of psi for the psi-reading strided pass whose rows are only 2^C columns
+// (C = PSI_TILED_COLS: 64 bytes): the amplitudes of 2^C columns, which a tile
+// reads, lie together, row after row. A bit permutation of the index (bits [0, C)
+// columns, then the row bits [lo, N), then the tile's bits [C, lo)), so the
+// partner of an amplitude is its place exclusive-or the place of x.
+constexpr int PSI_TILED_COLS = 3;
+__host__ __device__ __forceinline__ uint32_t psi_tiled_index(uint32_t b, int lo, int N) {
+    constexpr int C = PSI_TILED_COLS;
+    return (b & ((1u << C) - 1u)) | ((b >> lo) << C) | (((b & ((1u << lo) - 1u)) >> C) << (N - lo + C));
+}
+
 // ------------------------------------------------------------- pass args
-enum SrcMode { SRC_PSI_FAMILY = 0, SRC_PSI_Q = 1, SRC_BUF = 2, SRC_GRAM = 3 };
+enum SrcMode { SRC_PSI_FAMILY = 0, SRC_PSI_Q = 1, SRC_BUF = 2, SRC_GRAM = 3, SRC_PSI_TILED = 4 };
 enum DstMode {
     DST_BUF = 0,        // store the partially transformed tile
     DST_MOMENTS = 1,    // family epilogue: moments, candidates, z-range weights
@@ -214,6 +225,7 @@ enum DstMode {
 
 struct PassArgs {
     const float2 *psi;                 // complex64 state
+    const float2 *psi_tiled;           // psi in the order of psi_tiled_index, or NULL
     const unsigned long long *xs;      // family X-masks, or NULL: x = fam_base + slot
     long long fam_base;                // first family of the launch
     long long n_fam;                   // families in the launch
