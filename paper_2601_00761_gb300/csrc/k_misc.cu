@@ -130,10 +130,13 @@ __global__ void __launch_bounds__(256) fam_reduce_kernel(const TilePartial *tp, 
     const int j = x ? 63 - __clzll((long long)x) : n;
     // plain FP64: a family's tile partials are FP32 sums (relative error about
     // 1e-7), far above this sum's rounding
-    double m0 = 0, m1 = 0, m2 = 0, m3 = 0, c = 0;
+    double m[4] = {0.0, 0.0, 0.0, 0.0};
+    unsigned c = 0;
     for (int t = lane; t < tiles; t += 32) {
         const TilePartial &p = tp[(size_t)f * tiles + t];
-        m0 += p.m[0]; m1 += p.m[1]; m2 += p.m[2]; m3 += p.m[3]; c += (double)p.cand;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) m[k] += p.m[k];
+        c |= p.cand;
         if (W) {
             const unsigned long long zt = (unsigned long long)t << M_last;
             const unsigned long long rA = insert0(zt, j) >> RL;
@@ -142,18 +145,13 @@ __global__ void __launch_bounds__(256) fam_reduce_kernel(const TilePartial *tp, 
             W[(size_t)f * nr + rB] = (float)p.w[1];
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        m0 += __shfl_xor_sync(0xffffffffu, m0, o);
-        m1 += __shfl_xor_sync(0xffffffffu, m1, o);
-        m2 += __shfl_xor_sync(0xffffffffu, m2, o);
-        m3 += __shfl_xor_sync(0xffffffffu, m3, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    if (lane == 0) {
+    c = __reduce_or_sync(0xffffffffu, c);
+    int id;
+    const double s = warp_sums<4>(m, id);                // value v in lanes 8 v .. 8 v + 7
+    if ((lane & 7) == 0) {
         FamMoments &o = fm[perm ? (long long)perm[fam_base + f] : fm_base + f];
-        o.m[0] = m0; o.m[1] = m1; o.m[2] = m2; o.m[3] = m3;
-        o.cand = (unsigned long long)c;
+        o.m[id] = s;
+        if (lane == 0) o.cand = (unsigned long long)c;
     }
 }
 
