@@ -136,11 +136,12 @@ sre_status plan_for_tuned(int N, const sre_opts *o, int prec, Plan &P, bool swee
 // one exchange) above a register-only strided pass of up to six, then rows of
 // eleven and twelve (64 points per thread, one exchange). Per packed point,
 // both passes, against the 13-bit rows (one 14-bit tile at N = 15):
-//   N      15    16    17    18    19    20    21    22
-//   13    3.00  3.50  3.44  3.42  4.0   4.01  4.0   4.0  ps
-//   here  2.55  2.57  2.65  2.77  2.8   3.1   3.35  3.6  ps
-// n = 23 needs a third pass below 13 bits.
-int sweep_radix(int n) { return n <= 16 ? 10 : n == 17 ? 11 : n == 23 ? 13 : 12; }
+//   N      15    16    17    18    19    20    21    22    23
+//   13    3.00  3.50  3.11  3.11  3.09  3.18  3.61  3.73  4.10 ps
+//   here  2.5   2.4   2.54  2.90  2.94  3.18  3.54  3.73  3.96 ps
+// n = 19 and 21 are even or better with 13 (strided passes of 6 and 8 bits, not 7
+// and 9), n = 23 needs a third pass below 13.
+int sweep_radix(int n) { return n <= 16 ? 10 : n == 17 ? 11 : n == 19 || n == 21 || n == 23 ? 13 : 12; }
 constexpr int SWEEP_SINGLE_MMAX = 13;
 
 sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P, bool sweep) {
@@ -207,7 +208,11 @@ sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P, bool sweep) {
     if (prec == 32 && B < BATCH_MIN_LARGE)
         B = std::min(BATCH_MIN_LARGE, (long long)(BATCH_BYTES_LARGE / P.slot_bytes));
     if (B < 1) B = 1;
-    if (B > 4096) B = 4096;
+    // sweeps of small states: fewer, longer launches (exact calls with 4096 against
+    // 16384 families per launch: N = 15 1.69 and 1.53 ms, N = 16 5.93 and 5.63 ms,
+    // N = 17 23.2 and 22.3 ms, N = 18, 8192 families, 101.3 and 99.8 ms)
+    const long long most = sweep ? 16384 : 4096;
+    if (B > most) B = most;
     if (prec == 32 && o && o->x_batch > 0) B = o->x_batch;
     P.B = B;
     P.RL = fine_ranges(P) ? ZR_FINE : P.M_last;
@@ -299,6 +304,8 @@ struct McWS {
     double *y, *out;
     int *err;        // device error word (SRE_ERR_* bits)
 };
+
+constexpr int FAMILY_ORDER_NMIN = 21;    // sre_mc orders its families from here on
 
 // Whether the first strided pass reads a copy of psi in tile order: its rows have
 // 8 columns (10 bits: N = 24, and N = 23 without z draws) and there are families
@@ -1861,22 +1868,27 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
     // partner tiles of a launch span a few aligned blocks), then by index.
     // Each family keeps its own index for its moments, draw stream and
     // outputs, so no result depends on the order.
+    // Up to N = 20 (8 MB of psi) the order is not worth the trip to the host: calls
+    // of 300 and 5001 uniform families at N = 18 0.28 -> 0.24 and 2.41 -> 2.08 ms
+    // without it, at N = 20 0.69 -> 0.66 and 9.40 -> 9.13 ms; at N = 21 19.4 and
+    // 19.9 ms, at N = 24 178 and 198 ms.
     const unsigned long long *xs_run = w.xs, *perm = nullptr;
-    if (P.npass > 1) {
+    if (P.npass > 1 && N >= FAMILY_ORDER_NMIN) {
         std::vector<unsigned long long> hx((size_t)n_x), order((size_t)n_x), hxo((size_t)n_x);
         CK(cudaMemcpyAsync(hx.data(), w.xs, sizeof(unsigned long long) * (size_t)n_x, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
         const int cb = P.ms[0] - P.K[0], tb = P.lo[0] - cb;
-        auto key = [&](unsigned long long x) {
+        constexpr int IB = 40;                       // index bits: n_x < 2^40, and the keys fit the other 24
+        for (long long i = 0; i < n_x; ++i) {
+            const unsigned long long x = hx[(size_t)i];
             const unsigned long long j = x ? (unsigned long long)(63 - __builtin_clzll(x)) : 0ULL;
-            return (j << 40) | ((x >> cb) & ((1ULL << tb) - 1ULL));
-        };
-        for (long long i = 0; i < n_x; ++i) order[(size_t)i] = (unsigned long long)i;
-        std::sort(order.begin(), order.end(), [&](unsigned long long p, unsigned long long q) {
-            const unsigned long long kp = key(hx[p]), kq = key(hx[q]);
-            return kp != kq ? kp < kq : p < q;
-        });
-        for (long long i = 0; i < n_x; ++i) hxo[(size_t)i] = hx[order[(size_t)i]];
+            order[(size_t)i] = (((j << tb) | ((x >> cb) & ((1ULL << tb) - 1ULL))) << IB) | (unsigned long long)i;
+        }
+        std::sort(order.begin(), order.end());
+        for (long long i = 0; i < n_x; ++i) {
+            order[(size_t)i] &= (1ULL << IB) - 1ULL;
+            hxo[(size_t)i] = hx[order[(size_t)i]];
+        }
         CK(cudaMemcpyAsync(w.xs_ord, hxo.data(), sizeof(unsigned long long) * (size_t)n_x, cudaMemcpyHostToDevice, st));
         CK(cudaMemcpyAsync(w.perm, order.data(), sizeof(unsigned long long) * (size_t)n_x, cudaMemcpyHostToDevice,
                            st));
