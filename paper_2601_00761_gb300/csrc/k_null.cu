@@ -42,20 +42,25 @@ __device__ __forceinline__ double flip(double v, unsigned sgn) {
     return __hiloint2double(__double2hiint(v) ^ (int)sgn, __double2loint(v));
 }
 
-// h(g) in FP64 (exact products of the FP32 amplitudes, one rounding per sum)
-__device__ __forceinline__ void hval(const float2 *psi, uint32_t x, int j, uint32_t half, uint32_t g, double &hr,
-                                     double &hi) {
+// The amplitudes of h(g), widened: h = (wx ux + wy uy, wx uy - wy ux), or, for
+// x = 0, (ux^2 + uy^2, wx^2 + wy^2).
+struct Amps { double ux, uy, wx, wy; };
+__device__ __forceinline__ Amps hload(const float2 *psi, uint32_t x, int j, uint32_t half, uint32_t g) {
+    const uint32_t b = x ? (uint32_t)insert0(g, j) : g;
+    const float2 u = __ldg(psi + b), w = __ldg(psi + (x ? b ^ x : b + half));
+    return {f2d(u.x), f2d(u.y), f2d(w.x), f2d(w.y)};
+}
+// (ar, ai) += (-1)^sgn h: the products go into the sums by fused multiply-adds,
+// four FP64 operations a point instead of six (recounts of 128 states of N = 8..16
+// 15.7 -> 12.6 ms)
+__device__ __forceinline__ void hadd(uint32_t x, const Amps &a, unsigned sgn, double &ar, double &ai) {
     if (x) {
-        const uint32_t b = (uint32_t)insert0(g, j);
-        const float2 u = __ldg(psi + b), w = __ldg(psi + (b ^ x));
-        const double ux = f2d(u.x), uy = f2d(u.y), wx = f2d(w.x), wy = f2d(w.y);
-        hr = fma(wx, ux, wy * uy);
-        hi = fma(wx, uy, -(wy * ux));
+        const double wx = flip(a.wx, sgn), wy = flip(a.wy, sgn);
+        ar = fma(wy, a.uy, fma(wx, a.ux, ar));
+        ai = fma(-wy, a.ux, fma(wx, a.uy, ai));
     } else {
-        const float2 u = __ldg(psi + g), w = __ldg(psi + (g + half));
-        const double ux = f2d(u.x), uy = f2d(u.y), wx = f2d(w.x), wy = f2d(w.y);
-        hr = fma(ux, ux, uy * uy);
-        hi = fma(wx, wx, wy * wy);
+        ar = fma(flip(a.uy, sgn), a.uy, fma(flip(a.ux, sgn), a.ux, ar));
+        ai = fma(flip(a.wy, sgn), a.wy, fma(flip(a.wx, sgn), a.wx, ai));
     }
 }
 
@@ -66,13 +71,18 @@ __device__ __forceinline__ void direct_sums(const float2 *psi, uint32_t x, int j
                                             double (&ai)[NB_CHUNK]) {
 #pragma unroll 2
     for (uint32_t g = first; g < half; g += stride) {
-        double hr, hi;
-        hval(psi, x, j, half, g, hr, hi);
+        const Amps h = hload(psi, x, j, half, g);
+        double hr = 0.0, hi = 0.0;             // several sums take the same h: form it once
+        if (G > 1) hadd(x, h, 0u, hr, hi);
 #pragma unroll
         for (int i = 0; i < G; ++i) {
             const unsigned sgn = (unsigned)(__popc(g & zl[i]) & 1) << 31;
-            ar[i] += flip(hr, sgn);
-            ai[i] += flip(hi, sgn);
+            if (G > 1) {
+                ar[i] += flip(hr, sgn);
+                ai[i] += flip(hi, sgn);
+            } else {
+                hadd(x, h, sgn, ar[i], ai[i]);
+            }
         }
     }
 }
@@ -108,11 +118,7 @@ __device__ __forceinline__ void coset_sums(const float2 *psi, uint32_t x, int j,
 #pragma unroll
         for (int b = 0; b < NBIN; ++b) {
             const uint32_t g = G0 ^ offl[b];
-            double hr, hi;
-            hval(psi, x, j, half, g, hr, hi);
-            const unsigned sgn = (unsigned)(__popc(g & z0) & 1) << 31;
-            ar[b] += flip(hr, sgn);
-            ai[b] += flip(hi, sgn);
+            hadd(x, hload(psi, x, j, half, g), (unsigned)(__popc(g & z0) & 1) << 31, ar[b], ai[b]);
         }
     }
 }
