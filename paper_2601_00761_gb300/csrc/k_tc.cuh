@@ -24,14 +24,18 @@ __device__ __forceinline__ uint32_t pack_bf16x2(__nv_bfloat16 lo, __nv_bfloat16 
     return *reinterpret_cast<uint32_t *>(&v);
 }
 
-// x = sum of NSPLIT BF16 parts (part 0 the largest)
+// x0 and x1 each as a sum of NSPLIT BF16 parts (part 0 the largest), the parts of
+// a level packed as an MMA operand word (x0 low). One packed conversion a level
+// for both, on the ALU; converting one value at a time runs on the narrow
+// transcendental pipe.
 template <int NSPLIT>
-__device__ __forceinline__ void split_bf16(float x, __nv_bfloat16 (&p)[NSPLIT]) {
-    float r = x;
+__device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t (&p)[NSPLIT]) {
 #pragma unroll
     for (int s = 0; s < NSPLIT; ++s) {
-        p[s] = __float2bfloat16_rn(r);
-        r = r - __bfloat162float(p[s]);
+        const __nv_bfloat162 v = __floats2bfloat162_rn(x0, x1);
+        p[s] = *reinterpret_cast<const uint32_t *>(&v);
+        x0 -= __uint_as_float(p[s] << 16);
+        x1 -= __uint_as_float(p[s] & 0xffff0000u);
     }
 }
 
@@ -64,27 +68,29 @@ __device__ __forceinline__ uint32_t ins4(uint32_t c, int b, uint32_t p) {
 // One tensor-core round over bits [b, b+4) of the group's tile in shared
 // memory; warps of the group take 8-column blocks in turn. In place: a warp
 // reads and writes the same 16 x 8 block.
-template <class Cfg, int NSPLIT>
-__device__ __forceinline__ void tc_round(float2 *tile, int b, const uint32_t (&a)[4], int warp, int nwarps) {
+template <class Cfg, int NSPLIT, int NWARPS>
+__device__ __forceinline__ void tc_round(float2 *tile, int b, const uint32_t (&a)[4], int warp) {
     const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
     constexpr int COLS = 1 << (Cfg::M - 4);
-    for (int c0 = warp * 8; c0 < COLS; c0 += nwarps * 8) {
+#pragma unroll
+    for (int i0 = 0; i0 < COLS; i0 += NWARPS * 8) {
+        const int c0 = i0 + warp * 8;
+        if (COLS < NWARPS * 8 && c0 >= COLS) break;
         const uint32_t cin = (uint32_t)(c0 + g);
         float2 xv[4];
         const uint32_t pin[4] = {(uint32_t)(2 * q), (uint32_t)(2 * q + 1), (uint32_t)(2 * q + 8), (uint32_t)(2 * q + 9)};
 #pragma unroll
         for (int i = 0; i < 4; ++i) xv[i] = tile[Cfg::pad(ins4(cin, b, pin[i]))];
         float dre[4] = {0.f, 0.f, 0.f, 0.f}, dim[4] = {0.f, 0.f, 0.f, 0.f};
-        __nv_bfloat16 pr[4][NSPLIT], pi[4][NSPLIT];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            split_bf16<NSPLIT>(xv[i].x, pr[i]);
-            split_bf16<NSPLIT>(xv[i].y, pi[i]);
-        }
+        uint32_t re0[NSPLIT], re1[NSPLIT], im0[NSPLIT], im1[NSPLIT];
+        split_bf16x2<NSPLIT>(xv[0].x, xv[1].x, re0);
+        split_bf16x2<NSPLIT>(xv[2].x, xv[3].x, re1);
+        split_bf16x2<NSPLIT>(xv[0].y, xv[1].y, im0);
+        split_bf16x2<NSPLIT>(xv[2].y, xv[3].y, im1);
 #pragma unroll
         for (int s = NSPLIT - 1; s >= 0; --s) {   // smallest parts first
-            mma_bf16_16816(dre, a, pack_bf16x2(pr[0][s], pr[1][s]), pack_bf16x2(pr[2][s], pr[3][s]));
-            mma_bf16_16816(dim, a, pack_bf16x2(pi[0][s], pi[1][s]), pack_bf16x2(pi[2][s], pi[3][s]));
+            mma_bf16_16816(dre, a, re0[s], re1[s]);
+            mma_bf16_16816(dim, a, im0[s], im1[s]);
         }
         __syncwarp();
         // D(m, n): rows m = g, g+8 (output point), columns n = 2q, 2q+1
@@ -139,8 +145,9 @@ __device__ __forceinline__ void tc_tile_transform(float2 (&v)[Cfg::E], float2 *s
     const int warp = (int)(t >> 5);
     int b = Cfg::LO;
     static_assert(Cfg::T >= 32, "tensor-core rounds need whole warps per tile");
-    for (; b + 4 <= Cfg::M; b += 4) {
-        tc_round<Cfg, NSPLIT>(tile, b, a, warp, WPG);
+#pragma unroll
+    for (; b + 4 <= Cfg::M; b += 4) {             // unrolled: b and the addresses are constants
+        tc_round<Cfg, NSPLIT, WPG>(tile, b, a, warp);
         __syncthreads();
     }
     if (b < Cfg::M) {
