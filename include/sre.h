@@ -142,7 +142,9 @@ SRE_API const char *sre_last_error(void);
 /* Fill *opts with the defaults (FP32 SIMT, eps_null 1e-6, planned tiles). */
 SRE_API void sre_default_opts(sre_opts *opts);
 
-/* Plan of the transform passes (host only). opts may be NULL. */
+/* Plan of the transform passes (host only). opts may be NULL. Without tiling
+ * options it is the marginal estimator's; exact and uniform sweeps, which draw
+ * no z, may split the same bits otherwise (sre_result.n_passes tells). */
 SRE_API sre_status sre_make_plan(int N, const sre_opts *opts, sre_plan *plan);
 
 /* Device scratch that sre_exact (mode -1) or sre_mc (mode SRE_MC_*) needs
@@ -172,7 +174,7 @@ SRE_API sre_status sre_exact(const void *psi_c64_dev, int N, const sre_opts *opt
  * one call (Algorithm 1 per state; psi_ptrs_host[i] a device pointer,
  * Ns_host[i] in 1..20). States are grouped by N. In the FP32 sweep every
  * family of every state with N <= 14 (one shared-memory tile per family) is
- * one item of a single persistent launch; each launch for N >= 15 covers the
+ * one item of a single persistent launch; each launch for N >= 15 covers
  * (state, family) items of a chunk of same-N states. The launch sequence of
  * the whole batch is captured once into a CUDA graph (cached for the same
  * batch shape and plans) and replayed; the FP64 nullity recount of candidate

@@ -391,10 +391,9 @@ __global__ void __launch_bounds__(256) scan_chunk_apply(const double *p, unsigne
 }
 
 // chunk sums and their prefix; with cdf, the whole inclusive CDF as well
-cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, double *bsum, int *launches,
-                        cudaStream_t st) {
+cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, double *bsum, double *tot,
+                        int *launches, cudaStream_t st) {
     const long long nb = (long long)((n + SCAN_CHUNK - 1) / SCAN_CHUNK), tiles = (nb + SCAN_TILE - 1) / SCAN_TILE;
-    double *tot = bsum + nb + 1;
     scan_chunk_sums<<<(unsigned)nb, 256, 0, st>>>(p, n, bsum);
     scan_tile_offsets<<<(unsigned)tiles, 1024, 0, st>>>(bsum, nb, tot);
     if (tiles > 1) scan_tile_add<<<(unsigned)tiles, 1024, 0, st>>>(bsum, nb, tot);

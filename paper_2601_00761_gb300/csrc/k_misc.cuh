@@ -77,10 +77,10 @@ cudaError_t launch_fam_reduce(const TilePartial *tp, long long n_fam, int tiles,
                               long long fam_base, int N, int M_last, int RL, FamMoments *fm, long long fm_base,
                               float *W, long long nr, cudaStream_t st, const unsigned long long *perm = nullptr);
 cudaError_t launch_sum_u64(const unsigned long long *v, long long n, unsigned long long *out, cudaStream_t st);
-// bsum: n / SCAN_CHUNK + SCAN_EXTRA doubles, the exclusive prefix of p's chunk
-// sums and the total; cdf (or NULL): the inclusive CDF of p (may be p itself)
-constexpr long long SCAN_EXTRA = 40;
-cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, double *bsum, int *launches,
+// bsum: n / SCAN_CHUNK + 1 doubles (chunks rounded up), the exclusive prefix of p's
+// chunk sums and the total; tot: 32 doubles of scratch; cdf (or NULL): the
+// inclusive CDF of p (may be p itself)
+cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, double *bsum, double *tot, int *launches,
                         cudaStream_t st);
 cudaError_t launch_draw_x(const double *cdf, int N, long long n_x, int mode, unsigned long long seed,
                           unsigned long long ctr0, unsigned long long *xs, cudaStream_t st);

@@ -289,7 +289,7 @@ void layout_exact(Arena &A, const Plan &P, const Plan &P64, ExactWS &w) {
 
 struct McWS {
     double *scal, *npart;
-    double *p, *mwork, *bsum;
+    double *p, *mwork, *bsum;            // mwork is free once p is known: the scans' scratch
     unsigned long long *xs;
     unsigned long long *xs_ord, *perm;   // the families in processing order, and their own indices
     float2 *psi_tiled;                   // psi in tile order, or NULL
@@ -300,7 +300,6 @@ struct McWS {
     DrawInfo *draws;
     unsigned long long *zs;
     float *cz;
-    double *zsum;    // chunk sums of the range rows (rows of more than ZSEL_STAGE_MAX ranges)
     double *y, *out;
     int *err;        // device error word (SRE_ERR_* bits)
 };
@@ -323,7 +322,7 @@ void layout_mc(Arena &A, const Plan &P, int mode, long long n_x, int zpx, bool t
     w.npart = A.take<double>(NORM_BLOCKS);
     w.p = marg ? A.take<double>(d) : nullptr;
     w.mwork = marg ? A.take<double>(d) : nullptr;
-    w.bsum = marg ? A.take<double>(d / SCAN_CHUNK + SCAN_EXTRA) : nullptr;
+    w.bsum = marg ? A.take<double>((d + SCAN_CHUNK - 1) / SCAN_CHUNK + 1) : nullptr;
     w.xs = A.take<unsigned long long>(n_x);
     w.xs_ord = P.npass > 1 ? A.take<unsigned long long>(n_x) : nullptr;
     w.perm = P.npass > 1 ? A.take<unsigned long long>(n_x) : nullptr;
@@ -338,7 +337,6 @@ void layout_mc(Arena &A, const Plan &P, int mode, long long n_x, int zpx, bool t
     w.draws = marg ? A.take<DrawInfo>(nd) : nullptr;
     w.zs = marg ? A.take<unsigned long long>(nd) : nullptr;
     w.cz = A.take<float>(nd);
-    w.zsum = marg && nr > ZSEL_STAGE_MAX ? A.take<double>(256 * (size_t)B) : nullptr;
     w.y = A.take<double>(6 * (size_t)n_x);
     w.out = A.take<double>(24);
     w.err = A.take<int>(1);
@@ -694,6 +692,17 @@ sre_status exact_impl(const void *psi, int N, const sre_opts &o, void *ws, size_
     Arena dry(nullptr);
     ExactWS w;
     layout_exact(dry, P, P64, w);
+    if (ws && ws_bytes < dry.off) {
+        // a caller's workspace that holds the 13-bit split runs that one
+        Plan Q;
+        CS(plan_for_tuned(N, &o, 32, Q));
+        Arena small(nullptr);
+        layout_exact(small, Q, P64, w);
+        if (ws_bytes >= small.off) {
+            P = Q;
+            dry.off = small.off;
+        }
+    }
     void *base = nullptr;
     CS(resolve_workspace(ws, ws_bytes, dry.off, &base));
     Arena A(base);
@@ -1837,11 +1846,24 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
     CS(plan_for_tuned(N, &o, 32, P, mode == SRE_MC_UNIFORM));
     Arena dry(nullptr);
     McWS w;
-    layout_mc(dry, P, mode, n_x, z_per_x, tiled_psi(P, o, n_x), w);
+    bool tiled = tiled_psi(P, o, n_x);
+    layout_mc(dry, P, mode, n_x, z_per_x, tiled, w);
+    if (workspace && workspace_bytes < dry.off) {
+        // a caller's workspace that holds the 13-bit split without the copy of psi runs that one
+        Plan Q;
+        CS(plan_for_tuned(N, &o, 32, Q));
+        Arena small(nullptr);
+        layout_mc(small, Q, mode, n_x, z_per_x, false, w);
+        if (workspace_bytes >= small.off) {
+            P = Q;
+            tiled = false;
+            dry.off = small.off;
+        }
+    }
     void *base = nullptr;
     CS(resolve_workspace(workspace, workspace_bytes, dry.off, &base));
     Arena A(base);
-    layout_mc(A, P, mode, n_x, z_per_x, tiled_psi(P, o, n_x), w);
+    layout_mc(A, P, mode, n_x, z_per_x, tiled, w);
     const bool marg = mode == SRE_MC_MARGINAL;
     const unsigned long long d = 1ULL << N;
 
@@ -1853,7 +1875,7 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
         // whole CDF costs 10 ps per x: few draws on a large state skip the CDF
         const bool chunks = (unsigned long long)n_x <= d / 2048;
         int nl = 0;
-        CK(launch_scan(w.p, d, chunks ? nullptr : w.p, w.bsum, &nl, st));
+        CK(launch_scan(w.p, d, chunks ? nullptr : w.p, w.bsum, w.mwork, &nl, st));
         count_launches(nl);
         if (chunks) CK(launch_draw_x_chunks(w.p, w.bsum, N, n_x, seed, counter0, w.xs, st));
         else CK(launch_draw_x(w.p, N, n_x, 1, seed, counter0, w.xs, st));
@@ -1935,7 +1957,7 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
         count_launches(1);
         if (marg) {
             int nl = 0;
-            CK(launch_zrange_select(w.Wf, nr, nf, fb, z_per_x, seed, counter0, w.draws, perm, w.zsum, &nl, st));
+            CK(launch_zrange_select(w.Wf, nr, nf, fb, z_per_x, seed, counter0, w.draws, perm, w.mwork, &nl, st));
             count_launches(nl);
             PassArgs c = b;
             c.src = w.inter;

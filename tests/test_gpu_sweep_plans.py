@@ -41,3 +41,25 @@ def test_uniform_sweep_split(N):
     b = sre.sre_mc(psi, sre.SRE_MC_UNIFORM, n_x, seed=9, radix_log2=13)
     # the same families: S is (d - 1) times a mean, so compare M; M_1's rounding is relative to S_1 <= 2 N
     assert (np.abs(np.array(a["M"]) - b["M"]) <= _bound(N)).all()
+
+
+def test_workspace_of_the_13_bit_split():
+    """A workspace that holds the 13-bit split (and no copy of psi) is accepted and
+    runs that one; a smaller one is refused."""
+    psi = _psi(17)
+    n = sre.sre_workspace_bytes(17, -1, radix_log2=13)
+    assert n < sre.sre_workspace_bytes(17, -1)
+    ws = torch.empty(n + 256, dtype=torch.uint8, device="cuda")
+    ws = ws[-ws.data_ptr() % 256:][:n]
+    a, b = sre.sre_exact(psi, workspace=ws), sre.sre_exact(psi, radix_log2=13)
+    assert a["M"] == b["M"] and a["stab_count"] == b["stab_count"]
+    with pytest.raises(sre.SreError):
+        sre.sre_exact(psi, workspace=ws[:n // 2])
+    psi = _psi(24)
+    n = sre.sre_workspace_bytes(24, sre.SRE_MC_MARGINAL, 64, 4, precision=sre.SRE_BF16X3_TC)
+    assert n < sre.sre_workspace_bytes(24, sre.SRE_MC_MARGINAL, 64, 4)
+    ws = torch.empty(n + 256, dtype=torch.uint8, device="cuda")
+    ws = ws[-ws.data_ptr() % 256:][:n]
+    a = sre.sre_mc(psi, sre.SRE_MC_MARGINAL, 64, 4, seed=1, workspace=ws, return_samples=True)
+    b = sre.sre_mc(psi, sre.SRE_MC_MARGINAL, 64, 4, seed=1, return_samples=True)
+    assert all(torch.equal(a[k], b[k]) for k in ("xs", "zs", "c"))
