@@ -484,11 +484,11 @@ __device__ __forceinline__ void fwht_pass_body(const PassArgs &a, long long slot
 
     if constexpr (SRC == SRC_BUF && DST == DST_MOMENTS && Cfg::RB == 6) {
         // 12 warps per SM do not keep enough loads in flight for DRAM: the tile
-        // that a CTA one wave of SMs later reads is brought into L2 (the tiles
-        // of a launch are contiguous and run in order). N = 18, 4096 families,
-        // 2^11-point tiles: 1.49 against 1.79 ps per point; two or more waves
-        // ahead are slower, past twelve slower than none.
-        constexpr long long AHEAD = 152;
+        // that runs one wave later (152 SMs x 6 CTAs of 2^12 points; the tiles
+        // of a launch are contiguous and run in order) is brought into L2. Uniform
+        // sweep of N = 18, per point: 1.46 ps against 1.70 at 152 tiles ahead,
+        // 1.67 at 304, 1.46 at 608 and 1216 and 1.51 at 1824.
+        constexpr long long AHEAD = 912;
         const long long tiles = a.slot_elems >> Cfg::M, lin = slot * tiles + (long long)tile + AHEAD;
         if (t == 0 && lin < a.n_fam * tiles)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(

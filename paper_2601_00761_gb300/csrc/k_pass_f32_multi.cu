@@ -39,12 +39,11 @@ cudaError_t launch_f32_strided(int MS, int K, int src, int dst, const PassArgs &
     }
 }
 cudaError_t launch_f32_row(int M, int src, int dst, const PassArgs &a, int tiles, cudaStream_t st) {
-    // moments without z-range weights over 11 and 12 bits: 64 points per
-    // thread, one exchange through shared memory instead of two (per point,
-    // 4096 families of N = 18: 1.49 and 1.53 ps against 1.66 and 1.81)
-    if ((M == 11 || M == 12) && a.precision == 0 && src == SRC_BUF && dst == DST_MOMENTS && !a.want_ranges)
-        return M == 11 ? launch_cfg<TileCfg<float, 11, 0, 6, 1>, SRC_BUF, DST_MOMENTS, 0>(a, tiles, st)
-                       : launch_cfg<TileCfg<float, 12, 0, 6, 1>, SRC_BUF, DST_MOMENTS, 0>(a, tiles, st);
+    // moments without z-range weights over 12 bits: 64 points per thread, one
+    // exchange through shared memory instead of two (uniform sweep of N = 18,
+    // per point: 1.46 against 1.78 ps; over 11 bits 1.65 against 1.64)
+    if (M == 12 && a.precision == 0 && src == SRC_BUF && dst == DST_MOMENTS && !a.want_ranges)
+        return launch_cfg<TileCfg<float, 12, 0, 6, 1>, SRC_BUF, DST_MOMENTS, 0>(a, tiles, st);
     switch (M) {
 #define C(m) case m: return launch_sd<KIND_ROW, TileCfg<float, m, 0, (m == 13 ? F32_ROW13_RB : 5), 1>>(src, dst, a, tiles, st);
     C(10) C(11) C(12) C(13) C(14)

@@ -134,14 +134,13 @@ sre_status plan_for_tuned(int N, const sre_opts *o, int prec, Plan &P, bool swee
 // marginal estimator keeps 13-bit rows; the others take the split with the
 // fewest exchanges through shared memory: rows of ten bits (one warp per tile,
 // one exchange) above a register-only strided pass of up to six, then rows of
-// eleven and twelve (64 points per thread, one exchange). Per packed point,
-// both passes, against the 13-bit rows (one 14-bit tile at N = 15):
+// twelve (64 points per thread, one exchange). Per packed point of a uniform
+// sweep, both passes, against the 13-bit rows (one 14-bit tile at N = 15):
 //   N      15    16    17    18    19    20    21    22    23
-//   13    3.00  3.50  3.11  3.11  3.09  3.18  3.61  3.73  4.10 ps
-//   here  2.5   2.4   2.54  2.90  2.94  3.18  3.54  3.73  3.96 ps
-// n = 19 and 21 are even or better with 13 (strided passes of 6 and 8 bits, not 7
-// and 9), n = 23 needs a third pass below 13.
-int sweep_radix(int n) { return n <= 16 ? 10 : n == 17 ? 11 : n == 19 || n == 21 || n == 23 ? 13 : 12; }
+//   13    4.50  3.27  3.18  3.18  3.15  3.27  3.62  3.81  4.15 ps
+//   here  2.54  2.52  2.56  2.67  2.79  3.20  3.32  3.61  3.78 ps
+// n = 23 needs a third pass below 13 (5.17 against 4.31 ps).
+int sweep_radix(int n) { return n <= 16 ? 10 : n == 23 ? 13 : 12; }
 constexpr int SWEEP_SINGLE_MMAX = 13;
 
 sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P, bool sweep) {
