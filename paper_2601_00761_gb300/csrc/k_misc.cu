@@ -440,12 +440,17 @@ __global__ void draw_x_kernel(const double *cdf, int N, long long n_x, int mode,
 
 // x draws straight from p and the prefix of its chunk sums, without the CDF: a
 // block per draw finds the chunk by bisection and sums that chunk alone. Family 0
-// is x = 0; the others x ~ p(x | x != 0).
+// is x = 0; the others x ~ p(x | x != 0). Only x of positive p are drawn: the
+// prefixes round where threads, chunks and scan tiles meet, so t may lie at or
+// above the last sum (p(0) near 1 leaves few values between c0 and the total) or
+// in a gap before a p of zero. The last positive p below is taken then, in the
+// chunk or in the next lower one that holds any.
 __global__ void __launch_bounds__(128) draw_x_chunk_kernel(const double *p, const double *boff, int N, long long nb,
                                                            unsigned long long seed, unsigned long long ctr0,
                                                            unsigned long long *xs) {
     __shared__ double wsum[4];
-    __shared__ unsigned first;
+    __shared__ int first, last;            // of the chunk: the draw, and the last x of positive p
+    __shared__ long long below;
     const long long i = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (i == 0) {
@@ -459,41 +464,56 @@ __global__ void __launch_bounds__(128) draw_x_chunk_kernel(const double *p, cons
         const long long mid = (lo + hi) >> 1;
         if (boff[mid + 1] > t) hi = mid; else lo = mid + 1;
     }
-    constexpr int PER = (int)SCAN_CHUNK / 128;
-    const unsigned long long base = (unsigned long long)lo * SCAN_CHUNK;
-    const double *q = p + base + (unsigned long long)threadIdx.x * PER;
-    double v[PER], a = 0.0;
+    constexpr int CHUNK = (int)SCAN_CHUNK, PER = CHUNK / 128;
+    for (;;) {
+        const double *q = p + (unsigned long long)lo * CHUNK + (unsigned long long)threadIdx.x * PER;
+        double v[PER], a = 0.0;
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        v[k] = q[k];
-        a += v[k];
-    }
-    double s = a;
+        for (int k = 0; k < PER; ++k) {
+            v[k] = q[k];
+            a += v[k];
+        }
+        double s = a;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double u = __shfl_up_sync(0xffffffffu, s, o);
-        if (lane >= o) s += u;
-    }
-    if (lane == 31) wsum[warp] = s;
-    if (threadIdx.x == 0) first = (unsigned)SCAN_CHUNK;
-    __syncthreads();
-    double run = boff[lo];
-    for (int w = 0; w < warp; ++w) run += wsum[w];
-    run += s - a;
-    unsigned pick = (unsigned)SCAN_CHUNK;
+        for (int o = 1; o < 32; o <<= 1) {
+            const double u = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += u;
+        }
+        if (lane == 31) wsum[warp] = s;
+        if (threadIdx.x == 0) { first = CHUNK; last = -1; below = 0; }
+        __syncthreads();
+        double run = boff[lo];
+        for (int w = 0; w < warp; ++w) run += wsum[w];
+        run += s - a;
+        int pick = CHUNK, end = -1;
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        run += v[k];
-        if (run > t && pick == (unsigned)SCAN_CHUNK) pick = threadIdx.x * PER + k;
-    }
-    if (pick < (unsigned)SCAN_CHUNK) atomicMin(&first, pick);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long x = base + (first < (unsigned)SCAN_CHUNK ? first : (unsigned)SCAN_CHUNK - 1);
-        // rounding left the chunk's end at or below t: its last x of positive p
-        if (first == (unsigned)SCAN_CHUNK)
-            while (x > base && !(p[x] > 0.0)) --x;
-        xs[i] = x ? x : 1ULL;
+        for (int k = 0; k < PER; ++k) {
+            run += v[k];
+            if (v[k] > 0.0) {
+                end = (int)threadIdx.x * PER + k;
+                if (run > t && pick == CHUNK) pick = end;
+            }
+        }
+        if (pick < CHUNK) atomicMin(&first, pick);
+        if (end >= 0) atomicMax(&last, end);
+        __syncthreads();
+        const int f = first, l = last;
+        if (f < CHUNK || l >= 0 || lo == 0) {
+            if (threadIdx.x == 0) {
+                const unsigned long long x = (unsigned long long)lo * CHUNK + (unsigned)(f < CHUNK ? f : l >= 0 ? l : 0);
+                xs[i] = x ? x : 1ULL;
+            }
+            return;
+        }
+        // an empty chunk: the nearest one below whose sum moved the prefix, else chunk 0
+        for (hi = lo; hi > 0; hi -= 128) {
+            const long long c = hi - 1 - (long long)threadIdx.x;
+            const bool up = c >= 0 && boff[c + 1] > boff[c];
+            if (up) atomicMax((unsigned long long *)&below, (unsigned long long)c);
+            if (__syncthreads_or(up)) break;
+        }
+        lo = below;
+        __syncthreads();
     }
 }
 
