@@ -142,6 +142,7 @@ sre_status plan_for_tuned(int N, const sre_opts *o, int prec, Plan &P, bool swee
 // n = 23 needs a third pass below 13 (5.17 against 4.31 ps).
 int sweep_radix(int n) { return n <= 16 ? 10 : n == 23 ? 13 : 12; }
 constexpr int SWEEP_SINGLE_MMAX = 13;
+constexpr long long LAUNCH_FAMILIES = 4096, SWEEP_FAMILIES = 16384;   // most families of a launch
 
 sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P, bool sweep) {
     P = Plan();
@@ -210,11 +211,34 @@ sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P, bool sweep) {
     // sweeps of small states: fewer, longer launches (exact calls with 4096 against
     // 16384 families per launch: N = 15 1.69 and 1.53 ms, N = 16 5.93 and 5.63 ms,
     // N = 17 23.2 and 22.3 ms, N = 18, 8192 families, 101.3 and 99.8 ms)
-    const long long most = sweep ? 16384 : 4096;
+    const long long most = sweep ? SWEEP_FAMILIES : LAUNCH_FAMILIES;
     if (B > most) B = most;
     if (prec == 32 && o && o->x_batch > 0) B = o->x_batch;
     P.B = B;
     P.RL = fine_ranges(P) ? ZR_FINE : P.M_last;
+    return SRE_OK;
+}
+
+// The plans of a call over `families` families, in order of preference, each with
+// an intermediate for no more families than that. A sweep's own split runs up to
+// SWEEP_FAMILIES a launch (8 GiB of intermediate from N = 18 on); where memory is
+// short it runs LAUNCH_FAMILIES, and then the 13-bit split.
+sre_status plans_for_call(int N, const sre_opts *o, bool sweep, long long families, std::vector<Plan> &plans) {
+    plans.clear();
+    Plan P;
+    auto add = [&](Plan Q) {
+        Q.B = std::min(Q.B, families);
+        plans.push_back(Q);
+    };
+    CS(plan_for_tuned(N, o, 32, P, sweep));
+    add(P);
+    if (!sweep || P.npass == 1) return SRE_OK;
+    if (P.npass > 1 && P.B > LAUNCH_FAMILIES && families > LAUNCH_FAMILIES && !(o && o->x_batch > 0)) {
+        P.B = LAUNCH_FAMILIES;
+        add(P);
+    }
+    CS(plan_for_tuned(N, o, 32, P));
+    if (P.npass != plans[0].npass || P.M_last != plans[0].M_last) add(P);
     return SRE_OK;
 }
 
@@ -325,9 +349,9 @@ void layout_mc(Arena &A, const Plan &P, int mode, long long n_x, int zpx, bool t
     w.xs = A.take<unsigned long long>(n_x);
     w.xs_ord = P.npass > 1 ? A.take<unsigned long long>(n_x) : nullptr;
     w.perm = P.npass > 1 ? A.take<unsigned long long>(n_x) : nullptr;
-    const long long B = P.npass > 1 ? P.B : (n_x < P.B ? n_x : P.B);
+    const long long B = std::min(n_x, P.B);
     w.psi_tiled = tiled ? A.take<float2>(d) : nullptr;
-    w.inter = P.npass > 1 ? (void *)A.take<char>(P.slot_bytes * (size_t)P.B) : nullptr;
+    w.inter = P.npass > 1 ? (void *)A.take<char>(P.slot_bytes * (size_t)B) : nullptr;
     w.tiles = A.take<TilePartial>((size_t)B * (size_t)P.tiles_last);
     w.fm = A.take<FamMoments>(n_x);
     const long long nr = 1LL << (P.N - P.RL);
@@ -343,41 +367,68 @@ void layout_mc(Arena &A, const Plan &P, int mode, long long n_x, int zpx, bool t
 
 // ------------------------------------------------ library-owned workspace
 std::mutex g_ws_mu;
-struct DevWS { void *p = nullptr; size_t n = 0; };
+struct DevWS { void *p = nullptr; size_t n = 0, refused = SIZE_MAX; };
 std::vector<DevWS> g_ws;
 struct DevBuf { void *p = nullptr; size_t n = 0; };
 std::vector<DevBuf> g_gatebuf;
 
-sre_status own_workspace(size_t need, void **out) {
+// The library's workspace for the first of several layouts (needs, in order of
+// preference) that device memory holds; *which receives it. A size that was
+// refused is not tried again while the workspace holds a later layout, so that
+// calls under memory pressure do not free and allocate each time
+// (sre_release_workspace forgets it).
+sre_status own_workspace(const std::vector<size_t> &needs, size_t *which, void **out) {
     int dev = 0;
     CK(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lk(g_ws_mu);
     if ((int)g_ws.size() <= dev) g_ws.resize(dev + 1);
     DevWS &w = g_ws[dev];
-    if (w.n < need) {
-        if (w.p) CK(cudaFree(w.p));
-        w.p = nullptr;
-        w.n = 0;
-        cudaError_t e = cudaMalloc(&w.p, need);
-        g_allocs.fetch_add(1, std::memory_order_relaxed);
-        if (e != cudaSuccess) {
+    const size_t smallest = *std::min_element(needs.begin(), needs.end());
+    for (size_t i = 0; i < needs.size(); ++i) {
+        const size_t need = needs[i];
+        *which = i;
+        if (w.n < need) {
+            if (need >= w.refused && w.n >= smallest) continue;
+            if (w.p) CK(cudaFree(w.p));
             w.p = nullptr;
-            return fail(SRE_ENOMEM, "cudaMalloc(%zu) failed: %s", need, cudaGetErrorString(e));
+            w.n = 0;
+            cudaError_t e = cudaMalloc(&w.p, need);
+            if (e != cudaSuccess) {
+                cudaGetLastError();              // reported here, not by the next launch
+                w.p = nullptr;
+                w.refused = std::min(w.refused, need);
+                fail(SRE_ENOMEM, "cudaMalloc(%zu) failed: %s", need, cudaGetErrorString(e));
+                continue;
+            }
+            g_allocs.fetch_add(1, std::memory_order_relaxed);
+            w.n = need;
+            if (need >= w.refused) w.refused = SIZE_MAX;
         }
-        w.n = need;
+        *out = w.p;
+        return SRE_OK;
     }
-    *out = w.p;
+    return SRE_ENOMEM;
+}
+
+sre_status own_workspace(size_t need, void **out) {
+    size_t which = 0;
+    return own_workspace(std::vector<size_t>{need}, &which, out);
+}
+
+// The workspace for the first of several layouts that fits: a caller's by its
+// size, else the library's.
+sre_status resolve_workspace(void *ws, size_t ws_bytes, const std::vector<size_t> &needs, size_t *which, void **out) {
+    if (!ws) return own_workspace(needs, which, out);
+    for (*which = 0; *which < needs.size() && ws_bytes < needs[*which];) ++*which;
+    if (*which == needs.size()) return fail(SRE_EINVAL, "workspace of %zu bytes, %zu needed", ws_bytes, needs[0]);
+    if (((uintptr_t)ws) & 255) return fail(SRE_EINVAL, "workspace must be 256-byte aligned");
+    *out = ws;
     return SRE_OK;
 }
 
 sre_status resolve_workspace(void *ws, size_t ws_bytes, size_t need, void **out) {
-    if (ws) {
-        if (ws_bytes < need) return fail(SRE_EINVAL, "workspace of %zu bytes, %zu needed", ws_bytes, need);
-        if (((uintptr_t)ws) & 255) return fail(SRE_EINVAL, "workspace must be 256-byte aligned");
-        *out = ws;
-        return SRE_OK;
-    }
-    return own_workspace(need, out);
+    size_t which = 0;
+    return resolve_workspace(ws, ws_bytes, std::vector<size_t>{need}, &which, out);
 }
 
 // ------------------------------------------------------------ checks
@@ -685,29 +736,25 @@ sre_status nullity_from_count(long long cnt, int N, sre_result *r) {
 // exact sweep; with_moments=false still computes them (they are free)
 sre_status exact_impl(const void *psi, int N, const sre_opts &o, void *ws, size_t ws_bytes, cudaStream_t st,
                       sre_result *out) {
-    Plan P, P64;
-    CS(plan_for_tuned(N, &o, 32, P, true));
+    const unsigned long long d = 1ULL << N;
+    std::vector<Plan> plans;
+    Plan P64;
+    CS(plans_for_call(N, &o, true, (long long)d, plans));
     CS(plan_for(N, nullptr, 64, P64));
-    Arena dry(nullptr);
     ExactWS w;
-    layout_exact(dry, P, P64, w);
-    if (ws && ws_bytes < dry.off) {
-        // a caller's workspace that holds the 13-bit split runs that one
-        Plan Q;
-        CS(plan_for_tuned(N, &o, 32, Q));
-        Arena small(nullptr);
-        layout_exact(small, Q, P64, w);
-        if (ws_bytes >= small.off) {
-            P = Q;
-            dry.off = small.off;
-        }
+    std::vector<size_t> needs;
+    for (const Plan &Q : plans) {
+        Arena dry(nullptr);
+        layout_exact(dry, Q, P64, w);
+        needs.push_back(dry.off);
     }
     void *base = nullptr;
-    CS(resolve_workspace(ws, ws_bytes, dry.off, &base));
+    size_t which = 0;
+    CS(resolve_workspace(ws, ws_bytes, needs, &which, &base));
+    const Plan P = plans[which];
     Arena A(base);
     layout_exact(A, P, P64, w);
 
-    const unsigned long long d = 1ULL << N;
     CS(run_norm2(psi, N, w.scal, w.npart, st, w.nflag));
     PassArgs a = base_args(P, psi, w.scal);
     a.precision = prec_code(o);
@@ -783,6 +830,7 @@ struct BucketPlan {
     int N;
     std::vector<int> idx;       // caller indices of the bucket's states
     int off;                    // first slot of the bucket in the per-state arrays
+    std::vector<Plan> plans;    // by memory (plans_for_call); P is the one that runs
     Plan P, P64;
     int states_per_chunk;
     unsigned long long *flags;  // flagged families of the bucket (capacity: its families)
@@ -1001,7 +1049,7 @@ void layout_batch(Arena &A, int count, std::vector<BucketPlan> &B, BatchWS &w, c
             // the nullity recount of the flagged families still runs through
             // the chunked intermediates (its FP32 candidate pass and the FP64
             // transform)
-            if (b.P.npass > 1) inter_b = std::max(inter_b, b.P.slot_bytes * (size_t)b.P.B);
+            if (b.P.npass > 1) inter_b = std::max(inter_b, b.P.slot_bytes * (size_t)std::min(b.P.B, NULL_CHUNK));
             if (b.P64.npass > 1) inter64_b = std::max(inter64_b, b.P64.slot_bytes * (size_t)b.P64.B);
             continue;
         }
@@ -1171,9 +1219,10 @@ sre_status batched_impl(const void *const *psi_ptrs, const int *Ns, int count, c
             b.idx = by[N];
             b.off = off;
             off += (int)b.idx.size();
-            CS(plan_for_tuned(N, &o, 32, b.P, true));
             CS(plan_for(N, nullptr, 64, b.P64));
             b.states_per_chunk = (int)std::max(1LL, BATCH_CHUNK_FAMILIES >> N);
+            CS(plans_for_call(N, &o, true, (long long)std::min(b.states_per_chunk, (int)b.idx.size()) << N, b.plans));
+            b.P = b.plans[0];
             b.flags = nullptr;
             b.flag_cap = 0;
             b.persistent = false;
@@ -1183,12 +1232,23 @@ sre_status batched_impl(const void *const *psi_ptrs, const int *Ns, int count, c
     // one persistent launch over the single-pass buckets of the FP32 sweep
     // (with opts.batch_queue: over every bucket)
     PersistLayout L;
-    persist_plan(B, prec_code(o), o.batch_queue != 0, L);
-    Arena dry(nullptr);
     BatchWS w;
-    layout_batch(dry, count, B, w, &L);
+    size_t variants = 1, which = 0;
+    for (const BucketPlan &b : B) variants = std::max(variants, b.plans.size());
+    auto take_plans = [&](size_t i) {
+        for (BucketPlan &b : B) b.P = b.plans[std::min(i, b.plans.size() - 1)];
+        persist_plan(B, prec_code(o), o.batch_queue != 0, L);
+    };
+    std::vector<size_t> needs;
+    for (size_t i = 0; i < variants; ++i) {
+        take_plans(i);
+        Arena dry(nullptr);
+        layout_batch(dry, count, B, w, &L);
+        needs.push_back(dry.off);
+    }
     void *base = nullptr;
-    CS(own_workspace(dry.off, &base));
+    CS(own_workspace(needs, &which, &base));
+    take_plans(which);
     Arena A(base);
     layout_batch(A, count, B, w, &L);
     if (L.n_items > 0) {
@@ -1738,25 +1798,25 @@ sre_status sre_workspace_bytes(int N, int mode, long long n_x, int z_per_x, cons
     if (!bytes) return fail(SRE_EINVAL, "bytes is NULL");
     sre_opts o;
     CS(check_opts(opts, o));
-    Plan P;
+    std::vector<Plan> plans;
     if (mode == -1) {
         if (N < 1 || N > 26) return fail(SRE_EINVAL, "exact: N=%d outside 1..26", N);
         Plan P64;
-        CS(plan_for_tuned(N, &o, 32, P, true));
+        CS(plans_for_call(N, &o, true, 1LL << N, plans));
         CS(plan_for(N, nullptr, 64, P64));
         Arena A(nullptr);
         ExactWS w;
-        layout_exact(A, P, P64, w);
+        layout_exact(A, plans[0], P64, w);
         *bytes = A.off;
         return SRE_OK;
     }
     if (mode != SRE_MC_UNIFORM && mode != SRE_MC_MARGINAL) return fail(SRE_EINVAL, "unknown mode %d", mode);
     if (N < 2 || N > 30) return fail(SRE_EINVAL, "mc: N=%d outside 2..30", N);
     if (n_x < 2 || (mode == SRE_MC_MARGINAL && z_per_x < 1)) return fail(SRE_EINVAL, "n_x >= 2 and z_per_x >= 1 required");
-    CS(plan_for_tuned(N, &o, 32, P, mode == SRE_MC_UNIFORM));
+    CS(plans_for_call(N, &o, mode == SRE_MC_UNIFORM, n_x, plans));
     Arena A(nullptr);
     McWS w;
-    layout_mc(A, P, mode, n_x, z_per_x, tiled_psi(P, o, n_x), w);
+    layout_mc(A, plans[0], mode, n_x, z_per_x, tiled_psi(plans[0], o, n_x), w);
     *bytes = A.off;
     return SRE_OK;
 }
@@ -1841,26 +1901,23 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
     sre_opts o;
     CS(check_opts(opts, o));
     cudaStream_t st = (cudaStream_t)stream;
-    Plan P;
-    CS(plan_for_tuned(N, &o, 32, P, mode == SRE_MC_UNIFORM));
-    Arena dry(nullptr);
+    std::vector<Plan> plans;
+    CS(plans_for_call(N, &o, mode == SRE_MC_UNIFORM, n_x, plans));
+    const bool tiled_first = tiled_psi(plans[0], o, n_x);
+    if (tiled_first) plans.insert(plans.begin(), Plan(plans[0]));      // with the copy of psi, then without
     McWS w;
-    bool tiled = tiled_psi(P, o, n_x);
-    layout_mc(dry, P, mode, n_x, z_per_x, tiled, w);
-    if (workspace && workspace_bytes < dry.off) {
-        // a caller's workspace that holds the 13-bit split without the copy of psi runs that one
-        Plan Q;
-        CS(plan_for_tuned(N, &o, 32, Q));
-        Arena small(nullptr);
-        layout_mc(small, Q, mode, n_x, z_per_x, false, w);
-        if (workspace_bytes >= small.off) {
-            P = Q;
-            tiled = false;
-            dry.off = small.off;
-        }
+    std::vector<size_t> needs;
+    auto tiled_plan = [&](size_t i) { return tiled_first && i == 0; };
+    for (size_t i = 0; i < plans.size(); ++i) {
+        Arena dry(nullptr);
+        layout_mc(dry, plans[i], mode, n_x, z_per_x, tiled_plan(i), w);
+        needs.push_back(dry.off);
     }
     void *base = nullptr;
-    CS(resolve_workspace(workspace, workspace_bytes, dry.off, &base));
+    size_t which = 0;
+    CS(resolve_workspace(workspace, workspace_bytes, needs, &which, &base));
+    const Plan P = plans[which];
+    const bool tiled = tiled_plan(which);
     Arena A(base);
     layout_mc(A, P, mode, n_x, z_per_x, tiled, w);
     const bool marg = mode == SRE_MC_MARGINAL;
@@ -2289,6 +2346,7 @@ sre_status sre_profile_passes(const void *psi, int N, long long n_x, const sre_o
     CS(plan_for_tuned(N, &o, 32, P));
     Arena dry(nullptr);
     McWS w;
+    P.B = std::min(P.B, n_x);
     layout_mc(dry, P, SRE_MC_UNIFORM, n_x < 2 ? 2 : n_x, 1, tiled_psi(P, o, n_x), w);
     void *base = nullptr;
     CS(own_workspace(dry.off, &base));
