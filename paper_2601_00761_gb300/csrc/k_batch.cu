@@ -246,13 +246,10 @@ size_t batch_persistent_smem() {
 
 template <bool DEP>
 cudaError_t launch_queue(const BatchQueue &q, int grid, cudaStream_t st) {
-    static bool attr = false;
+    static SmemOptIn optin;
     const size_t smem = batch_persistent_smem();
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(batch_persistent_kernel<DEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    const cudaError_t e = optin.allow((const void *)batch_persistent_kernel<DEP>, smem);
+    if (e != cudaSuccess) return e;
     batch_persistent_kernel<DEP><<<grid, 256, smem, st>>>(q);
     return cudaGetLastError();
 }

@@ -344,15 +344,12 @@ cudaError_t launch_gate_blocks(float2 *psi, int N, const GateRow *gates_dev, con
     const size_t tile_max = sizeof(float2) << (N < GATE_BLOCK_Q ? N : GATE_BLOCK_Q);
     const size_t smem_max = rounds_dev && mats_dev ? tile_max + sizeof(float2) * 16 * (size_t)max_ng : tile_max;
     if (smem_max > 200 * 1024) return cudaErrorInvalidValue;
-    static size_t attr[3] = {0, 0, 0};
+    static SmemOptIn optin[3];
     const int which = !rounds_dev ? 0 : mats_dev ? 1 : 2;
-    if (attr[which] < smem_max) {
-        const void *k = which == 0 ? (const void *)gate_inplace_kernel
-                      : which == 1 ? (const void *)gate_block_kernel<true> : (const void *)gate_block_kernel<false>;
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
-        if (e != cudaSuccess) return e;
-        attr[which] = smem_max;
-    }
+    const cudaError_t ea = optin[which].allow(which == 0 ? (const void *)gate_inplace_kernel
+                                              : which == 1 ? (const void *)gate_block_kernel<true>
+                                                           : (const void *)gate_block_kernel<false>, smem_max);
+    if (ea != cudaSuccess) return ea;
     for (int b = 0; b < n_blocks; ++b) {
         GateBlockParams p;
         p.r0 = blocks[b].r0;

@@ -346,15 +346,12 @@ cudaError_t launch_gram(const float2 *psi, int N, int NA, float2 *C, void *plane
     const unsigned long long dA = 1ULL << NA, dBc = 1ULL << cl;
     const int nt = (int)(dA / GRAM_T);
     const int ntiles = nt * (nt + 1) / 2;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GRAM_SMEM);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static SmemOptIn optin;
+    cudaError_t e = optin.allow((const void *)gram_tc_kernel, GRAM_SMEM);
+    if (e != cudaSuccess) return e;
     CUtensorMap tp;
     // each plane as (d_A dBc / 16) rows of 16 columns (the tiled layout of gram_split_kernel)
-    cudaError_t e = tc05_make_map_bf16(&tp, planes, dA * (dBc / GRAM_KB), GRAM_KB, GRAM_KB, GRAM_T, 32, 6);
+    e = tc05_make_map_bf16(&tp, planes, dA * (dBc / GRAM_KB), GRAM_KB, GRAM_KB, GRAM_T, 32, 6);
     if (e != cudaSuccess) return e;
     for (long long e0 = 0; e0 < (1LL << NB); e0 += (long long)dBc) {
         gram_split_kernel<<<dim3((unsigned)(dA / 32), (unsigned)(dBc / 32)), 256, 0, st>>>(

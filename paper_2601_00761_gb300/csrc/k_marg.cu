@@ -354,18 +354,10 @@ __global__ void __launch_bounds__(MT, 2) marg_row(double2 *buf) {
     for (int k = 0; k < 16; ++k) row[melem(t, k, 8)] = make_double2(unfix(v[k].x, E), unfix_alu(v[k].y, E));
 }
 
-template <class Kernel>
-cudaError_t smem_attr(Kernel *k, bool &done) {
-    if (done) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MARG_SMEM);
-    done = e == cudaSuccess;
-    return e;
-}
-
 template <int K, int SRC, int DST>
 cudaError_t strided(const float2 *psi, double2 *buf, double *p, int n, int lo, const double *scal, cudaStream_t st) {
-    static bool done = false;
-    const cudaError_t e = smem_attr(marg_strided<K, SRC, DST>, done);
+    static SmemOptIn optin;
+    const cudaError_t e = optin.allow((const void *)marg_strided<K, SRC, DST>, MARG_SMEM);
     if (e != cudaSuccess) return e;
     marg_strided<K, SRC, DST><<<1u << (n - MB), MT, MARG_SMEM, st>>>(psi, buf, buf, p, n, lo, scal);
     return cudaGetLastError();
@@ -402,8 +394,8 @@ cudaError_t launch_marginal(const float2 *psi, int N, const double *scal, double
                    : strided_k<MS_BUF, MD_BUF>(K[i], psi, buf, p, n, lo[i], scal, st);
         if (e != cudaSuccess) return e;
     }
-    static bool done = false;
-    e = smem_attr(marg_row, done);
+    static SmemOptIn optin;
+    e = optin.allow((const void *)marg_row, MARG_SMEM);
     if (e != cudaSuccess) return e;
     marg_row<<<1u << (n - MB), MT, MARG_SMEM, st>>>(buf);
     e = cudaGetLastError();

@@ -772,13 +772,9 @@ cudaError_t launch_zrange_select(const float *Wf, long long nr, long long n_fam,
     if (nr & (nr - 1)) return cudaErrorInvalidValue;         // 2^(N - RL)
     if (nr <= ZSEL_STAGE_MAX) {
         const size_t smem = sizeof(float) * (size_t)(nr + 256 + 1);
-        static bool attr = false;
-        if (!attr) {
-            cudaError_t e = cudaFuncSetAttribute(zrange_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)(sizeof(float) * (ZSEL_STAGE_MAX + 257)));
-            if (e != cudaSuccess) return e;
-            attr = true;
-        }
+        static SmemOptIn optin;
+        const cudaError_t e = optin.allow((const void *)zrange_select_kernel, sizeof(float) * (ZSEL_STAGE_MAX + 257));
+        if (e != cudaSuccess) return e;
         zrange_select_kernel<<<(unsigned)n_fam, 256, smem, st>>>(Wf, nr, n_fam, fam_base, z_per_x, seed, ctr0, draws,
                                                                  perm);
         *launches = 1;

@@ -691,13 +691,9 @@ template <class Cfg, int SRC, int DST, int PREC = 0>
 cudaError_t launch_cfg(const PassArgs &a, int tiles, cudaStream_t st) {
     const size_t tile_smem = (Cfg::NR > 1 || PREC != 0) ? sizeof(typename Cfg::C2) * (size_t)Cfg::G * Cfg::PSIZE : 0;
     const size_t smem = tile_smem + sizeof(double) * (8 * (Cfg::NT / 32) + 8);
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(fwht_pass_kernel<Cfg, SRC, DST, PREC>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static SmemOptIn optin;
+    const cudaError_t e = optin.allow((const void *)fwht_pass_kernel<Cfg, SRC, DST, PREC>, smem);
+    if (e != cudaSuccess) return e;
     dim3 grid;
     PassArgs b = a;
     b.fam_fast = 0;

@@ -142,13 +142,9 @@ template <class Cfg, int SRC, int PREC>
 cudaError_t launch_zs1(const PassArgs &a, const DrawInfo *draws, int z_per_x, unsigned long long *zs, float *cz,
                        const unsigned long long *perm, cudaStream_t st) {
     const size_t smem = sizeof(float2) * (size_t)Cfg::PSIZE + sizeof(double) * ((Cfg::NT + 31) / 32 + 4);
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(zsample_kernel<Cfg, SRC, PREC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static SmemOptIn optin;
+    const cudaError_t e = optin.allow((const void *)zsample_kernel<Cfg, SRC, PREC>, smem);
+    if (e != cudaSuccess) return e;
     const long long nd = a.n_fam * (long long)z_per_x;
     dim3 grid((unsigned)(nd < 65535 ? nd : 65535), (unsigned)((nd + 65534) / 65535));
     zsample_kernel<Cfg, SRC, PREC><<<grid, Cfg::NT, smem, st>>>(a, draws, z_per_x, zs, cz, perm);
@@ -444,13 +440,9 @@ template <int M>
 cudaError_t launch_fold(const PassArgs &a, const DrawInfo *draws, int z_per_x, unsigned long long *zs, float *cz,
                         const unsigned long long *perm, cudaStream_t st) {
     constexpr size_t smem = FOLD_SMEM;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(zsample_fold_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static SmemOptIn optin;
+    const cudaError_t e = optin.allow((const void *)zsample_fold_kernel<M>, smem);
+    if (e != cudaSuccess) return e;
     const long long nd = a.n_fam * (long long)z_per_x;
     const long long nb = (nd + FOLD_WARPS - 1) / FOLD_WARPS;
     if (nb > 0x7fffffffLL) return cudaErrorInvalidValue;

@@ -145,12 +145,9 @@ cudaError_t launch_tc05_gemm_sw(const void *A, const void *B, float *D, int M, i
     e = tc05_make_map_bf16(&tb, B, (unsigned long long)N, (unsigned long long)K, (unsigned long long)K, BN, SW);
     if (e != cudaSuccess) return e;
     const size_t smem = 1024 + 2 * (128 * SW + BN * SW) + 64;
-    static bool attr = false;
-    if (!attr) {
-        e = cudaFuncSetAttribute(tc05_gemm_kernel<BN, SW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static SmemOptIn optin;
+    e = optin.allow((const void *)tc05_gemm_kernel<BN, SW>, smem);
+    if (e != cudaSuccess) return e;
     tc05_gemm_kernel<BN, SW><<<dim3(N / BN, M / 128), 128, smem, st>>>(ta, tb, D, N, K, err);
     return cudaGetLastError();
 }

@@ -26,6 +26,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "smem_optin.cuh"
+
 namespace sre {
 
 template <typename R> struct V2;
