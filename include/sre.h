@@ -186,17 +186,19 @@ SRE_API sre_status sre_exact_batched(const void *const *psi_ptrs_host, const int
                              const sre_opts *opts, void *workspace, size_t workspace_bytes,
                              void *stream, sre_result *out);
 
-/* Autotuner: times every admissible tiling (radix_log2, tile_log2, x_batch)
- * of the family transform for N on the caller's state psi and keeps the
- * fastest in a process-wide table that sre_exact, sre_exact_batched, sre_mc
- * and the plan/workspace queries use whenever opts leaves those three fields
- * at 0 (so query workspace sizes after tuning). If the environment variable
- * SRE_TUNE_FILE names a file, the table is read from and written to it.
- * *best receives the choice (the defaults when N needs a single pass). N in
- * 2..26. */
+/* Autotuner: times the tilings (radix_log2, tile_log2, x_batch) of the family
+ * transform for N on the caller's state psi against the planned one, once as the
+ * marginal estimator runs them and once as the sweeps without z draws (sre_exact,
+ * sre_exact_batched, uniform sre_mc) do. A tiling that is faster than the plan's
+ * goes into a process-wide table with an entry for each of the two, used whenever
+ * opts leaves those three fields at 0 (so query workspace sizes after tuning);
+ * where the plan wins nothing is stored. If the environment variable SRE_TUNE_FILE
+ * names a file, the table is read from and written to it. *best receives the
+ * marginal estimator's tiling, which sre_make_plan then reports (the defaults when
+ * its plan for N has a single pass). N in 2..26. */
 SRE_API sre_status sre_autotune(const void *psi_c64_dev, int N, void *stream, sre_opts *best);
 
-/* Drops the autotuner's choice for N (N = 0: for every N), so that plans go
+/* Drops the autotuner's entries for N (N = 0: for every N), so that plans go
  * back to the planned defaults; rewrites SRE_TUNE_FILE when it is set. N in
  * 0..32, else SRE_EINVAL. Host only. */
 SRE_API sre_status sre_autotune_clear(int N);

@@ -80,12 +80,16 @@ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 bool fine_ranges(const Plan &P) { return P.npass > 1 && P.M_last > ZR_FINE; }
 
 // ------------------------------------------------------------ autotuner table
-// Best (radix_log2, tile_log2, x_batch) per N found by sre_autotune; used when
-// the caller leaves all three options at 0. Optionally persisted in the file
-// named by SRE_TUNE_FILE (lines "N radix tile x_batch").
+// (radix_log2, tile_log2, x_batch) per N where sre_autotune found a tiling that
+// beats the planned one; used when the caller leaves all three options at 0. The
+// marginal estimator and the sweeps without z draws have entries of their own: they
+// run different kernels and plans. Optionally persisted in the file named by
+// SRE_TUNE_FILE (lines "N radix tile x_batch" and "marginal" or "sweep"; a line
+// without that word is an entry for both).
 struct TuneEntry { int radix = 0, tile = 0, xbatch = 0; bool valid = false; };
+constexpr const char *TUNE_KIND[2] = {"marginal", "sweep"};
 std::mutex g_tune_mu;
-TuneEntry g_tune[33];
+TuneEntry g_tune[2][33];                 // [sweep][N]
 bool g_tune_loaded = false;
 
 void tune_load_locked() {
@@ -95,9 +99,16 @@ void tune_load_locked() {
     if (!fn) return;
     FILE *f = fopen(fn, "r");
     if (!f) return;
-    int N, r, t, b;
-    while (fscanf(f, "%d %d %d %d", &N, &r, &t, &b) == 4)
-        if (N >= 1 && N <= 32) { g_tune[N].radix = r; g_tune[N].tile = t; g_tune[N].xbatch = b; g_tune[N].valid = true; }
+    char line[128], kind[16];
+    while (fgets(line, sizeof line, f)) {
+        int N;
+        TuneEntry t;
+        t.valid = true;
+        const int got = sscanf(line, "%d %d %d %d %15s", &N, &t.radix, &t.tile, &t.xbatch, kind);
+        if (got < 4 || N < 1 || N > 32) continue;
+        for (int k = 0; k < 2; ++k)
+            if (got == 4 || !strcmp(kind, TUNE_KIND[k])) g_tune[k][N] = t;
+    }
     fclose(f);
 }
 
@@ -107,7 +118,10 @@ void tune_save_locked() {
     FILE *f = fopen(fn, "w");
     if (!f) return;
     for (int N = 1; N <= 32; ++N)
-        if (g_tune[N].valid) fprintf(f, "%d %d %d %d\n", N, g_tune[N].radix, g_tune[N].tile, g_tune[N].xbatch);
+        for (int k = 0; k < 2; ++k) {
+            const TuneEntry &t = g_tune[k][N];
+            if (t.valid) fprintf(f, "%d %d %d %d %s\n", N, t.radix, t.tile, t.xbatch, TUNE_KIND[k]);
+        }
     fclose(f);
 }
 
@@ -120,10 +134,10 @@ sre_status plan_for_tuned(int N, const sre_opts *o, int prec, Plan &P, bool swee
     if (prec == 32 && t.radix_log2 == 0 && t.tile_log2 == 0 && t.x_batch == 0) {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         tune_load_locked();
-        if (N >= 1 && N <= 32 && g_tune[N].valid) {
-            t.radix_log2 = g_tune[N].radix;
-            t.tile_log2 = g_tune[N].tile;
-            t.x_batch = g_tune[N].xbatch;
+        if (N >= 1 && N <= 32 && g_tune[sweep][N].valid) {
+            t.radix_log2 = g_tune[sweep][N].radix;
+            t.tile_log2 = g_tune[sweep][N].tile;
+            t.x_batch = g_tune[sweep][N].xbatch;
         }
     }
     return plan_for(N, &t, prec, P, sweep);
@@ -222,22 +236,24 @@ sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P, bool sweep) {
 // The plans of a call over `families` families, in order of preference, each with
 // an intermediate for no more families than that. A sweep's own split runs up to
 // SWEEP_FAMILIES a launch (8 GiB of intermediate from N = 18 on); where memory is
-// short it runs LAUNCH_FAMILIES, and then the 13-bit split.
-sre_status plans_for_call(int N, const sre_opts *o, bool sweep, long long families, std::vector<Plan> &plans) {
+// short it runs LAUNCH_FAMILIES, and then the 13-bit split. tuned = false leaves
+// the autotuner's entries out.
+sre_status plans_for_call(int N, const sre_opts *o, bool sweep, long long families, std::vector<Plan> &plans,
+                          bool tuned = true) {
     plans.clear();
     Plan P;
     auto add = [&](Plan Q) {
         Q.B = std::min(Q.B, families);
         plans.push_back(Q);
     };
-    CS(plan_for_tuned(N, o, 32, P, sweep));
+    CS(tuned ? plan_for_tuned(N, o, 32, P, sweep) : plan_for(N, o, 32, P, sweep));
     add(P);
     if (!sweep || P.npass == 1) return SRE_OK;
     if (P.npass > 1 && P.B > LAUNCH_FAMILIES && families > LAUNCH_FAMILIES && !(o && o->x_batch > 0)) {
         P.B = LAUNCH_FAMILIES;
         add(P);
     }
-    CS(plan_for_tuned(N, o, 32, P));
+    CS(plan_for(N, o, 32, P));
     if (P.npass != plans[0].npass || P.M_last != plans[0].M_last) add(P);
     return SRE_OK;
 }
@@ -1362,74 +1378,170 @@ sre_status batched_impl(const void *const *psi_ptrs, const int *Ns, int count, c
     return SRE_OK;
 }
 
+// Multi-pass plans process the families in an order that lets the
+// families of one launch share psi in L2: by the top bit j of x (the same
+// rows b for every family with that j), then by x's bits over the first
+// strided pass's tile index (partner tile = tile ^ those bits, so the
+// partner tiles of a launch span a few aligned blocks), then by index.
+// Each family keeps its own index for its moments, draw stream and
+// outputs, so no result depends on the order.
+// Up to N = 20 (8 MB of psi) the order is not worth the trip to the host: calls
+// of 300 and 5001 uniform families at N = 18 0.28 -> 0.24 and 2.41 -> 2.08 ms
+// without it, at N = 20 0.69 -> 0.66 and 9.40 -> 9.13 ms; at N = 21 19.4 and
+// 19.9 ms, at N = 24 178 and 198 ms.
+sre_status order_families(const Plan &P, long long n_x, const McWS &w, cudaStream_t st, const unsigned long long **xs_run,
+                          const unsigned long long **perm) {
+    *xs_run = w.xs;
+    *perm = nullptr;
+    if (P.npass == 1 || P.N < FAMILY_ORDER_NMIN) return SRE_OK;
+    std::vector<unsigned long long> hx((size_t)n_x), order((size_t)n_x), hxo((size_t)n_x);
+    CK(cudaMemcpyAsync(hx.data(), w.xs, sizeof(unsigned long long) * (size_t)n_x, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    const int cb = P.ms[0] - P.K[0], tb = P.lo[0] - cb;
+    constexpr int IB = 40;                       // index bits: n_x < 2^40, and the keys fit the other 24
+    for (long long i = 0; i < n_x; ++i) {
+        const unsigned long long x = hx[(size_t)i];
+        const unsigned long long j = x ? (unsigned long long)(63 - __builtin_clzll(x)) : 0ULL;
+        order[(size_t)i] = (((j << tb) | ((x >> cb) & ((1ULL << tb) - 1ULL))) << IB) | (unsigned long long)i;
+    }
+    std::sort(order.begin(), order.end());
+    for (long long i = 0; i < n_x; ++i) {
+        order[(size_t)i] &= (1ULL << IB) - 1ULL;
+        hxo[(size_t)i] = hx[order[(size_t)i]];
+    }
+    CK(cudaMemcpyAsync(w.xs_ord, hxo.data(), sizeof(unsigned long long) * (size_t)n_x, cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(w.perm, order.data(), sizeof(unsigned long long) * (size_t)n_x, cudaMemcpyHostToDevice,
+                       st));
+    CK(cudaStreamSynchronize(st));   // the host vectors go out of scope
+    *xs_run = w.xs_ord;
+    *perm = w.perm;
+    return SRE_OK;
+}
+
 // --------------------------------------------------------------- autotuner
-// Times the family-transform launch sequence of every admissible plan for N
-// on the caller's state and keeps the fastest (radix, tile, x_batch).
+// Families per second of plan P on psi, timed as calls run it: families drawn
+// uniformly and in the call's order, psi in tile order where a call copies it,
+// z ranges for the marginal estimator and candidates for the sweeps. *rate = 0
+// where device memory does not hold the plan.
+sre_status time_plan(const void *psi, const Plan &P, bool sweep, long long fams, cudaStream_t st, double *rate) {
+    *rate = 0.0;
+    sre_opts o;
+    sre_default_opts(&o);
+    const bool tiled = tiled_psi(P, o, fams), fine = fine_ranges(P);
+    const long long nr = 1LL << (P.N - P.RL), step = std::min(P.B, fams);
+    McWS w;
+    auto layout = [&](Arena &A) {
+        layout_mc(A, P, SRE_MC_UNIFORM, fams, 1, tiled, w);
+        w.Wf = sweep ? nullptr : A.take<float>((size_t)step * (size_t)nr);
+    };
+    Arena dry(nullptr);
+    layout(dry);
+    void *base = nullptr;
+    const sre_status got = own_workspace(dry.off, &base);
+    if (got == SRE_ENOMEM) return SRE_OK;
+    CS(got);
+    Arena A(base);
+    layout(A);
+    CS(run_norm2(psi, P.N, w.scal, w.npart, st));
+    CK(launch_draw_x(nullptr, P.N, fams, 0, 12345ULL, 0ULL, w.xs, st));
+    count_launches(1);
+    PassArgs a = base_args(P, psi, w.scal);
+    const unsigned long long *perm = nullptr;
+    CS(order_families(P, fams, w, st, &a.xs, &perm));
+    if (tiled) {
+        CK(launch_psi_tiled((const float2 *)psi, w.psi_tiled, P.lo[0], P.N, st));
+        count_launches(1);
+        a.psi_tiled = w.psi_tiled;
+    }
+    a.tile_out = w.tiles;
+    a.want_cand = sweep ? 1 : 0;
+    a.want_ranges = sweep ? 0 : 1;
+    a.rw_out = w.Wf;
+    a.rw_stride = nr;
+    struct Events {
+        cudaEvent_t e[2] = {nullptr, nullptr};
+        ~Events() {
+            for (cudaEvent_t v : e)
+                if (v) cudaEventDestroy(v);
+        }
+    } ev;
+    CK(cudaEventCreate(&ev.e[0]));
+    CK(cudaEventCreate(&ev.e[1]));
+    for (int rep = 0; rep < 4; ++rep) {                 // rep 0 warms up; the fastest of three
+        CK(cudaEventRecord(ev.e[0], st));
+        for (long long fb = 0; fb < fams; fb += step) {
+            PassArgs b = a;
+            b.fam_base = fb;
+            b.n_fam = std::min(step, fams - fb);
+            if (!sweep && fine && f32_row_ranges_accumulate(P.M_last))
+                CK(cudaMemsetAsync(w.Wf, 0, sizeof(float) * (size_t)b.n_fam * (size_t)nr, st));
+            CS(run_transform(P, b, SRC_PSI_FAMILY, DST_MOMENTS, w.inter, st));
+            CK(launch_fam_reduce(w.tiles, b.n_fam, (int)P.tiles_last, a.xs, fb, P.N, P.M_last, P.RL, w.fm, fb,
+                                 !sweep && !fine ? w.Wf : nullptr, nr, st, perm));
+            count_launches(1);
+        }
+        CK(cudaEventRecord(ev.e[1], st));
+        CK(cudaEventSynchronize(ev.e[1]));
+        float ms = 0.f;
+        CK(cudaEventElapsedTime(&ms, ev.e[0], ev.e[1]));
+        if (rep > 0 && ms > 0.f) *rate = std::max(*rate, (double)fams / ms);
+    }
+    return SRE_OK;
+}
+
+// A tiling replaces the planned one only where it is faster by more than the
+// timings scatter; else the entry is dropped and calls keep the plans' own rules.
+constexpr double TUNE_MARGIN = 1.02;
+
 sre_status autotune_impl(const void *psi, int N, cudaStream_t st, sre_opts *best) {
     sre_default_opts(best);
-    Plan P0;
-    CS(plan_for(N, nullptr, 32, P0));
-    if (P0.npass == 1) return SRE_OK;   // nothing to choose
-    struct Cand { int radix, tile, xb; };
-    std::vector<Cand> cands;
-    for (int r = F32_ROW_MMIN; r <= F32_ROW_MMAX; ++r)
-        for (int t : {0, 8})
-            for (int xb : {0, 8})
-                cands.push_back({r, t, xb});
-    double best_rate = -1.0;
     const long long d = 1LL << N;
-    for (const Cand &c : cands) {
-        sre_opts q;
-        sre_default_opts(&q);
-        q.radix_log2 = c.radix;
-        q.tile_log2 = c.tile;
-        q.x_batch = c.xb;
-        Plan P;
-        if (plan_for(N, &q, 32, P) != SRE_OK) continue;
-        const long long fams = std::min(d, std::max(P.B * 4, 64LL));
-        Arena dry(nullptr);
-        McWS w;
-        layout_mc(dry, P, SRE_MC_UNIFORM, fams, 1, false, w);
-        void *base = nullptr;
-        CS(own_workspace(dry.off, &base));
-        Arena A(base);
-        layout_mc(A, P, SRE_MC_UNIFORM, fams, 1, false, w);
-        CS(run_norm2(psi, N, w.scal, w.npart, st));
-        PassArgs a = base_args(P, psi, w.scal);
-        a.tile_out = w.tiles;
-        cudaEvent_t e0, e1;
-        CK(cudaEventCreate(&e0));
-        CK(cudaEventCreate(&e1));
-        float ms = 0.f;
-        for (int rep = 0; rep < 2; ++rep) {   // rep 0 warms up
-            CK(cudaEventRecord(e0, st));
-            for (long long fb = 0; fb < fams; fb += P.B) {
-                PassArgs b = a;
-                b.fam_base = fb;
-                b.n_fam = std::min(P.B, fams - fb);
-                CS(run_transform(P, b, SRC_PSI_FAMILY, DST_MOMENTS, w.inter, st));
-            }
-            CK(cudaEventRecord(e1, st));
-            CK(cudaEventSynchronize(e1));
-            CK(cudaEventElapsedTime(&ms, e0, e1));
+    for (const bool sweep : {false, true}) {
+        std::vector<Plan> tried;
+        TuneEntry entry;
+        double planned = 0.0, top = 0.0;
+        auto try_plan = [&](const Plan &P, double *rate) -> sre_status {
+            *rate = 0.0;
+            for (const Plan &Q : tried)
+                if (Q.npass == P.npass && Q.M_last == P.M_last && Q.B == P.B && std::equal(Q.K, Q.K + 4, P.K)) return SRE_OK;
+            tried.push_back(P);
+            return time_plan(psi, P, sweep, std::min(d, std::max(P.B * 4, 64LL)), st, rate);
+        };
+        std::vector<Plan> plans;
+        CS(plans_for_call(N, nullptr, sweep, d, plans, false));
+        if (plans[0].npass == 1) continue;              // nothing to choose
+        for (size_t i = 0; i < plans.size() && planned == 0.0; ++i) CS(try_plan(plans[i], &planned));
+        for (int r = F32_ROW_MMIN; r <= F32_ROW_MMAX; ++r)
+            for (int t : {0, 8})
+                for (int xb : {0, 8}) {
+                    sre_opts q;
+                    sre_default_opts(&q);
+                    q.radix_log2 = r;
+                    q.tile_log2 = t;
+                    q.x_batch = xb;
+                    Plan P;
+                    if (plan_for(N, &q, 32, P, sweep) != SRE_OK || P.npass == 1) continue;
+                    P.B = std::min(P.B, d);
+                    double rate = 0.0;
+                    CS(try_plan(P, &rate));
+                    if (rate > top && rate > TUNE_MARGIN * planned) {
+                        top = rate;
+                        entry.radix = r;
+                        entry.tile = t;
+                        entry.xbatch = xb;
+                        entry.valid = true;
+                    }
+                }
+        if (!sweep) {
+            best->radix_log2 = entry.valid ? entry.radix : plans[0].M_last;
+            best->tile_log2 = entry.tile;
+            best->x_batch = entry.xbatch;
         }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        const double rate = (double)fams * (double)d / (ms * 1e-3);
-        if (rate > best_rate) {
-            best_rate = rate;
-            best->radix_log2 = c.radix;
-            best->tile_log2 = c.tile;
-            best->x_batch = c.xb;
-        }
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        tune_load_locked();
+        g_tune[sweep][N] = entry;
+        tune_save_locked();
     }
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    tune_load_locked();
-    g_tune[N].radix = best->radix_log2;
-    g_tune[N].tile = best->tile_log2;
-    g_tune[N].xbatch = best->x_batch;
-    g_tune[N].valid = true;
-    tune_save_locked();
     return SRE_OK;
 }
 
@@ -1882,7 +1994,7 @@ sre_status sre_autotune_clear(int N) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     tune_load_locked();
     for (int n = 1; n <= 32; ++n)
-        if (N == 0 || n == N) g_tune[n] = TuneEntry();
+        if (N == 0 || n == N) g_tune[0][n] = g_tune[1][n] = TuneEntry();
     tune_save_locked();
     return SRE_OK;
 }
@@ -1939,41 +2051,8 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
         CK(launch_draw_x(nullptr, N, n_x, 0, seed, counter0, w.xs, st));
     }
     count_launches(1);
-    // Multi-pass plans process the families in an order that lets the
-    // families of one launch share psi in L2: by the top bit j of x (the same
-    // rows b for every family with that j), then by x's bits over the first
-    // strided pass's tile index (partner tile = tile ^ those bits, so the
-    // partner tiles of a launch span a few aligned blocks), then by index.
-    // Each family keeps its own index for its moments, draw stream and
-    // outputs, so no result depends on the order.
-    // Up to N = 20 (8 MB of psi) the order is not worth the trip to the host: calls
-    // of 300 and 5001 uniform families at N = 18 0.28 -> 0.24 and 2.41 -> 2.08 ms
-    // without it, at N = 20 0.69 -> 0.66 and 9.40 -> 9.13 ms; at N = 21 19.4 and
-    // 19.9 ms, at N = 24 178 and 198 ms.
-    const unsigned long long *xs_run = w.xs, *perm = nullptr;
-    if (P.npass > 1 && N >= FAMILY_ORDER_NMIN) {
-        std::vector<unsigned long long> hx((size_t)n_x), order((size_t)n_x), hxo((size_t)n_x);
-        CK(cudaMemcpyAsync(hx.data(), w.xs, sizeof(unsigned long long) * (size_t)n_x, cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        const int cb = P.ms[0] - P.K[0], tb = P.lo[0] - cb;
-        constexpr int IB = 40;                       // index bits: n_x < 2^40, and the keys fit the other 24
-        for (long long i = 0; i < n_x; ++i) {
-            const unsigned long long x = hx[(size_t)i];
-            const unsigned long long j = x ? (unsigned long long)(63 - __builtin_clzll(x)) : 0ULL;
-            order[(size_t)i] = (((j << tb) | ((x >> cb) & ((1ULL << tb) - 1ULL))) << IB) | (unsigned long long)i;
-        }
-        std::sort(order.begin(), order.end());
-        for (long long i = 0; i < n_x; ++i) {
-            order[(size_t)i] &= (1ULL << IB) - 1ULL;
-            hxo[(size_t)i] = hx[order[(size_t)i]];
-        }
-        CK(cudaMemcpyAsync(w.xs_ord, hxo.data(), sizeof(unsigned long long) * (size_t)n_x, cudaMemcpyHostToDevice, st));
-        CK(cudaMemcpyAsync(w.perm, order.data(), sizeof(unsigned long long) * (size_t)n_x, cudaMemcpyHostToDevice,
-                           st));
-        CK(cudaStreamSynchronize(st));   // the host vectors go out of scope
-        xs_run = w.xs_ord;
-        perm = w.perm;
-    }
+    const unsigned long long *xs_run = nullptr, *perm = nullptr;
+    CS(order_families(P, n_x, w, st, &xs_run, &perm));
 
     PassArgs a = base_args(P, psi, w.scal);
     a.precision = prec_code(o);
