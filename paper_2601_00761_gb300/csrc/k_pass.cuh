@@ -16,6 +16,8 @@
 // pass's global bit offset and the family come from PassArgs / the grid.
 #pragma once
 
+#include <type_traits>
+
 #include "sre_internal.cuh"
 #include "k_tc.cuh"
 
@@ -111,6 +113,34 @@ __device__ __forceinline__ void group_reduce(float (&v)[NV], float &mx, double (
                 }
             }
         }
+    }
+}
+
+// The same sums of four values where a thread holds 64 points, in a CTA of 64
+// threads: FP32 trees over 16 lanes (1024 points, as many as a warp of 32-point
+// threads sums), then FP64. Each exchange hands half of the values to the partner
+// lane: five shuffles for the four sums.
+__device__ __forceinline__ void half_warp_reduce(const float (&v)[4], float mx, double (&out)[4], float &omx, double *red) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float *rf = reinterpret_cast<float *>(red);
+    const bool u8 = lane & 8, u4 = lane & 4;       // value (lane >> 2) & 3 ends in this lane
+    const float a = (u8 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, u8 ? v[0] : v[2], 8);
+    const float b = (u8 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, u8 ? v[1] : v[3], 8);
+    float c = (u4 ? b : a) + __shfl_xor_sync(0xffffffffu, u4 ? a : b, 4);
+    c += __shfl_xor_sync(0xffffffffu, c, 2);
+    c += __shfl_xor_sync(0xffffffffu, c, 1);
+    mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));   // not negative, not NaN
+    __syncthreads();
+    if ((lane & 3) == 0) rf[4 * ((lane >> 2) & 3) + (threadIdx.x >> 4)] = c;
+    if (lane == 0) rf[16 + w] = mx;
+    __syncthreads();
+    if (w == 0) {
+        double sd = (double)rf[lane & 15];
+        sd += __shfl_xor_sync(0xffffffffu, sd, 2);
+        sd += __shfl_xor_sync(0xffffffffu, sd, 1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) out[i] = __shfl_sync(0xffffffffu, sd, 4 * i);
+        omx = fmaxf(rf[16], rf[17]);
     }
 }
 
@@ -311,12 +341,13 @@ __device__ __forceinline__ float lg2_ftz(float x) {
 // it leaves every q >= 2^-102 unchanged and makes q = 0 contribute 0.
 // SWAP orders each pair so that c(z0) comes first (bit k of pm set: swap);
 // CAND keeps the running maximum of q for the nullity candidates.
-template <int E, bool SWAP, bool CAND>
+// Points K0 .. K1 - 1.
+template <int E, bool SWAP, bool CAND, int K0 = 0, int K1 = E>
 __device__ __forceinline__ void moment_sums(const float2 (&h)[E], float2 sc, uint32_t pm, float2 &s2, float2 &s4,
                                             float2 &s6, float2 &sl, float &qmax) {
     const float2 tiny = make_float2(1.17549435e-38f, 1.17549435e-38f);
 #pragma unroll
-    for (int k = 0; k < E; ++k) {
+    for (int k = K0; k < K1; ++k) {
         float2 c = mul2(sc, h[k]);
         if constexpr (SWAP) {
             if ((pm >> k) & 1u) c = make_float2(c.y, c.x);
@@ -592,63 +623,95 @@ __device__ __forceinline__ void fwht_pass_body(const PassArgs &a, long long slot
         float s;
         if constexpr (S_SHARED) s = s_sh[grp];
         else s = (float)(*s_ptr);
-        const uint32_t zb = (uint32_t)gbase | Cfg::elem(t, 0, 0);
-        float2 s2 = make_float2(0.f, 0.f), s4 = s2, s6 = s2, sl = s2, w = s2;
-        float qmax = 0.f;
+        const bool cand = a.want_cand;
+        float qmax = 0.f, omx;
+        double out[6];
         constexpr bool RANGES = Cfg::E <= 32;     // 64 points per thread: launched without ranges only
-        const bool wr = RANGES && a.want_ranges, cand = a.want_cand;
-        // ranges of 2^ZR_FINE z (written per warp) or tile halves (2^M z)
-        constexpr bool FINE = RANGES && SRC == SRC_BUF && Cfg::M > ZR_FINE;
-        constexpr int RLS = FINE ? ZR_FINE : Cfg::M;
-        if (x) {
-            const float2 sc = make_float2(2.0f * s, 2.0f * s);
-            if (wr && j >= RLS) {
-                // every c(z0) and every c(z1) of a range block lie in ranges
-                // of their own: order each pair as (c(z0)^2, c(z1)^2) and s2
-                // is the pair of weights. Bit k of pm: parity of |x & z0| for
-                // z' = zb | k (z0 then carries the Im part).
-                const uint32_t xd = (uint32_t)((x & ((1ULL << j) - 1ULL)) | ((x >> (j + 1)) << j));
-                const uint32_t pm = walsh_mask5(xd & (Cfg::E - 1) & 31u) ^ ((__popc(xd & zb) & 1) ? 0xFFFFFFFFu : 0u);
-                if (cand) moment_sums<Cfg::E, RANGES, true>(v, sc, pm, s2, s4, s6, sl, qmax);
-                else moment_sums<Cfg::E, RANGES, false>(v, sc, pm, s2, s4, s6, sl, qmax);
-                w = s2;
-            } else {
-                if (cand) moment_sums<Cfg::E, false, true>(v, sc, 0u, s2, s4, s6, sl, qmax);
-                else moment_sums<Cfg::E, false, false>(v, sc, 0u, s2, s4, s6, sl, qmax);
-                if (wr && !FINE) {
-                    // both c of a pair lie in the range picked by bit M-1 of z'
-                    constexpr int RBIT = Cfg::M > 0 ? Cfg::M - 1 : 0;
-                    if constexpr (RBIT >= Cfg::RB) {
-                        const float all = s2.x + s2.y;
-                        w = ((zb >> RBIT) & 1u) ? make_float2(0.f, all) : make_float2(all, 0.f);
-                    } else {
-                        // tiles of at most 2 RB bits: the range bit is a slot bit
+        if constexpr (!RANGES) {
+            static_assert(Cfg::E == 64 && Cfg::T == 64 && Cfg::NT == 64, "32 + 32 points a thread, two warps");
+            // chains of 32 points, as in the other rows. The maximum is kept
+            // whether candidates are asked for or not: it costs nothing here, and a
+            // second copy of the sums without it ran 6% slower
+            float acc[4];
+            auto sums = [&](const float2 (&h)[Cfg::E], float2 sc) {
+                float2 p[4], q[4];
 #pragma unroll
-                        for (int k = 0; k < Cfg::E; ++k) {
-                            const float2 c = mul2(sc, v[k]);
-                            const float qq = c.x * c.x + c.y * c.y;
-                            if ((k >> RBIT) & 1) w.y += qq;
-                            else w.x += qq;
+                for (int i = 0; i < 4; ++i) p[i] = q[i] = make_float2(0.f, 0.f);
+                moment_sums<Cfg::E, false, true, 0, 32>(h, sc, 0u, p[0], p[1], p[2], p[3], qmax);
+                moment_sums<Cfg::E, false, true, 32, 64>(h, sc, 0u, q[0], q[1], q[2], q[3], qmax);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    p[i] = add2(p[i], q[i]);
+                    acc[i] = p[i].x + p[i].y;
+                }
+            };
+            if (x) {
+                sums(v, make_float2(2.0f * s, 2.0f * s));
+            } else {
+                float2 hs[Cfg::E];
+#pragma unroll
+                for (int k = 0; k < Cfg::E; ++k) hs[k] = make_float2(v[k].x + v[k].y, v[k].x - v[k].y);
+                sums(hs, make_float2(s, s));
+            }
+            double m[4];
+            half_warp_reduce(acc, qmax, m, omx, red);
+#pragma unroll
+            for (int i = 0; i < 6; ++i) out[i] = i < 4 ? m[i] : 0.0;
+        } else {
+            const uint32_t zb = (uint32_t)gbase | Cfg::elem(t, 0, 0);
+            float2 s2 = make_float2(0.f, 0.f), s4 = s2, s6 = s2, sl = s2, w = s2;
+            const bool wr = a.want_ranges;
+            // ranges of 2^ZR_FINE z (written per warp) or tile halves (2^M z)
+            constexpr bool FINE = SRC == SRC_BUF && Cfg::M > ZR_FINE;
+            constexpr int RLS = FINE ? ZR_FINE : Cfg::M;
+            if (x) {
+                const float2 sc = make_float2(2.0f * s, 2.0f * s);
+                if (wr && j >= RLS) {
+                    // every c(z0) and every c(z1) of a range block lie in ranges
+                    // of their own: order each pair as (c(z0)^2, c(z1)^2) and s2
+                    // is the pair of weights. Bit k of pm: parity of |x & z0| for
+                    // z' = zb | k (z0 then carries the Im part).
+                    const uint32_t xd = (uint32_t)((x & ((1ULL << j) - 1ULL)) | ((x >> (j + 1)) << j));
+                    const uint32_t pm = walsh_mask5(xd & (Cfg::E - 1)) ^ ((__popc(xd & zb) & 1) ? 0xFFFFFFFFu : 0u);
+                    if (cand) moment_sums<Cfg::E, true, true>(v, sc, pm, s2, s4, s6, sl, qmax);
+                    else moment_sums<Cfg::E, true, false>(v, sc, pm, s2, s4, s6, sl, qmax);
+                    w = s2;
+                } else {
+                    if (cand) moment_sums<Cfg::E, false, true>(v, sc, 0u, s2, s4, s6, sl, qmax);
+                    else moment_sums<Cfg::E, false, false>(v, sc, 0u, s2, s4, s6, sl, qmax);
+                    if (wr && !FINE) {
+                        // both c of a pair lie in the range picked by bit M-1 of z'
+                        constexpr int RBIT = Cfg::M > 0 ? Cfg::M - 1 : 0;
+                        if constexpr (RBIT >= Cfg::RB) {
+                            const float all = s2.x + s2.y;
+                            w = ((zb >> RBIT) & 1u) ? make_float2(0.f, all) : make_float2(all, 0.f);
+                        } else {
+                            // tiles of at most 2 RB bits: the range bit is a slot bit
+#pragma unroll
+                            for (int k = 0; k < Cfg::E; ++k) {
+                                const float2 c = mul2(sc, v[k]);
+                                const float qq = c.x * c.x + c.y * c.y;
+                                if ((k >> RBIT) & 1) w.y += qq;
+                                else w.x += qq;
+                            }
                         }
                     }
                 }
-            }
-        } else {
-            const float2 sc = make_float2(s, s);
-            typename Cfg::C2 hs[Cfg::E];
+            } else {
+                const float2 sc = make_float2(s, s);
+                typename Cfg::C2 hs[Cfg::E];
 #pragma unroll
-            for (int k = 0; k < Cfg::E; ++k) hs[k] = make_float2(v[k].x + v[k].y, v[k].x - v[k].y);
-            if (cand) moment_sums<Cfg::E, false, true>(hs, sc, 0u, s2, s4, s6, sl, qmax);
-            else moment_sums<Cfg::E, false, false>(hs, sc, 0u, s2, s4, s6, sl, qmax);
-            w = s2;                    // z' -> range A, z' + d/2 -> range B
+                for (int k = 0; k < Cfg::E; ++k) hs[k] = make_float2(v[k].x + v[k].y, v[k].x - v[k].y);
+                if (cand) moment_sums<Cfg::E, false, true>(hs, sc, 0u, s2, s4, s6, sl, qmax);
+                else moment_sums<Cfg::E, false, false>(hs, sc, 0u, s2, s4, s6, sl, qmax);
+                w = s2;                    // z' -> range A, z' + d/2 -> range B
+            }
+            if constexpr (FINE) {
+                if (wr) fine_range_weights<Cfg::E>(s2, x, j, half, zb, a.rw_out + (size_t)slot * (size_t)a.rw_stride, active);
+            }
+            float acc[6] = {s2.x + s2.y, s4.x + s4.y, s6.x + s6.y, sl.x + sl.y, w.x, w.y};
+            group_reduce<Cfg::T, Cfg::NT, 6>(acc, qmax, out, omx, red);
         }
-        if constexpr (FINE) {
-            if (wr) fine_range_weights<Cfg::E>(s2, x, j, half, zb, a.rw_out + (size_t)slot * (size_t)a.rw_stride, active);
-        }
-        float acc[6] = {s2.x + s2.y, s4.x + s4.y, s6.x + s6.y, sl.x + sl.y, w.x, w.y};
-        double out[6];
-        float omx;
-        group_reduce<Cfg::T, Cfg::NT, 6>(acc, qmax, out, omx, red);
         if (active && t == 0 && a.fam_out) {
             FamMoments &o = a.fam_out[a.fam_base + slot];
             o.m[0] = out[0]; o.m[1] = out[1]; o.m[2] = out[2]; o.m[3] = out[3];
