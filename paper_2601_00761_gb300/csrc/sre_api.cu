@@ -186,26 +186,17 @@ sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P, bool sweep) {
     }
     // the first pass reads psi (8 bytes << N), which L2 holds up to N = 24
     auto ms_of = [&](int K, int pass) { return prec == 32 ? f32_strided_ms(K, pass == 0 && N >= 25) : F64_STRIDED_M; };
-    // A strided tile is 2^K rows x 2^(ms-K) columns and its columns must fit
-    // below the pass's row stride 2^lo: ms - K <= lo. Only the bottom strided
-    // pass (lo = nlo) can violate it: K_bottom >= 13 - nlo.
+    // A strided tile is 2^K rows x 2^(ms-K) columns, and its columns fit below the
+    // pass's row stride 2^lo in every plan: FP32 tiles of up to five bits hold 2^10
+    // points, and rows are at least 10 bits; the FP64 tiles have at most 2^12
+    // columns above 12-bit rows. Options of one or two strided bits a pass are raised above rows
+    // of 10 and 11 bits, where they would need more than three passes.
     const int rest = P.n - nlo;
-    const int kmin_bottom = 13 - nlo > 1 ? 13 - nlo : 1;
-    if (kmax < kmin_bottom) kmax = kmin_bottom;
-    int ns = (rest + kmax - 1) / kmax;
+    kmax = std::max(kmax, 13 - nlo);
+    const int ns = (rest + kmax - 1) / kmax;
     if (ns > 3) return fail(SRE_ENOTSUP, "N=%d needs %d strided passes", N, ns);
     // balanced, extra bits to the lower passes
     for (int i = 0; i < ns; ++i) P.K[i] = rest / ns + (i >= ns - rest % ns ? 1 : 0);
-    if (P.K[ns - 1] < kmin_bottom) {
-        if (rest < kmin_bottom) return fail(SRE_EINVAL, "N=%d: radix %d leaves %d strided bits", N, nlo, rest);
-        P.K[ns - 1] = kmin_bottom;
-        const int rem = rest - kmin_bottom;
-        const int no = ns - 1 > 0 ? ns - 1 : (rem > 0 ? 1 : 0);
-        if (no + 1 > 3) return fail(SRE_ENOTSUP, "N=%d needs %d strided passes", N, no + 1);
-        for (int i = 0; i < no; ++i) P.K[i] = rem / no + (i >= no - rem % no ? 1 : 0);
-        P.K[no] = kmin_bottom;
-        ns = no + 1;
-    }
     P.nstrided = ns;
     P.npass = ns + 1;
     int top = P.n;
