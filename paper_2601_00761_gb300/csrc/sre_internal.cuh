@@ -109,9 +109,9 @@ struct TileCfg {
     static constexpr int SIZE = 1 << M;
     // CTAs per SM the register budget is sized for: FP32 tiles of at most 64 KB
     // keep 16 warps of 128 registers on an SM (12 warps of 168 when a thread
-    // holds 64 points), in as many CTAs as that makes, so that load, exchange
-    // and butterfly phases of different CTAs overlap
-    static constexpr int REGS = RB >= 6 ? 168 : 128;
+    // holds 64 points, 32 of 64 in tiles of 512 threads with 16), in as many CTAs as that makes,
+    // so that load, exchange and butterfly phases of different CTAs overlap
+    static constexpr int REGS = RB >= 6 ? 168 : RB == 4 && NT == 512 ? 64 : 128;
     static constexpr int MINB = (sizeof(C2) == 8 && sizeof(C2) * SIZE * G <= 65536) ? 65536 / (REGS * NT) : 1;
     static_assert(TB >= 0, "tile smaller than a thread's registers");
     static_assert(K >= 0, "bad tile");
