@@ -825,9 +825,12 @@ __global__ void __launch_bounds__(256) mc_family_stats_kernel(const FamMoments *
     int id;
     const double t = warp_sums<4>(a, id);                // value v in lanes 8 v .. 8 v + 7
     if ((lane & 7) == 0 && id < 3) {
-        const double exact = (id == 0 ? -m.m[3] : id == 1 ? m.m[1] : m.m[2]) / m.m[0];
+        // p(x) may be the marginal's rounding alone (below 2^-50 or so of p(0)): a
+        // drawn family whose c are all zero has no conditional means and adds nothing
+        const bool none = m.m[0] == 0.0;
+        const double exact = none ? 0.0 : (id == 0 ? -m.m[3] : id == 1 ? m.m[1] : m.m[2]) / m.m[0];
         o[3 + id] = exact;
-        o[id] = i == 0 ? exact : t / z_per_x;
+        o[id] = i == 0 ? exact : none ? 0.0 : t / z_per_x;
     }
 }
 

@@ -36,3 +36,22 @@ def test_all_mass_at_zero():
     for n_x in (512, 513):                  # chunk sums, the whole CDF
         r = sre.sre_mc(psi, sre.SRE_MC_MARGINAL, n_x, 1, seed=1, return_samples=True)
         assert r["xs"][0] == 0 and bool((r["xs"][1:] == 1).all())
+
+
+@pytest.mark.parametrize("N", [8, 10, 12])
+@pytest.mark.parametrize("b", [1e-7, 3e-8])
+def test_families_of_rounding_noise(N, b):
+    """|0> + sum b_k |x_k>: 1 - p(0) is some 1e-14, so the rounding of the marginal (1e-17)
+    is drawn too, and with it families without any weight. The estimates stay what
+    the x = 0 stratum makes them (1e-5, the bound of every M)."""
+    r = np.random.Generator(np.random.PCG64(N))
+    for seed in range(8):
+        at = torch.from_numpy(r.choice(np.arange(1, 1 << N), 6, replace=False)).cuda()
+        psi = torch.zeros(1 << N, dtype=torch.complex64, device="cuda")
+        psi[0] = 1
+        psi[at] = torch.from_numpy(b * np.sqrt(r.random(6) + 0.1)).to(psi)
+        got = sre.sre_mc(psi, sre.SRE_MC_MARGINAL, 4000, 2, seed=seed)
+        exact = sre.sre_exact(psi)
+        for k in ("M", "M_rb"):
+            assert np.abs(np.array(got[k]) - exact["M"]).max() <= 1e-5
+        assert np.isfinite(got["err_M"]).all() and np.isfinite(got["err_rb"]).all()
