@@ -403,23 +403,28 @@ cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, doub
 }
 
 // ---------------------------------------------------------------- draws
-__device__ __forceinline__ unsigned long long cdf_search(const double *cdf, unsigned long long n, double t) {
-    // smallest i with cdf[i] > t; if none, the last i with a positive step
-    if (!(cdf[n - 1] > t)) {
-        unsigned long long i = n - 1;
-        while (i > 0 && !(cdf[i] > cdf[i - 1])) --i;
-        return i;
-    }
+// The smallest x with cdf[x] > t, or n - 1, and from there down to the last x of
+// positive p: the prefixes round differently where threads, chunks and scan tiles
+// meet, so the CDF may step at an x whose p is zero. Chunks whose sum did not move
+// the prefix are passed over (boff as in launch_scan).
+__device__ __forceinline__ unsigned long long cdf_search(const double *cdf, const double *p, const double *boff,
+                                                         unsigned long long n, double t) {
     unsigned long long lo = 0, hi = n - 1;
     while (lo < hi) {
         const unsigned long long mid = lo + ((hi - lo) >> 1);
         if (cdf[mid] > t) hi = mid; else lo = mid + 1;
     }
-    return lo;
+    for (;;) {
+        unsigned long long c = lo / SCAN_CHUNK;
+        while (lo > c * SCAN_CHUNK && !(p[lo] > 0.0)) --lo;
+        if (c == 0 || p[lo] > 0.0) return lo;
+        do --c; while (c > 0 && !(boff[c + 1] > boff[c]));
+        lo = (c + 1) * SCAN_CHUNK - 1;
+    }
 }
 
-__global__ void draw_x_kernel(const double *cdf, int N, long long n_x, int mode, unsigned long long seed,
-                              unsigned long long ctr0, unsigned long long *xs) {
+__global__ void draw_x_kernel(const double *cdf, const double *p, const double *boff, int N, long long n_x, int mode,
+                              unsigned long long seed, unsigned long long ctr0, unsigned long long *xs) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_x) return;
     const unsigned long long d = 1ULL << N;
@@ -432,7 +437,7 @@ __global__ void draw_x_kernel(const double *cdf, int N, long long n_x, int mode,
         if (x >= d) x = d - 1;
     } else {                  // x ~ p(x | x != 0): inverse CDF over x >= 1
         const double c0 = cdf[0];
-        x = cdf_search(cdf, d, c0 + u * (cdf[d - 1] - c0));
+        x = cdf_search(cdf, p, boff, d, c0 + u * (cdf[d - 1] - c0));
         if (x == 0) x = 1;
     }
     xs[i] = x;
@@ -524,9 +529,9 @@ cudaError_t launch_draw_x_chunks(const double *p, const double *boff, int N, lon
     return cudaGetLastError();
 }
 
-cudaError_t launch_draw_x(const double *cdf, int N, long long n_x, int mode, unsigned long long seed,
-                          unsigned long long ctr0, unsigned long long *xs, cudaStream_t st) {
-    draw_x_kernel<<<(unsigned)((n_x + 255) / 256), 256, 0, st>>>(cdf, N, n_x, mode, seed, ctr0, xs);
+cudaError_t launch_draw_x(const double *cdf, const double *p, const double *boff, int N, long long n_x, int mode,
+                          unsigned long long seed, unsigned long long ctr0, unsigned long long *xs, cudaStream_t st) {
+    draw_x_kernel<<<(unsigned)((n_x + 255) / 256), 256, 0, st>>>(cdf, p, boff, N, n_x, mode, seed, ctr0, xs);
     return cudaGetLastError();
 }
 

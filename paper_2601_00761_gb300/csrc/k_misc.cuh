@@ -79,11 +79,12 @@ cudaError_t launch_fam_reduce(const TilePartial *tp, long long n_fam, int tiles,
 cudaError_t launch_sum_u64(const unsigned long long *v, long long n, unsigned long long *out, cudaStream_t st);
 // bsum: n / SCAN_CHUNK + 1 doubles (chunks rounded up), the exclusive prefix of p's
 // chunk sums and the total; tot: 32 doubles of scratch; cdf (or NULL): the
-// inclusive CDF of p (may be p itself)
+// inclusive CDF of p
 cudaError_t launch_scan(const double *p, unsigned long long n, double *cdf, double *bsum, double *tot, int *launches,
                         cudaStream_t st);
-cudaError_t launch_draw_x(const double *cdf, int N, long long n_x, int mode, unsigned long long seed,
-                          unsigned long long ctr0, unsigned long long *xs, cudaStream_t st);
+// mode 0: uniform on 1 .. d - 1 (no arrays); 1: from the CDF of p, boff as above
+cudaError_t launch_draw_x(const double *cdf, const double *p, const double *boff, int N, long long n_x, int mode,
+                          unsigned long long seed, unsigned long long ctr0, unsigned long long *xs, cudaStream_t st);
 // marginal draws from p and the prefix of its chunk sums (N >= 12)
 cudaError_t launch_draw_x_chunks(const double *p, const double *boff, int N, long long n_x, unsigned long long seed,
                                  unsigned long long ctr0, unsigned long long *xs, cudaStream_t st);

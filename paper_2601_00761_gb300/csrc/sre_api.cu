@@ -319,7 +319,7 @@ void layout_exact(Arena &A, const Plan &P, const Plan &P64, ExactWS &w) {
 
 struct McWS {
     double *scal, *npart;
-    double *p, *mwork, *bsum;            // mwork is free once p is known: the scans' scratch
+    double *p, *mwork, *bsum;            // mwork: the marginal's work, then the CDF, then the range draws' sums
     unsigned long long *xs;
     unsigned long long *xs_ord, *perm;   // the families in processing order, and their own indices
     float2 *psi_tiled;                   // psi in tile order, or NULL
@@ -1434,7 +1434,7 @@ sre_status time_plan(const void *psi, const Plan &P, bool sweep, long long fams,
     Arena A(base);
     layout(A);
     CS(run_norm2(psi, P.N, w.scal, w.npart, st));
-    CK(launch_draw_x(nullptr, P.N, fams, 0, 12345ULL, 0ULL, w.xs, st));
+    CK(launch_draw_x(nullptr, nullptr, nullptr, P.N, fams, 0, 12345ULL, 0ULL, w.xs, st));
     count_launches(1);
     PassArgs a = base_args(P, psi, w.scal);
     const unsigned long long *perm = nullptr;
@@ -2034,12 +2034,12 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
         // whole CDF costs 10 ps per x: few draws on a large state skip the CDF
         const bool chunks = (unsigned long long)n_x <= d / 2048;
         int nl = 0;
-        CK(launch_scan(w.p, d, chunks ? nullptr : w.p, w.bsum, w.mwork, &nl, st));
+        CK(launch_scan(w.p, d, chunks ? nullptr : w.mwork, w.bsum, w.npart, &nl, st));
         count_launches(nl);
         if (chunks) CK(launch_draw_x_chunks(w.p, w.bsum, N, n_x, seed, counter0, w.xs, st));
-        else CK(launch_draw_x(w.p, N, n_x, 1, seed, counter0, w.xs, st));
+        else CK(launch_draw_x(w.mwork, w.p, w.bsum, N, n_x, 1, seed, counter0, w.xs, st));
     } else {
-        CK(launch_draw_x(nullptr, N, n_x, 0, seed, counter0, w.xs, st));
+        CK(launch_draw_x(nullptr, nullptr, nullptr, N, n_x, 0, seed, counter0, w.xs, st));
     }
     count_launches(1);
     const unsigned long long *xs_run = nullptr, *perm = nullptr;
@@ -2423,7 +2423,7 @@ sre_status sre_profile_passes(const void *psi, int N, long long n_x, const sre_o
     Arena A(base);
     layout_mc(A, P, SRE_MC_UNIFORM, n_x < 2 ? 2 : n_x, 1, tiled_psi(P, o, n_x), w);
     CS(run_norm2(psi, N, w.scal, w.npart, st));
-    CK(launch_draw_x(nullptr, N, n_x, 0, 12345ULL, 0ULL, w.xs, st));
+    CK(launch_draw_x(nullptr, nullptr, nullptr, N, n_x, 0, 12345ULL, 0ULL, w.xs, st));
     count_launches(1);
     PassArgs a = base_args(P, psi, w.scal);
     a.precision = prec_code(o);

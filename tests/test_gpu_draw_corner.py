@@ -55,3 +55,21 @@ def test_families_of_rounding_noise(N, b):
         for k in ("M", "M_rb"):
             assert np.abs(np.array(got[k]) - exact["M"]).max() <= 1e-5
         assert np.isfinite(got["err_M"]).all() and np.isfinite(got["err_rb"]).all()
+
+
+# few draws go through the chunk sums, many through the CDF (n_x > 2^N / 2048)
+@pytest.mark.parametrize("N,n_x", [(10, 4000), (12, 4000), (16, 4000), (20, 512), (20, 4000), (22, 4000)])
+@pytest.mark.parametrize("b", [1e-7, 3e-8])
+def test_several_x_of_little_mass(N, n_x, b):
+    """|0> + sum b_k |x_k>: prefixes over several of the p(x_k) round differently from
+    chunk to chunk, by as much as a p(x_k) is worth."""
+    r = np.random.Generator(np.random.PCG64(N))
+    for seed in range(4):
+        at = torch.from_numpy(r.choice(np.arange(1, 1 << N), 6, replace=False)).cuda()
+        psi = torch.zeros(1 << N, dtype=torch.complex64, device="cuda")
+        psi[0] = 1
+        psi[at] = torch.from_numpy(b * np.sqrt(r.random(6) + 0.1)).to(psi)
+        p = sre.pauli_x_marginal(psi)
+        got = sre.sre_mc(psi, sre.SRE_MC_MARGINAL, n_x, 2, seed=seed, return_samples=True)
+        assert float(p[got["xs"]].min()) > 0
+        assert np.isfinite(got["M_rb"]).all()
