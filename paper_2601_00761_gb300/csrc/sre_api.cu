@@ -224,14 +224,27 @@ sre_status plan_for(int N, const sre_opts *o, int prec, Plan &P, bool sweep) {
     return SRE_OK;
 }
 
+// A few values without a heap allocation: a call has at most four plans
+// (plans_for_call, and one more with psi in tile order), each with its workspace.
+template <class T>
+struct Few {
+    T v[4];
+    size_t n = 0;
+    void push_back(const T &t) { v[n++] = t; }
+    size_t size() const { return n; }
+    const T &operator[](size_t i) const { return v[i]; }
+    const T *begin() const { return v; }
+    const T *end() const { return v + n; }
+};
+
 // The plans of a call over `families` families, in order of preference, each with
 // an intermediate for no more families than that. A sweep's own split runs up to
 // SWEEP_FAMILIES a launch (8 GiB of intermediate from N = 18 on); where memory is
 // short it runs LAUNCH_FAMILIES, and then the 13-bit split. tuned = false leaves
 // the autotuner's entries out.
-sre_status plans_for_call(int N, const sre_opts *o, bool sweep, long long families, std::vector<Plan> &plans,
+sre_status plans_for_call(int N, const sre_opts *o, bool sweep, long long families, Few<Plan> &plans,
                           bool tuned = true) {
-    plans.clear();
+    plans.n = 0;
     Plan P;
     auto add = [&](Plan Q) {
         Q.B = std::min(Q.B, families);
@@ -384,7 +397,7 @@ std::vector<DevBuf> g_gatebuf;
 // refused is not tried again while the workspace holds a later layout, so that
 // calls under memory pressure do not free and allocate each time
 // (sre_release_workspace forgets it).
-sre_status own_workspace(const std::vector<size_t> &needs, size_t *which, void **out) {
+sre_status own_workspace(const Few<size_t> &needs, size_t *which, void **out) {
     int dev = 0;
     CK(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lk(g_ws_mu);
@@ -417,14 +430,20 @@ sre_status own_workspace(const std::vector<size_t> &needs, size_t *which, void *
     return SRE_ENOMEM;
 }
 
+Few<size_t> one_need(size_t need) {
+    Few<size_t> f;
+    f.push_back(need);
+    return f;
+}
+
 sre_status own_workspace(size_t need, void **out) {
     size_t which = 0;
-    return own_workspace(std::vector<size_t>{need}, &which, out);
+    return own_workspace(one_need(need), &which, out);
 }
 
 // The workspace for the first of several layouts that fits: a caller's by its
 // size, else the library's.
-sre_status resolve_workspace(void *ws, size_t ws_bytes, const std::vector<size_t> &needs, size_t *which, void **out) {
+sre_status resolve_workspace(void *ws, size_t ws_bytes, const Few<size_t> &needs, size_t *which, void **out) {
     if (!ws) return own_workspace(needs, which, out);
     for (*which = 0; *which < needs.size() && ws_bytes < needs[*which];) ++*which;
     if (*which == needs.size()) return fail(SRE_EINVAL, "workspace of %zu bytes, %zu needed", ws_bytes, needs[0]);
@@ -435,7 +454,7 @@ sre_status resolve_workspace(void *ws, size_t ws_bytes, const std::vector<size_t
 
 sre_status resolve_workspace(void *ws, size_t ws_bytes, size_t need, void **out) {
     size_t which = 0;
-    return resolve_workspace(ws, ws_bytes, std::vector<size_t>{need}, &which, out);
+    return resolve_workspace(ws, ws_bytes, one_need(need), &which, out);
 }
 
 // ------------------------------------------------------------ checks
@@ -744,12 +763,12 @@ sre_status nullity_from_count(long long cnt, int N, sre_result *r) {
 sre_status exact_impl(const void *psi, int N, const sre_opts &o, void *ws, size_t ws_bytes, cudaStream_t st,
                       sre_result *out) {
     const unsigned long long d = 1ULL << N;
-    std::vector<Plan> plans;
+    Few<Plan> plans;
     Plan P64;
     CS(plans_for_call(N, &o, true, (long long)d, plans));
     CS(plan_for(N, nullptr, 64, P64));
     ExactWS w;
-    std::vector<size_t> needs;
+    Few<size_t> needs;
     for (const Plan &Q : plans) {
         Arena dry(nullptr);
         layout_exact(dry, Q, P64, w);
@@ -837,7 +856,7 @@ struct BucketPlan {
     int N;
     std::vector<int> idx;       // caller indices of the bucket's states
     int off;                    // first slot of the bucket in the per-state arrays
-    std::vector<Plan> plans;    // by memory (plans_for_call); P is the one that runs
+    Few<Plan> plans;            // by memory (plans_for_call); P is the one that runs
     Plan P, P64;
     int states_per_chunk;
     unsigned long long *flags;  // flagged families of the bucket (capacity: its families)
@@ -1246,7 +1265,7 @@ sre_status batched_impl(const void *const *psi_ptrs, const int *Ns, int count, c
         for (BucketPlan &b : B) b.P = b.plans[std::min(i, b.plans.size() - 1)];
         persist_plan(B, prec_code(o), o.batch_queue != 0, L);
     };
-    std::vector<size_t> needs;
+    Few<size_t> needs;
     for (size_t i = 0; i < variants; ++i) {
         take_plans(i);
         Arena dry(nullptr);
@@ -1498,7 +1517,7 @@ sre_status autotune_impl(const void *psi, int N, cudaStream_t st, sre_opts *best
             tried.push_back(P);
             return time_plan(psi, P, sweep, std::min(d, std::max(P.B * 4, 64LL)), st, rate);
         };
-        std::vector<Plan> plans;
+        Few<Plan> plans;
         CS(plans_for_call(N, nullptr, sweep, d, plans, false));
         if (plans[0].npass == 1) continue;              // nothing to choose
         for (size_t i = 0; i < plans.size() && planned == 0.0; ++i) CS(try_plan(plans[i], &planned));
@@ -1901,7 +1920,7 @@ sre_status sre_workspace_bytes(int N, int mode, long long n_x, int z_per_x, cons
     if (!bytes) return fail(SRE_EINVAL, "bytes is NULL");
     sre_opts o;
     CS(check_opts(opts, o));
-    std::vector<Plan> plans;
+    Few<Plan> plans;
     if (mode == -1) {
         if (N < 1 || N > 26) return fail(SRE_EINVAL, "exact: N=%d outside 1..26", N);
         Plan P64;
@@ -2004,22 +2023,23 @@ sre_status sre_mc(const void *psi, int N, int mode, long long n_x, int z_per_x, 
     sre_opts o;
     CS(check_opts(opts, o));
     cudaStream_t st = (cudaStream_t)stream;
-    std::vector<Plan> plans;
+    Few<Plan> plans;
     CS(plans_for_call(N, &o, mode == SRE_MC_UNIFORM, n_x, plans));
     const bool tiled_first = tiled_psi(plans[0], o, n_x);
-    if (tiled_first) plans.insert(plans.begin(), Plan(plans[0]));      // with the copy of psi, then without
     McWS w;
-    std::vector<size_t> needs;
+    Few<size_t> needs;
+    // the first plan with the copy of psi comes before all of them without
     auto tiled_plan = [&](size_t i) { return tiled_first && i == 0; };
-    for (size_t i = 0; i < plans.size(); ++i) {
+    auto plan_of = [&](size_t i) -> const Plan & { return plans[tiled_first && i > 0 ? i - 1 : i]; };
+    for (size_t i = 0; i < plans.size() + (tiled_first ? 1 : 0); ++i) {
         Arena dry(nullptr);
-        layout_mc(dry, plans[i], mode, n_x, z_per_x, tiled_plan(i), w);
+        layout_mc(dry, plan_of(i), mode, n_x, z_per_x, tiled_plan(i), w);
         needs.push_back(dry.off);
     }
     void *base = nullptr;
     size_t which = 0;
     CS(resolve_workspace(workspace, workspace_bytes, needs, &which, &base));
-    const Plan P = plans[which];
+    const Plan P = plan_of(which);
     const bool tiled = tiled_plan(which);
     Arena A(base);
     layout_mc(A, P, mode, n_x, z_per_x, tiled, w);
