@@ -227,9 +227,10 @@ SRE_API sre_status sre_mc(const void *psi_c64_dev, int N, int mode, long long n_
                   unsigned long long *xs_dev, unsigned long long *zs_dev, float *c_dev);
 
 /* The exact X-mask marginal p(x) = sum_z c_{x,z}^2 / d = (q*q)(x), the XOR
- * autocorrelation of q = s|psi|^2, computed as WHT(WHT(q)^2)/d in FP64
- * (WHT(q) is the x = 0 family, Eq. Z-FWHT). p_dev: d doubles. N in 1..30.
- * workspace: 8*d bytes or NULL. */
+ * autocorrelation of q = s|psi|^2, computed as WHT(WHT(q)^2)/d (WHT(q) is the
+ * x = 0 family, Eq. Z-FWHT) with the transforms in 64-bit integers, in FP64 up
+ * to N = 12: a few units of 2^-53 p(0). p_dev: d doubles. N in 1..30.
+ * workspace: 8 d + 16384 bytes, 256-byte aligned, or NULL. */
 SRE_API sre_status pauli_x_marginal(const void *psi_c64_dev, int N, double *p_dev,
                             void *workspace, size_t workspace_bytes, void *stream);
 
@@ -266,8 +267,9 @@ SRE_API sre_status sre_mixed_workspace_bytes(int N, int N_A, size_t *bytes);
  * the basis index, b = a + 2^{N_A} e) of psi: c_P = Tr(rho_A P) for the
  * 4^{N_A} Pauli strings on A. The family x_A needs h(a) = sum_e
  * conj(psi(a ^ x_A, e)) psi(a, e), an entry of the Gram matrix C = Psi Psi^H
- * of psi viewed as a d_A x d_B matrix (one cuBLAS GEMM, FP32 emulated on the
- * BF16 tensor cores with each input split into three BF16 parts), then
+ * of psi viewed as a d_A x d_B matrix (on the BF16 tensor cores, each amplitude
+ * split into three BF16 parts, six part products summed in FP32, the diagonal to
+ * FP64 precision; FP64 sums for small shapes), then
  * one N_A-bit transform per x_A with the moments fused (O(2^{N+N_A}) overall).
  * N in 1..30, N_A in 1..min(N, 15). workspace: >= sre_mixed_workspace_bytes,
  * 256-byte aligned, or NULL (library-owned). out: host. Synchronises the stream. */

@@ -7,9 +7,12 @@
 // those exactly, and writes doubles again. Per pass a number is rounded twice,
 // once to the tile's quantum and once back to 53 bits, instead of once per
 // transform stage. The quantum is 2^-62 times (less than twice) the largest sum
-// of magnitudes over one transform of the tile, so no sum can overflow; over
-// at most 11 bits it rounds random data no worse than 11 FP64 stages do
-// (measured against extended precision: not above the FP64 passes' error).
+// of magnitudes over one transform of the tile, so no sum can overflow; strided
+// passes of K < 4 bits (N = 13 to 15) take the magnitudes of 2^(4-K) columns
+// together, a quantum up to eight times that and still 2^-58 of the column's sum.
+// Over at most 11 bits it rounds random data no worse than 11 FP64 stages do
+// (measured against extended precision, N = 13 to 22: not above the FP64 passes'
+// error).
 //
 // The transforms are packed: element g < 2^n (n = N - 1) holds the pair
 // (value(g), value(g + d/2)), two real transforms side by side, and the top bit
@@ -21,8 +24,9 @@
 // Tiles are 2^12 pairs (64 KB), 256 threads x 16 pairs: two per SM. The row pass
 // in the middle saves one trip through memory.
 //
-// N = 27 (2^27 numbers, 1 GB): 17.2 ms with FP64 passes (FP64 pipe 76-83%
-// busy), 2.9 ms with these (16.2 against 2.9 without the norm both need).
+// N = 27 (2^27 numbers, 1 GB), without the norm that both need (0.23 ms): 16.2 ms
+// with FP64 passes (FP64 pipe 76-83% busy), 2.9 ms with these; whole calls 17.2 and
+// 3.2 ms.
 #include "k_misc.cuh"
 #include "k_fp64.cuh"
 
@@ -162,7 +166,7 @@ __device__ __forceinline__ void exchange(Pair (&v)[16], Pair *sm, uint32_t t) {
 enum { MS_PSI = 0, MS_BUF = 1 };
 enum { MD_BUF = 0, MD_P = 1 };
 
-// Power of two h with sum |psi|^2 4^h in [1/2, 4): psi 2^h is summed without
+// Power of two h with sum |psi|^2 4^h in (1/4, 1]: psi 2^h is summed without
 // overflow or harmful underflow in the FP32 magnitudes.
 __device__ __forceinline__ int psi_shift(double s) {
     const int ex = (int)(((unsigned)__double2hiint(s) >> 20) & 0x7ffu) - 1023;     // s = 1 / sum |psi|^2

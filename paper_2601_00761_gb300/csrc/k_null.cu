@@ -14,7 +14,7 @@
 //  - coset: the listed z' lie in z'_0 + span(v_1..v_m), m <= 6 (stabilizer
 //    structure). One sweep over g accumulates h(g) (-1)^{g.z'_0} into 2^m bins
 //    keyed by the parities g.v_i, and an m-bit WHT of the bins gives H on the
-//    whole coset: 6 FP64 operations per point for any number of candidates.
+//    whole coset: 4 FP64 operations per point for any number of candidates.
 //  - direct: wider spans with at most kdirect candidates: H at each listed z'
 //    by its own signed sum, 4 + 2k operations per point for k candidates.
 //  - overflow: the rest (or more than cand_max candidates, the list then being
